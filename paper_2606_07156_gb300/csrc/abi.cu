@@ -344,6 +344,23 @@ static bool wide_tables_fp32(const anns_precision_policy& P) {
   }
 }
 
+// Whether the policy can pick tables of at most 4 bits (the filter only marks
+// such pairs; the grouped kernels scan them).
+static bool nibble_possible(const anns_precision_policy& P) {
+  return P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 || P.lut_mode == ANNS_LUT_EXPLICIT ||
+         P.lut_mode == ANNS_LUT_SVR;
+}
+
+static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
+  return filter_supported(ix, P, nq, nprobe, k) && (!nibble_possible(P) || grouped_supported(ix, k));
+}
+
+// Whether the grouped kernels follow the filter: for the pairs on 1..4-bit
+// tables, and for the 5..8-bit pairs of the queries it does not settle.
+static bool grouped_after_filter(const Index& ix, const anns_precision_policy& P, int k) {
+  return (nibble_possible(P) || (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8)) && grouped_supported(ix, k);
+}
+
 static bool use_lpt(const Index& ix, const int32_t* nprobe_per_q) {
   return ix.opt_schedule == ANNS_SCHED_LPT || (ix.opt_schedule == ANNS_SCHED_AUTO && nprobe_per_q);
 }
@@ -352,16 +369,25 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
                    const int32_t* nprobe_per_q) {
   int rc = ensure_workspace(ix, nq, nprobe);
   if (rc) return rc;
-  if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, k)) {
-    ListWork w{};
-    const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
-    if ((rc = list_workspace(ix, nq, nprobe, k, w, qchunk))) return rc;
-  }
-  if (use_grouped(ix, P, k) || ix.opt_kernel == ANNS_KERNEL_SPLIT) {
-    if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
-  }
-  if (ix.opt_kernel != ANNS_KERNEL_LIST_MAJOR && use_lpt(ix, nprobe_per_q)) {
-    if ((rc = grow(&ix.ws_sched, &ix.ws_sched_cap, lpt_workspace_bytes(nq)))) return rc;
+  if (use_filter(ix, P, nq, nprobe, k)) {
+    if ((rc = grow(&ix.ws_fl, &ix.ws_fl_cap, filter_workspace_bytes(ix, nq, nprobe, k)))) return rc;
+    if (grouped_after_filter(ix, P, k)) {
+      ListWork w{};
+      if ((rc = list_workspace(ix, nq, nprobe, k, w, nq))) return rc;
+      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
+    }
+  } else {
+    if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, k)) {
+      ListWork w{};
+      const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
+      if ((rc = list_workspace(ix, nq, nprobe, k, w, qchunk))) return rc;
+    }
+    if (use_grouped(ix, P, k) || ix.opt_kernel == ANNS_KERNEL_SPLIT) {
+      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
+    }
+    if (ix.opt_kernel != ANNS_KERNEL_LIST_MAJOR && use_lpt(ix, nprobe_per_q)) {
+      if ((rc = grow(&ix.ws_sched, &ix.ws_sched_cap, lpt_workspace_bytes(nq)))) return rc;
+    }
   }
   if (coarse_tc_format(P.cl_prec)) {
     if ((rc = grow(&ix.ws_tc, &ix.ws_tc_cap, coarse_tc_workspace_bytes(ix, nq)))) return rc;
@@ -395,8 +421,51 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
   if ((rc = launch_policy(ix, P, nq, nprobe, nprobe_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits,
                           want_feat ? ix.ws_feat : nullptr, s)))
     return rc;
-  e = launch_query_tables(ix, Q, nq, ix.ws_qt, s);
+  const bool filter = use_filter(ix, P, nq, nprobe, k);
+  // the filtered search forms the few FP32 entries it needs itself
+  const bool tables_for_all = !filter || P.lut_mode != ANNS_LUT_PLAIN_FP32;
+  e = tables_for_all ? launch_query_tables(ix, Q, nq, ix.ws_qt, s) : cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(e, "query tables");
+  if (filter) {
+    if (ev) cudaEventRecord(ev[3], s);
+    const bool nib = nibble_possible(P), grouped = grouped_after_filter(ix, P, k);
+    // the top-k over the pairs the filter settles: the result itself, or with
+    // pairs on 1..4-bit tables a partial result
+    float* part_d = (float*)ix.ws_grp;
+    int64_t* part_i = (int64_t*)((char*)ix.ws_grp + (((size_t)nq * k * 4 + 255) & ~size_t(255)));
+    int64_t* di = nib ? part_i : ids_out;
+    float* dd = nib ? part_d : dists_out;
+    void* q16 = nullptr;
+    float* q16_rows = nullptr;
+    if (P.cl_prec == ANNS_PREC_FP16) coarse_tc_operand(ix, ix.ws_tc, nq, &q16, &q16_rows);
+    FilterResult r{};
+    e = launch_search_filter(ix, Q, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
+                             ix.ws_bits, ix.ws_fl, q16, q16_rows, tables_for_all, di, dd, grouped ? part_i : nullptr,
+                             grouped ? part_d : nullptr, &r, s);
+    if (e != cudaSuccess) return cuda_fail(e, "filter kernels");
+    // queries with more candidates than fit (usually none): their FP32, 12- and
+    // 16-bit pairs query-major, the 5..8-bit ones grouped
+    if (!tables_for_all) {
+      e = launch_query_tables(ix, Q, nq, ix.ws_qt, s, r.over, r.nover);
+      if (e != cudaSuccess) return cuda_fail(e, "query tables");
+    }
+    if (!(P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8 && grouped))
+      e = launch_search(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits,
+                        r.over, grouped ? part_i : di, grouped ? part_d : dd, s, grouped ? 2 : 0,
+                        P.lut_mode == ANNS_LUT_PLAIN_FP32 ? QM_TABLES_FP32 : QM_TABLES_ALL, nullptr, nullptr, r.nover);
+    if (e == cudaSuccess && ev) cudaEventRecord(ev[4], s);
+    if (e == cudaSuccess && grouped) {
+      ListWork w{};
+      if ((rc = list_workspace(ix, nq, nprobe, k, w, nq))) return rc;
+      e = launch_search_alive(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
+                              ix.ws_bits, r, nib, w, ix.ws_grp, ids_out, dists_out, s, ev ? ev[5] : nullptr,
+                              ev ? ev[6] : nullptr);
+      if (e == cudaSuccess && ev) cudaEventRecord(ev[7], s);
+    } else if (e == cudaSuccess && ev) {
+      for (int st = 5; st <= Index::kStages; ++st) cudaEventRecord(ev[st], s);
+    }
+    return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "search kernel");
+  }
   // table width the policy may need: FP32 (4 bytes), 16-bit or 8-bit levels
   const int tbytes = table_bytes_for(P);
   // AUTO: query-major (measured faster on the SIFT-shaped workload for every
@@ -464,7 +533,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
 
 void free_workspace(Index& ix) {
   void* ptrs[] = {ix.ws_qt, ix.ws_lists, ix.ws_d2, ix.ws_probes /* base of the pair block */,
-                  ix.ws_counter, ix.ws_sched, ix.ws_tc, ix.ws_grp, ix.st_q, ix.st_out, ix.st_pq};
+                  ix.ws_counter, ix.ws_sched, ix.ws_tc, ix.ws_grp, ix.ws_fl, ix.st_q, ix.st_out, ix.st_pq};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   ix.ws_qt = nullptr; ix.ws_lists = nullptr; ix.ws_d2 = nullptr; ix.ws_probes = nullptr;
@@ -474,6 +543,8 @@ void free_workspace(Index& ix) {
   ix.ws_tc_valid = false;
   ix.ws_grp = nullptr;
   ix.ws_grp_cap = 0;
+  ix.ws_fl = nullptr;
+  ix.ws_fl_cap = 0;
   ix.ws_qt_cap = ix.ws_lists_cap = ix.ws_d2_cap = ix.ws_pair_cap = ix.ws_counter_cap = 0;
   ix.ws_sched_cap = ix.st_q_cap = ix.st_out_cap = ix.st_pq_cap = 0;
   ix.ws_nq = ix.ws_nprobe = 0;

@@ -39,11 +39,9 @@
 // records ANNS_DEV_TIMEOUT in the index's device status word, tells its other
 // roles to stop, waits (with the long limit) for the copies and MMAs it has
 // issued, frees its TMEM and returns.
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cmath>
@@ -53,6 +51,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "scan.cuh"
+#include "tc.cuh"
 
 namespace anns {
 namespace {
@@ -69,7 +68,6 @@ constexpr int kEpiStride = 36;            // floats per staged epilogue row (16-
 constexpr uint32_t kEpiBytes = 4 * 32 * kEpiStride * 4;
 // alignment slack + ring + epilogue transposes + barriers; one CTA per SM (all 512 TMEM columns)
 constexpr size_t kGemmSmem = 1024 + (size_t)kStages * kStageBytes + kEpiBytes + 256;
-constexpr long long kWaitCycles = 2000000000LL;  // ~1 s at 2 GHz: the default limit and the drain's
 
 // Operand formats. Instruction descriptor (kind::f16 and kind::f8f6f4): D F32
 // (bits 4-5 = 1), A format bits 7-9 and B format bits 10-12 (kind::f16: F16 0,
@@ -111,63 +109,6 @@ template <> struct TcFmt<ANNS_PREC_FP8E4M3> {
   }
 };
 
-// Shared-memory matrix descriptor of a K-major operand written by TMA with the
-// 128-byte swizzle: start address >> 4 (bits 0-13), leading offset unused for
-// swizzled K-major (encoded 1), stride between 8-row groups 1024 bytes >> 4
-// (bits 32-45), descriptor version 1 (46-47), base offset 0 (1024-byte
-// aligned atoms), layout 128-byte swizzle (61-63 = 2). Within the 128-byte
-// row, the k-th 32-byte group (one MMA's K) starts 32 k bytes further.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1u << 16) | ((uint64_t)(1024u >> 4) << 32) |
-         (1ull << 46) | (2ull << 61);
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// 2-D tiled TMA load of box (x, y) of the tensor map into shared memory,
-// completing `bytes` on the mbarrier.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-      "[%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
-
-// Wait, for at most `limit` clock cycles, for the phase of parity `parity` of
-// the mbarrier to complete; false on timeout, or as soon as *abort is set
-// (another role of the CTA gave up).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long limit = kWaitCycles,
-                                          const volatile int* abort = nullptr) {
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (abort && *abort) return false;
-    if (clock64() - t0 > limit) return false;
-  }
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 template <int F>
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   if constexpr (F == ANNS_PREC_FP8E4M3) {
@@ -183,29 +124,6 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t
         "l"(adesc), "l"(bdesc), "r"(TcFmt<F>::kIdesc), "r"(accumulate)
         : "memory");
   }
-}
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-// 32 consecutive FP32 columns of this thread's TMEM lane.
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-      "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
-        "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
-        "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 // 2^e as an FP32 value, e in [-126, 127].
@@ -986,31 +904,6 @@ int prepare_coarse_tc(Index& ix, const std::vector<float>& cent) {
   return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "coarse fast-path setup");
 }
 
-// Tensor map of a row-major operand [rows x Dp] (elements of `elem` bytes):
-// boxes of 128 bytes x box_rows rows, 128-byte swizzle, zero fill past the
-// last row. Built through the driver entry point (no link to the driver
-// library).
-static cudaError_t make_tmap(CUtensorMap* map, CUtensorMapDataType type, int elem, const void* base, int64_t rows,
-                             int Dp, int box_rows) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qr;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qr);
-    if (e != cudaSuccess) return e;
-    if (qr != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-  }
-  const cuuint64_t dims[2] = {(cuuint64_t)Dp, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)Dp * elem};
-  const cuuint32_t box[2] = {(cuuint32_t)(kKB / elem), (cuuint32_t)box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = encode(map, type, 2, const_cast<void*>(base), dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 // Workspace: the queries' operand [nq x Dp] (any format) | rows [3][nq] |
 // candidate counts [nq] | item count | candidate lists [nq][kCap] | their
 // distances [nq][kCap] | work items [nq * kCap / 32].
@@ -1026,6 +919,15 @@ size_t coarse_tc_workspace_bytes(const Index& ix, int64_t nq) {
   return tc_operand_bytes(ix, nq) + tc_small_bytes(nq) + (size_t)nq * kCap * 8 + (size_t)nq * (kCap / 32) * 8;
 }
 
+cudaError_t launch_center_fp16(const Index& ix, const float* Q, int64_t nq, void* Qf, float* rows, cudaStream_t s) {
+  return center_any(ANNS_PREC_FP16, Q, nq, (int)ix.dim, coarse_tc_dp(ix, ANNS_PREC_FP16), ix.tc_mu, Qf, rows, s);
+}
+
+void coarse_tc_operand(const Index& ix, void* ws, int64_t nq, void** Qf, float** rows) {
+  *Qf = ws;
+  *rows = (float*)((char*)ws + tc_operand_bytes(ix, nq));
+}
+
 const int* coarse_tc_candidates(const Index& ix, const void* ws, int64_t nq) {
   return (const int*)((const char*)ws + tc_operand_bytes(ix, nq) + (size_t)nq * 12);
 }
@@ -1035,8 +937,8 @@ static cudaError_t launch_gemm(const Index& ix, void* Qf, const float* qrows, in
   using Fm = TcFmt<F>;
   const int f = fmt_slot(F), Dp = coarse_tc_dp(ix, F);
   CUtensorMap tmQ, tmC;
-  cudaError_t e = make_tmap(&tmQ, Fm::kMap, Fm::kElem, Qf, nq, Dp, kTM);
-  if (e == cudaSuccess) e = make_tmap(&tmC, Fm::kMap, Fm::kElem, ix.tc_c[f], ix.nlist, Dp, kTN);
+  cudaError_t e = make_tmap(&tmQ, Fm::kMap, Fm::kElem, Qf, nq, Dp, kKB / Fm::kElem, kTM);
+  if (e == cudaSuccess) e = make_tmap(&tmC, Fm::kMap, Fm::kElem, ix.tc_c[f], ix.nlist, Dp, kKB / Fm::kElem, kTN);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(coarse_tc_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
   int sms = 0;

@@ -35,6 +35,8 @@ void make_shadow(const Index& ix, Index& sh) {
   sh.ws_sched = nullptr; sh.ws_tc = nullptr; sh.st_q = nullptr; sh.st_out = nullptr; sh.st_pq = nullptr;
   sh.ws_tc_cap = 0;
   sh.ws_tc_valid = false;
+  sh.ws_fl = nullptr;
+  sh.ws_fl_cap = 0;
   sh.ws_grp = nullptr;
   sh.ws_grp_cap = 0;
   sh.ws_qt_cap = sh.ws_d2_cap = sh.ws_pair_cap = sh.ws_counter_cap = sh.ws_lists_cap = 0;

@@ -50,6 +50,7 @@ static void free_index(anns_index* ix) {
                   ix->tc_crows[2], ix->dev_status, ix->svr_dev};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  free_filter(*ix);
   free_workspace(*ix);
   free_subspaces(*ix);
   for (auto& set : ix->prof_ev)
@@ -245,7 +246,7 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
       (rc = upload(&ix->vec_off, voff.data(), voff.size(), "upload vec_off")) ||
       (rc = upload(&ix->tile_off, toff.data(), toff.size(), "upload tile_off")) ||
       (rc = upload(&ix->radius, ix->h_radius, (size_t)nlist, "upload radius")) ||
-      (rc = prepare_coarse_tc(*ix, cent))) {
+      (rc = prepare_coarse_tc(*ix, cent)) || (rc = prepare_filter(*ix, cent, books))) {
     free_index(ix);
     cudaSetDevice(prev);
     return rc;

@@ -12,6 +12,7 @@
 namespace anns {
 
 struct Subspaces;  // sub-space partitions (subspace.cu)
+struct FilterResult;
 
 constexpr int kKsub = 256;
 constexpr int kTileVecs = 32;         // vectors per code tile (one per lane)
@@ -53,6 +54,16 @@ struct Index {
   void* tc_c[3] = {};
   float* tc_crows[3] = {};
   int* dev_status = nullptr;
+  // tensor-core filter (filter.cu): decoded residuals in FP16 [ntiles*32][fl_w]
+  // (fl_w = 0: not available), s_x [ntiles*32], per list (largest |y|, largest
+  // rounding error, |c - mu|, 0), per sub-space the largest |y_m|
+  void* fl_y = nullptr;
+  float* fl_s = nullptr;
+  void* fl_stat = nullptr;
+  float* fl_ym = nullptr;
+  int fl_w = 0;
+  float fl_yscale = 1.f, fl_mu = 0.f;  // 1 / scale of the rows, |mu|
+  int64_t fl_tiles = 0;                // sum over the lists of their 256-vector tiles
   // host copies of the small per-list tables
   std::string err;
   int64_t* h_list_len64 = nullptr;
@@ -75,6 +86,8 @@ struct Index {
   size_t ws_sched_cap = 0;
   void* ws_grp = nullptr;        // query-major partial top-k of the grouped search
   size_t ws_grp_cap = 0;
+  void* ws_fl = nullptr;         // plan, thresholds and candidates of the filter (filter.cu)
+  size_t ws_fl_cap = 0;
   void* ws_tc = nullptr;         // BF16 centred queries, norms, candidate counts (coarse_tc.cu)
   size_t ws_tc_cap = 0;
   bool ws_tc_valid = false;      // the last search (or anns_locate) used the CL fast path
@@ -135,11 +148,17 @@ int coarse_tc_dp(const Index& ix, int prec);
 int prepare_coarse_tc(Index& ix, const std::vector<float>& cent);
 size_t coarse_tc_workspace_bytes(const Index& ix, int64_t nq);
 const int* coarse_tc_candidates(const Index& ix, const void* ws, int64_t nq);
+// The queries' FP16 operand (centred, scaled, rounded; [nq x coarse_tc_dp]) and
+// its rows [3 x nq] by themselves, and where a tensor-core CL left them.
+cudaError_t launch_center_fp16(const Index& ix, const float* Q, int64_t nq, void* Qf, float* rows, cudaStream_t s);
+void coarse_tc_operand(const Index& ix, void* ws, int64_t nq, void** Qf, float** rows);
 cudaError_t launch_coarse_tc(const Index& ix, int prec, const float* Q, int64_t nq, int nprobe,
                              const int32_t* nprobe_per_q, void* ws, float* dt, int32_t* probes,
                              float* probe_d2, cudaStream_t s);
 // Per-query tables 2*Q_q[m][c] = 2 <q_m, y_mc> (FP32 dot rule), rows M..Mp-1 zero.
-cudaError_t launch_query_tables(const Index& ix, const float* Q, int64_t nq, float* qt, cudaStream_t s);
+// With `list`, only of the *count (device) queries it names.
+cudaError_t launch_query_tables(const Index& ix, const float* Q, int64_t nq, float* qt, cudaStream_t s,
+                                const int32_t* list = nullptr, const int* count = nullptr);
 // Precision choice per (query, probe rank).
 int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq, int nprobe,
                   const int32_t* nprobe_per_q, const int32_t* probes, const float* probe_d2,
@@ -149,8 +168,9 @@ int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq,
 // table: fewer bytes of shared memory per block, more blocks per SM).
 enum { QM_TABLES_ALL = 0, QM_TABLES_FP32 = 1, QM_TABLES_NARROW = 2 };
 // RC + LC + quantise + DC + TS for every query; `order` (NULL = 0..nq-1) is
-// the order in which blocks take the queries. skip_narrow 1 leaves out the
-// 1..8-bit pairs of probe rank >= 1, 2 those of every rank. With
+// the order in which blocks take the queries; with `count` (device) only its
+// first *count entries run. skip_narrow 1 leaves out the 1..8-bit pairs of
+// probe rank >= 1, 2 those of every rank, 3 the 1..4-bit pairs of every rank. With
 // QM_TABLES_NARROW only the 1..8-bit pairs are scanned, and part_d / part_i
 // (or NULL), the query's top-k over its other pairs ([nq * k]), bound the
 // scan and join the final merge.
@@ -159,7 +179,7 @@ cudaError_t launch_search(const Index& ix, const float* qt, int64_t nq, int npro
                           const int32_t* probes, const float* probe_d2, const uint8_t* bits,
                           const int32_t* order, int64_t* ids_out, float* dists_out, cudaStream_t s,
                           int skip_narrow = 0, int tables = QM_TABLES_ALL, const float* part_d = nullptr,
-                          const int64_t* part_i = nullptr);
+                          const int64_t* part_i = nullptr, const int* count = nullptr);
 // Longest-first query order (schedule.cu) into a workspace of
 // lpt_workspace_bytes(nq); the order is at lpt_order_ptr(ws, nq).
 size_t lpt_workspace_bytes(int64_t nq);
@@ -197,10 +217,12 @@ struct ListWork {
   int *cnt4, *off4, *ioff4, *fill4, *gtab4, *counter4;
   int32_t* pairs4;
 };
-// With narrow_bits, only the pairs of probe rank >= 1 on tables of blo..bhi bits.
+// With narrow_bits, only the pairs of probe rank >= jmin on tables of blo..bhi
+// bits and, with `left`, only those the filter leaves to the grouped kernels.
 cudaError_t launch_invert(const Index& ix, const int32_t* probes, const int32_t* npq, int64_t nq,
                           int nprobe, int batch, const ListWork& w, cudaStream_t s,
-                          const uint8_t* narrow_bits = nullptr, int blo = 1, int bhi = 8);
+                          const uint8_t* narrow_bits = nullptr, int blo = 1, int bhi = 8, int jmin = 1,
+                          const FilterResult* left = nullptr);
 // Warps per block the list-major kernel gets for tables of `table_bytes_per_entry`.
 int list_major_warps(const Index& ix, int table_bytes_per_entry);
 cudaError_t launch_search_lists(const Index& ix, const float* qt, int64_t nq, int nprobe,
@@ -223,6 +245,15 @@ cudaError_t launch_search_grouped(const Index& ix, const float* qt, int64_t nq, 
                                   cudaStream_t s, cudaEvent_t after_qm = nullptr,
                                   cudaEvent_t after_packed = nullptr, cudaEvent_t after_nibble = nullptr,
                                   const int32_t* qm_order = nullptr);
+// What the filter leaves to the grouped kernels, merged with the queries' top-k
+// over their other pairs, which qm_ws holds: the pairs with a candidate (any
+// rank) on 1..4-bit tables (`nibbles`) and, of the queries not settled, on
+// 5..8-bit tables. Without `nibbles` only the unsettled queries are written.
+cudaError_t launch_search_alive(const Index& ix, const float* qt, int64_t nq, int nprobe,
+                                const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
+                                const float* probe_d2, const uint8_t* bits, const FilterResult& f, bool nibbles,
+                                const ListWork& w, void* qm_ws, int64_t* ids_out, float* dists_out, cudaStream_t s,
+                                cudaEvent_t after_packed = nullptr, cudaEvent_t after_nibble = nullptr);
 // Pair-level debug paths; qt are the queries' tables from launch_query_tables.
 cudaError_t launch_compute_luts(const Index& ix, const float* Q, const float* qt, int64_t nq,
                                 const int32_t* pq, const int32_t* pl, const uint8_t* pb,
@@ -232,6 +263,29 @@ cudaError_t launch_scan_pairs(const Index& ix, const float* Q, const float* qt, 
                               const int32_t* pq, const int32_t* pl, const uint8_t* pb,
                               int64_t npairs, const int64_t* off, float* dist_out, int32_t* S_out,
                               cudaStream_t s);
+
+// Tensor-core filter in front of the exact rules (filter.cu).
+int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<float>& books);
+void free_filter(Index& ix);
+bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k);
+size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k);
+// What the filter leaves: queries for the scanning kernel (their number on the
+// device) and the pairs on tables of at most 4 bits that are worth a scan.
+struct FilterResult {
+  const int32_t* over; const int* nover;  // queries not settled, their number
+  const uint8_t* overflag;                // [nq] the same as marks
+  const uint8_t* alive;                   // [nq * nprobe] pairs with a candidate
+  const float* thr;                       // [nq] upper bounds of the k-th distance
+};
+// The top-k over the pairs that are not on 1..4-bit tables, per query, except
+// for the queries in out->over, which get padding in over_i / over_d (if
+// given). `quantised`: some pairs are on 5..16-bit tables (qt then holds the
+// query tables); q16 and q16_rows are the queries' FP16 operand if it exists.
+cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* qt, int64_t nq, int nprobe,
+                                 const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
+                                 const float* probe_d2, const uint8_t* bits, void* ws, const void* q16,
+                                 const float* q16_rows, bool quantised, int64_t* ids_out, float* dists_out,
+                                 int64_t* over_i, float* over_d, FilterResult* out, cudaStream_t s);
 
 // Index training (train.cu): Lloyd k-means of the S rows of X [S x dim]
 // (device) into C [k x dim] (device), and the nearest centroid of each row

@@ -29,18 +29,21 @@ namespace anns {
 namespace {
 
 // Pair i takes part: probed (rank below the query's nprobe, list >= 0) and,
-// with `bits`, one the grouped kernel packs: a table of 1..8 bits and probe
-// rank >= 1 (rank 0 goes through the query-major kernel, whose result bounds
-// the query's k-th distance for the grouped pairs).
+// with `bits`, one the grouped kernel packs: a table of blo..bhi bits and probe
+// rank >= jmin (1: rank 0 goes through the query-major kernel, whose result
+// bounds the query's k-th distance for the grouped pairs), and left by the
+// filter where `alive` and `over` are given: marked in `alive` and, on a table
+// of more than 4 bits, of a query marked in `over`.
 __device__ __forceinline__ bool pair_selected(const int32_t* probes, const int32_t* npq, const uint8_t* bits,
-                                              int64_t i, int nprobe, int blo, int bhi) {
+                                              int64_t i, int nprobe, int blo, int bhi, int jmin,
+                                              const uint8_t* alive, const uint8_t* over) {
   const int64_t q = i / nprobe;
   const int j = (int)(i % nprobe);
   const int np = npq ? min(max(npq[q], 0), nprobe) : nprobe;
   if (j >= np || probes[i] < 0) return false;
   if (!bits) return true;
   const int b = bits[i];
-  return j >= 1 && b >= blo && b <= bhi;
+  return j >= jmin && b >= blo && b <= bhi && (!alive || (alive[i] && (b <= 4 || over[q])));
 }
 
 __device__ __forceinline__ int bucket_of(const int32_t* probes, int64_t i, int nprobe, int64_t qchunk, int nlist) {
@@ -49,10 +52,11 @@ __device__ __forceinline__ int bucket_of(const int32_t* probes, int64_t i, int n
 
 __global__ void count_kernel(const int32_t* __restrict__ probes, const int32_t* __restrict__ npq,
                              const uint8_t* __restrict__ bits, int blo, int bhi, int64_t nq, int nprobe,
-                             int64_t qchunk, int nlist, int* __restrict__ cnt) {
+                             int64_t qchunk, int nlist, int jmin, const uint8_t* __restrict__ alive,
+                             const uint8_t* __restrict__ over, int* __restrict__ cnt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nq * nprobe) return;
-  if (pair_selected(probes, npq, bits, i, nprobe, blo, bhi))
+  if (pair_selected(probes, npq, bits, i, nprobe, blo, bhi, jmin, alive, over))
     atomicAdd(cnt + bucket_of(probes, i, nprobe, qchunk, nlist), 1);
 }
 
@@ -106,11 +110,11 @@ __global__ void __launch_bounds__(1024) offsets_kernel(const int* __restrict__ c
 
 __global__ void scatter_kernel(const int32_t* __restrict__ probes, const int32_t* __restrict__ npq,
                                const uint8_t* __restrict__ bits, int blo, int bhi, int64_t nq, int nprobe,
-                               int64_t qchunk, int nlist, const int* __restrict__ off, int* __restrict__ fill,
-                               int32_t* __restrict__ pairs) {
+                               int64_t qchunk, int nlist, int jmin, const uint8_t* __restrict__ alive,
+                               const uint8_t* __restrict__ over, const int* __restrict__ off, int* __restrict__ fill, int32_t* __restrict__ pairs) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nq * nprobe) return;
-  if (!pair_selected(probes, npq, bits, i, nprobe, blo, bhi)) return;
+  if (!pair_selected(probes, npq, bits, i, nprobe, blo, bhi, jmin, alive, over)) return;
   const int b = bucket_of(probes, i, nprobe, qchunk, nlist);
   pairs[off[b] + atomicAdd(fill + b, 1)] = (int32_t)i;
 }
@@ -126,17 +130,20 @@ __global__ void group_table_kernel(const int* __restrict__ ioff, int nb, int* __
 
 cudaError_t launch_invert(const Index& ix, const int32_t* probes, const int32_t* npq, int64_t nq,
                           int nprobe, int batch, const ListWork& w, cudaStream_t s, const uint8_t* narrow_bits,
-                          int blo, int bhi) {
+                          int blo, int bhi, int jmin, const FilterResult* left) {
+  const uint8_t* alive = left ? left->alive : nullptr;
+  const uint8_t* over = left ? left->overflag : nullptr;
   const int64_t n = nq * nprobe;
   const int nlist = (int)ix.nlist;
   cudaError_t e = cudaMemsetAsync(w.cnt, 0, sizeof(int) * w.nbuckets, s);
   if (e != cudaSuccess) return e;
   const unsigned g = (unsigned)((n + 255) / 256);
-  count_kernel<<<g, 256, 0, s>>>(probes, npq, narrow_bits, blo, bhi, nq, nprobe, w.qchunk, nlist, w.cnt);
+  count_kernel<<<g, 256, 0, s>>>(probes, npq, narrow_bits, blo, bhi, nq, nprobe, w.qchunk, nlist, jmin, alive,
+                               over, w.cnt);
   note_launch();
   offsets_kernel<<<1, 1024, 0, s>>>(w.cnt, ix.order, nlist, w.nbuckets, batch, w.off, w.ioff, w.fill); note_launch();
-  scatter_kernel<<<g, 256, 0, s>>>(probes, npq, narrow_bits, blo, bhi, nq, nprobe, w.qchunk, nlist, w.off, w.fill,
-                                   w.pairs);
+  scatter_kernel<<<g, 256, 0, s>>>(probes, npq, narrow_bits, blo, bhi, nq, nprobe, w.qchunk, nlist, jmin, alive,
+                                   over, w.off, w.fill, w.pairs);
   note_launch();
   if (narrow_bits) {  // the grouped kernel looks its groups up in a table
     group_table_kernel<<<(unsigned)((w.nbuckets + 255) / 256), 256, 0, s>>>(w.ioff, w.nbuckets, w.gtab);

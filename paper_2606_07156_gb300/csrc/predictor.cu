@@ -548,7 +548,10 @@ int make_training_set(Index& ix, const float* Q, int64_t nq, int nprobe, int k, 
     return rc;
   tau_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>((const float*)dists.p, nq, k, (double*)tau.p);
   note_launch();
-  // the workspace now holds this batch's probes, probe D2 and query tables
+  // the workspace now holds this batch's probes and probe D2; the query tables
+  // are formed here (the search may not need them)
+  const cudaError_t eq = launch_query_tables(ix, Q, nq, ix.ws_qt, s);
+  if (eq != cudaSuccess) return cuda_fail(eq, "query tables");
   anns_precision_policy eq2{};
   eq2.lut_mode = ANNS_LUT_HEURISTIC_EQ2;
   if ((rc = launch_policy(ix, eq2, nq, nprobe, nullptr, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits, feat, s)))

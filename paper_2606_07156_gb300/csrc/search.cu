@@ -424,9 +424,10 @@ struct SearchArgs {
   int M, Mp, nprobe, k;
   const int32_t* npq; const int32_t* kpq;
   const int32_t* probes; const float* probe_d2; const uint8_t* bits;
-  const int32_t* order;
+  const int32_t* order; const int* count;  // count: only the first *count entries of `order`
   // 1: leave out the pairs on 1..8-bit tables of rank >= 1 (the grouped
-  // kernels take them); 2: of every rank (the narrow pass takes them)
+  // kernels take them); 2: of every rank (the narrow pass takes them); 3: the
+  // pairs on 1..4-bit tables (the grouped kernels take the ones worth a scan)
   int skip_narrow;
   int ids32;  // every id fits in int32 (the 128-entry lists then hold 32-bit ids)
   int64_t* ids_out; float* dists_out;
@@ -501,7 +502,8 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
   Smem s(a.lay);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tstride = (int64_t)a.Mp * kKsub;
-  for (int64_t qi = blockIdx.x; qi < a.nq; qi += gridDim.x) {
+  const int64_t nq = a.count ? *a.count : a.nq;
+  for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
     const int np = a.npq ? min(max(a.npq[q], 0), a.nprobe) : a.nprobe;
     const int kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
@@ -534,7 +536,8 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
         const bool narrow = b >= 1 && b <= 8;
         const bool use = l >= 0 && n_l > 0 &&
                          (MODE == kModeNarrow ? narrow
-                                              : !(narrow && (a.skip_narrow == 2 || (a.skip_narrow == 1 && j >= 1))));
+                                              : !(narrow && (a.skip_narrow == 2 || (a.skip_narrow == 1 && j >= 1) ||
+                                                             (a.skip_narrow == 3 && b <= 4))));
         const unsigned m = __ballot_sync(kFull, use);
         if (use) s.plist[base + __popc(m & ((1u << lane) - 1u))] = make_int4(l, n_l, b, __float_as_int(d2));
         base += __popc(m);
@@ -724,7 +727,7 @@ template <typename K>
 cudaError_t launch_query_major(K kern, const SearchArgs& a, cudaStream_t s) {
   cudaError_t e = prep(kern, a.lay.total);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min<int64_t>(a.nq, 1 << 30);
+  const unsigned grid = (unsigned)std::min<int64_t>(a.nq, a.count ? 1024 : 1 << 30);
   kern<<<grid, kThreads, a.lay.total, s>>>(a); note_launch();
   return cudaGetLastError();
 }
@@ -769,12 +772,13 @@ cudaError_t launch_search(const Index& ix, const float* qt, int64_t nq, int npro
                           const int32_t* nprobe_per_q, int k, const int32_t* k_per_q,
                           const int32_t* probes, const float* probe_d2, const uint8_t* bits,
                           const int32_t* order, int64_t* ids_out, float* dists_out, cudaStream_t s,
-                          int skip_narrow, int tables, const float* part_d, const int64_t* part_i) {
+                          int skip_narrow, int tables, const float* part_d, const int64_t* part_i, const int* count) {
   const int R = k <= 32 ? 1 : 4;
   const int mode = tables == QM_TABLES_FP32 ? kModeFp32 : tables == QM_TABLES_NARROW ? kModeNarrow : kModeFull;
   SearchArgs a = make_args(ix, nullptr, qt, R, mode);
   a.nq = nq; a.nprobe = nprobe; a.k = k; a.npq = nprobe_per_q; a.kpq = k_per_q;
-  a.probes = probes; a.probe_d2 = probe_d2; a.bits = bits; a.order = order; a.skip_narrow = skip_narrow;
+  a.probes = probes; a.probe_d2 = probe_d2; a.bits = bits; a.order = order; a.count = count;
+  a.skip_narrow = skip_narrow;
   a.ids32 = ix.ids32 ? 1 : 0;
   a.ids_out = ids_out; a.dists_out = dists_out;
   a.part_d = mode == kModeNarrow ? part_d : nullptr;

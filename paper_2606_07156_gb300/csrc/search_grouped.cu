@@ -53,6 +53,7 @@ struct GArgs {
   const int32_t* kpq;
   float* part_d; int64_t* part_i;
   const float* qm_d;  // [nq * k] query-major results (rank 0 and wide pairs): the bound
+  const float* thr;   // [nq] another upper bound of the query's k-th distance, or null
   int* counter;
 };
 
@@ -186,6 +187,7 @@ __device__ __forceinline__ void fetch_group(const GArgs& a, int ngroups, GItemT<
       d2 = a.probe_d2[p];
       kq = a.kpq ? min(max(a.kpq[qs], 0), a.k) : a.k;
       if (kq > 0) bound = a.qm_d[(size_t)qs * a.k + kq - 1];
+      if (a.thr && kq > 0) bound = fminf(bound, a.thr[qs]);
     }
     out->pid[lane] = p; out->q[lane] = qs; out->bits[lane] = bs; out->kq[lane] = kq;
     out->d2[lane] = d2; out->bound[lane] = bound;
@@ -724,11 +726,12 @@ template <int R>
 __global__ void __launch_bounds__(256) merge_grouped_kernel(
     const float* __restrict__ qm_d, const int64_t* __restrict__ qm_i, const float* __restrict__ part_d,
     const int64_t* __restrict__ part_i, const int32_t* __restrict__ probes, const uint8_t* __restrict__ bits,
-    const int32_t* __restrict__ npq, const int32_t* __restrict__ kpq, int64_t nq, int nprobe, int k,
+    const int32_t* __restrict__ npq, const int32_t* __restrict__ kpq, int64_t nq, int nprobe, int k, int jmin,
+    const uint8_t* __restrict__ alive, const uint8_t* __restrict__ over, int only_over,
     int64_t* __restrict__ ids_out, float* __restrict__ dists_out) {
   const int64_t q = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (q >= nq) return;
+  if (q >= nq || (only_over && !over[q])) return;
   const int np = npq ? min(max(npq[q], 0), nprobe) : nprobe;
   const int kq = kpq ? min(max(kpq[q], 0), k) : k;
   WarpTopK<R, int64_t> top;
@@ -747,7 +750,8 @@ __global__ void __launch_bounds__(256) merge_grouped_kernel(
   for (int j = 0; kq > 0 && j < np; ++j) {
     const int64_t pid = q * nprobe + j;
     const int b = bits[pid];
-    if (j == 0 || probes[pid] < 0 || b < 1 || b > 8) continue;
+    if (j < jmin || probes[pid] < 0 || b < 1 || b > 8) continue;
+    if (alive && !(alive[pid] && (b <= 4 || over[q]))) continue;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int e = r * 32 + lane;
@@ -817,6 +821,60 @@ bool nibble_used(const Index& ix, int k) {
   return NLayout((int)ix.Mp).total <= (size_t)optin;
 }
 
+cudaError_t run_packed_any(const Index& ix, const GArgs& a, cudaStream_t s) {
+  switch (ix.nchunk) {
+    case 1: return run_packed<1>(a, s);
+    case 2: return run_packed<2>(a, s);
+    case 3: return run_packed<3>(a, s);
+    case 4: return run_packed<4>(a, s);
+    case 5: return run_packed<5>(a, s);
+    case 6: return run_packed<6>(a, s);
+    case 7: return run_packed<7>(a, s);
+    default: return run_packed<8>(a, s);
+  }
+}
+
+cudaError_t run_nibble_any(const Index& ix, const GArgs& a, cudaStream_t s) {
+  switch (ix.nchunk) {
+    case 1: return run_nibble<1>(a, s);
+    case 2: return run_nibble<2>(a, s);
+    case 3: return run_nibble<3>(a, s);
+    case 4: return run_nibble<4>(a, s);
+    case 5: return run_nibble<5>(a, s);
+    case 6: return run_nibble<6>(a, s);
+    case 7: return run_nibble<7>(a, s);
+    default: return run_nibble<8>(a, s);
+  }
+}
+
+// The per-query merge over the partial results of the pairs of rank >= jmin on
+// 1..8-bit tables (with `left`: of those the filter leaves; only_over: of the
+// queries it did not settle only).
+cudaError_t run_merge(const float* qm_d, const int64_t* qm_i, const GArgs& a, const int32_t* probes,
+                      const uint8_t* bits, const int32_t* npq, const int32_t* kpq, int64_t nq, int nprobe, int k,
+                      int jmin, const FilterResult* left, bool only_over, int64_t* ids_out, float* dists_out,
+                      cudaStream_t s) {
+  auto kern = grouped_R(k) == 1 ? merge_grouped_kernel<1> : merge_grouped_kernel<4>;
+  kern<<<(unsigned)((nq + 7) / 8), 256, 0, s>>>(qm_d, qm_i, a.part_d, a.part_i, probes, bits, npq, kpq, nq, nprobe, k,
+                                                jmin, left ? left->alive : nullptr, left ? left->overflag : nullptr,
+                                                only_over ? 1 : 0, ids_out, dists_out);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// Arguments of the grouped kernels over the buckets of w.
+GArgs group_args(const Index& ix, const float* qt, const float* probe_d2, const uint8_t* bits, const ListWork& w,
+                 int nprobe, int k, const int32_t* kpq, const float* qm_d) {
+  GArgs a{};
+  a.qt = qt; a.ltab = ix.ltab; a.probe_d2 = probe_d2; a.bits = bits;
+  a.codes = ix.codes; a.ids = ix.ids; a.list_len = ix.list_len; a.vec_off = ix.vec_off;
+  a.tile_off = ix.tile_off; a.order = ix.order; a.cnt = w.cnt; a.off = w.off; a.ioff = w.ioff;
+  a.pairs = w.pairs; a.gtab = w.gtab; a.nlist = (int)ix.nlist; a.nb = w.nbuckets;
+  a.M = (int)ix.M; a.Mp = (int)ix.Mp; a.nprobe = nprobe; a.k = k;
+  a.kpq = kpq; a.part_d = w.part_d; a.part_i = w.part_i; a.counter = w.counter; a.qm_d = qm_d;
+  return a;
+}
+
 }  // namespace
 
 bool grouped_supported(const Index& ix, int k) {
@@ -870,51 +928,49 @@ cudaError_t launch_search_grouped(const Index& ix, const float* qt, int64_t nq, 
                     true);
   if (e != cudaSuccess) return e;
   if (after_qm) cudaEventRecord(after_qm, s);
-  GArgs a{};
-  a.qt = qt; a.ltab = ix.ltab; a.probe_d2 = probe_d2; a.bits = bits;
-  a.codes = ix.codes; a.ids = ix.ids; a.list_len = ix.list_len; a.vec_off = ix.vec_off;
-  a.tile_off = ix.tile_off; a.order = ix.order; a.cnt = w.cnt; a.off = w.off; a.ioff = w.ioff;
-  a.pairs = w.pairs; a.gtab = w.gtab; a.nlist = (int)ix.nlist; a.nb = w.nbuckets;
-  a.M = (int)ix.M; a.Mp = (int)ix.Mp; a.nprobe = nprobe; a.k = k;
-  a.kpq = k_per_q; a.part_d = w.part_d; a.part_i = w.part_i; a.counter = w.counter; a.qm_d = qm_d;
-  switch (ix.nchunk) {
-    case 1: e = run_packed<1>(a, s); break;
-    case 2: e = run_packed<2>(a, s); break;
-    case 3: e = run_packed<3>(a, s); break;
-    case 4: e = run_packed<4>(a, s); break;
-    case 5: e = run_packed<5>(a, s); break;
-    case 6: e = run_packed<6>(a, s); break;
-    case 7: e = run_packed<7>(a, s); break;
-    default: e = run_packed<8>(a, s); break;
-  }
+  const GArgs a = group_args(ix, qt, probe_d2, bits, w, nprobe, k, k_per_q, qm_d);
+  e = run_packed_any(ix, a, s);
   if (e != cudaSuccess) return e;
   if (after_packed) cudaEventRecord(after_packed, s);
   if (nib) {
     GArgs b = a;
     b.cnt = w4.cnt; b.off = w4.off; b.ioff = w4.ioff; b.pairs = w4.pairs; b.gtab = w4.gtab; b.counter = w4.counter;
-    switch (ix.nchunk) {
-      case 1: e = run_nibble<1>(b, s); break;
-      case 2: e = run_nibble<2>(b, s); break;
-      case 3: e = run_nibble<3>(b, s); break;
-      case 4: e = run_nibble<4>(b, s); break;
-      case 5: e = run_nibble<5>(b, s); break;
-      case 6: e = run_nibble<6>(b, s); break;
-      case 7: e = run_nibble<7>(b, s); break;
-      default: e = run_nibble<8>(b, s); break;
-    }
+    e = run_nibble_any(ix, b, s);
     if (e != cudaSuccess) return e;
   }
   if (after_nibble) cudaEventRecord(after_nibble, s);
-  if (grouped_R(k) == 1)
-    merge_grouped_kernel<1><<<(unsigned)((nq + 7) / 8), 256, 0, s>>>(qm_d, qm_i, w.part_d, w.part_i, probes, bits,
-                                                                   nprobe_per_q, k_per_q, nq, nprobe, k, ids_out,
-                                                                   dists_out);
-  else
-    merge_grouped_kernel<4><<<(unsigned)((nq + 7) / 8), 256, 0, s>>>(qm_d, qm_i, w.part_d, w.part_i, probes, bits,
-                                                                   nprobe_per_q, k_per_q, nq, nprobe, k, ids_out,
-                                                                   dists_out);
-  note_launch();
-  return cudaGetLastError();
+  return run_merge(qm_d, qm_i, a, probes, bits, nprobe_per_q, k_per_q, nq, nprobe, k, 1, nullptr, false, ids_out,
+                   dists_out, s);
+}
+
+cudaError_t launch_search_alive(const Index& ix, const float* qt, int64_t nq, int nprobe,
+                                const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
+                                const float* probe_d2, const uint8_t* bits, const FilterResult& f, bool nibbles,
+                                const ListWork& w, void* qm_ws, int64_t* ids_out, float* dists_out, cudaStream_t s,
+                                cudaEvent_t after_packed, cudaEvent_t after_nibble) {
+  const bool nib = nibbles && nibble_used(ix, k);
+  ListWork w4 = w;
+  w4.cnt = w.cnt4; w4.off = w.off4; w4.ioff = w.ioff4; w4.fill = w.fill4; w4.pairs = w.pairs4;
+  w4.gtab = w.gtab4; w4.counter = w.counter4;
+  cudaError_t e = launch_invert(ix, probes, nprobe_per_q, nq, nprobe, kSlots, w, s, bits, nib ? 5 : 1, 8, 0, &f);
+  if (e == cudaSuccess && nib)
+    e = launch_invert(ix, probes, nprobe_per_q, nq, nprobe, kNSlots, w4, s, bits, 1, 4, 0, &f);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.counter, 0, 16 * sizeof(int), s);  // both queues' counters
+  if (e != cudaSuccess) return e;
+  const float* qm_d = (const float*)qm_ws;
+  const int64_t* qm_i = (const int64_t*)((char*)qm_ws + (((size_t)nq * k * 4 + 255) & ~size_t(255)));
+  GArgs a = group_args(ix, qt, probe_d2, bits, w, nprobe, k, k_per_q, qm_d);
+  a.thr = f.thr;
+  if ((e = run_packed_any(ix, a, s)) != cudaSuccess) return e;
+  if (after_packed) cudaEventRecord(after_packed, s);
+  if (nib) {
+    GArgs b = group_args(ix, qt, probe_d2, bits, w4, nprobe, k, k_per_q, qm_d);
+    b.thr = f.thr;
+    if ((e = run_nibble_any(ix, b, s)) != cudaSuccess) return e;
+  }
+  if (after_nibble) cudaEventRecord(after_nibble, s);
+  return run_merge(qm_d, qm_i, a, probes, bits, nprobe_per_q, k_per_q, nq, nprobe, k, 0, &f, !nibbles, ids_out,
+                   dists_out, s);
 }
 
 }  // namespace anns

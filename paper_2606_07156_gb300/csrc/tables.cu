@@ -11,7 +11,7 @@
 namespace anns {
 namespace {
 
-// One block per query (grid-stride), thread c computes entry c of every row m
+// One block per query (grid-stride; the queries of `list`, when given), thread c computes entry c of every row m
 // and stores it coalesced. The query sub-vector is a broadcast; the codebook
 // (M x 256 x dsub floats, L1/L2 resident) is read with 16-byte loads when dsub
 // is a multiple of 4 and 8-byte loads when it is 2. Four rows at a time, their
@@ -21,9 +21,13 @@ template <int DS>  // dsub when fixed at compile time (2, 4, 8), else 0
 __global__ void __launch_bounds__(256) query_table_kernel(const float* __restrict__ Q,
                                                           const float* __restrict__ books,
                                                           int64_t nq, int dim, int M, int Mp,
-                                                          int dsub, float* __restrict__ qt) {
+                                                          int dsub, float* __restrict__ qt,
+                                                          const int32_t* __restrict__ list,
+                                                          const int* __restrict__ count) {
   const int c = threadIdx.x;
-  for (int64_t q = blockIdx.x; q < nq; q += gridDim.x) {
+  const int64_t n = list ? *count : nq;
+  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+    const int64_t q = list ? list[i] : i;
     const float* qv = Q + q * dim;
     float* out = qt + q * (int64_t)Mp * kKsub;
     if constexpr (DS > 0) {
@@ -75,17 +79,19 @@ __global__ void __launch_bounds__(256) query_table_kernel(const float* __restric
 
 }  // namespace
 
-cudaError_t launch_query_tables(const Index& ix, const float* Q, int64_t nq, float* qt, cudaStream_t s) {
+cudaError_t launch_query_tables(const Index& ix, const float* Q, int64_t nq, float* qt, cudaStream_t s,
+                                const int32_t* list, const int* count) {
   if (nq == 0) return cudaSuccess;
   static_assert(kKsub == 256, "one thread per codebook entry");
-  const int64_t grid = std::min<int64_t>(nq, (int64_t)1 << 30);
+  // the queries of a list (its length on the device): usually none or few
+  const int64_t grid = std::min<int64_t>(nq, list ? 1024 : (int64_t)1 << 30);
   const unsigned g = (unsigned)grid;
   const int dim = (int)ix.dim, M = (int)ix.M, Mp = (int)ix.Mp, ds = (int)ix.dsub;
   switch (ds) {
-    case 2: query_table_kernel<2><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt); break;
-    case 4: query_table_kernel<4><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt); break;
-    case 8: query_table_kernel<8><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt); break;
-    default: query_table_kernel<0><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt);
+    case 2: query_table_kernel<2><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt, list, count); break;
+    case 4: query_table_kernel<4><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt, list, count); break;
+    case 8: query_table_kernel<8><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt, list, count); break;
+    default: query_table_kernel<0><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt, list, count);
   }
   note_launch();
   return cudaGetLastError();
