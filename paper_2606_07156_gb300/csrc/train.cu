@@ -188,6 +188,79 @@ __global__ void __launch_bounds__(256) encode_kernel(const float* __restrict__ X
   codes[i * M + m] = (uint8_t)bc;
 }
 
+// ---- the PQ codebooks: M independent k-means of 256 clusters over the
+// sub-vectors of the same rows, run side by side (cluster m * 256 + c, member
+// m * S + row), one set of launches and one wait an iteration for all of them.
+
+// Initial entries: entry j of sub-space m = the sub-vector of row floor(j S / 256).
+__global__ void pq_init_kernel(const float* __restrict__ R, int64_t S, int64_t dim, int M, int dsub,
+                               float* __restrict__ books) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)M * 256 * dsub) return;
+  const int64_t m = t / (256 * dsub), j = t / dsub % 256, c = t % dsub;
+  books[t] = R[(j * S / 256) * dim + m * dsub + c];
+}
+
+// Nearest entry of each (row, sub-space) and its distance (FP32 rule, ties to
+// the lower entry), block (256 rows, m), the entries in shared memory: no
+// distance matrix. Bound by the FP32 pipe (3 operations a dimension and entry).
+template <int DS>
+__global__ void __launch_bounds__(256) pq_assign_kernel(const float* __restrict__ R, int64_t S, int64_t dim, int dsub,
+                                                        const float* __restrict__ books, int32_t* __restrict__ a,
+                                                        float* __restrict__ dist, int* __restrict__ cnt) {
+  float* cb = (float*)anns_dyn_smem;  // [256 * dsub]
+  __shared__ int hist[256];
+  const int m = blockIdx.y, ds = DS ? DS : dsub;
+  for (int t = threadIdx.x; t < 256 * ds; t += blockDim.x) cb[t] = books[(int64_t)m * 256 * ds + t];
+  hist[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < S) {
+    float r[DS ? DS : 16];
+#pragma unroll
+    for (int j = 0; j < (DS ? DS : 16); ++j)
+      if (j < ds) r[j] = R[i * dim + (int64_t)m * ds + j];
+    float bd = INFINITY;
+    int bc = 0;
+#pragma unroll 4
+    for (int c = 0; c < 256; ++c) {
+      float acc = 0.f;
+#pragma unroll
+      for (int j = 0; j < (DS ? DS : 16); ++j)
+        if (j < ds) {
+          const float e = sub_rn(r[j], cb[c * ds + j]);
+          acc = add_rn(acc, mul_rn(e, e));
+        }
+      if (acc < bd) { bd = acc; bc = c; }
+    }
+    a[(int64_t)m * S + i] = m * 256 + bc;
+    dist[(int64_t)m * S + i] = bd;
+    atomicAdd(&hist[bc], 1);
+  }
+  __syncthreads();
+  if (hist[threadIdx.x]) atomicAdd(cnt + m * 256 + threadIdx.x, hist[threadIdx.x]);
+}
+
+// update_kernel for the clusters of all sub-spaces: block = cluster.
+__global__ void pq_update_kernel(const float* __restrict__ R, int64_t S, int64_t dim, int dsub,
+                                 const int* __restrict__ off, const int32_t* __restrict__ members,
+                                 float* __restrict__ books) {
+  const int j = blockIdx.x, m = j >> 8;
+  const int b = off[j], e = off[j + 1];
+  if (e == b) return;  // empty: re-seeded on the host side
+  const float cntf = (float)(e - b);
+  const float* X = R + (int64_t)m * dsub - (int64_t)m * S * dim;  // member i is row i - m S
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int c = warp; c < dsub; c += nw) {
+    ExactSum acc;
+    xsum_init(acc);
+    for (int i = b + lane; i < e; i += 32) xsum_add(acc, X[(int64_t)members[i] * dim + c]);
+    xsum_warp(acc);
+    const float s = xsum_round(acc);
+    if (lane == 0) books[(int64_t)j * dsub + c] = __fdiv_rn(s, cntf);
+  }
+}
+
 struct DevBuf {
   void* p = nullptr;
   ~DevBuf() { if (p) cudaFree(p); }
@@ -307,6 +380,67 @@ int kmeans(const float* X, int64_t S, int64_t dim, int64_t k, int iters, float* 
   return ANNS_OK;
 }
 
+// The k-means of kmeans() (k = 256) for the sub-vectors m of R [S x dim], all
+// m at once (in batches of at most 2^26 members): the same codebooks.
+static int kmeans_pq(const float* R, int64_t S, int64_t dim, int64_t M_all, int iters, float* books_all, cudaStream_t s) {
+  if (S < 256) return fail(ANNS_ERR_INVALID_ARG, "the training sample has fewer rows than clusters");
+  const int dsub = (int)(dim / M_all);
+  const int64_t batch = std::max<int64_t>(1, std::min<int64_t>(M_all, ((int64_t)1 << 26) / S));
+  DevBuf a, dist, cnt, fill, members, best;
+  TRY(a.alloc(batch * S * 4));
+  TRY(dist.alloc(batch * S * 4));
+  TRY(cnt.alloc((batch * 256 + 1) * 4));
+  TRY(fill.alloc((batch * 256 + 1) * 4));
+  TRY(members.alloc(batch * S * 4));
+  TRY(best.alloc(8));
+  std::vector<int> hcnt(batch * 256);
+  for (int64_t m0 = 0; m0 < M_all; m0 += batch) {
+    const int M = (int)std::min(batch, M_all - m0);
+    const int64_t k = (int64_t)M * 256, n = (int64_t)M * S;
+    const float* Rm = R + m0 * dsub;
+    float* books = books_all + m0 * 256 * dsub;
+    pq_init_kernel<<<blocks_for(k * dsub, 256), 256, 0, s>>>(Rm, S, dim, M, dsub, books); note_launch();
+    for (int it = 0; it < iters; ++it) {
+      TRY(cudaMemsetAsync(cnt.p, 0, (k + 1) * 4, s));
+      const dim3 grid(blocks_for(S, 256), (unsigned)M);
+      const size_t smem = (size_t)256 * dsub * 4;
+      auto assign = dsub == 2 ? pq_assign_kernel<2> : dsub == 4 ? pq_assign_kernel<4>
+                                                  : dsub == 8 ? pq_assign_kernel<8> : pq_assign_kernel<0>;
+      assign<<<grid, 256, smem, s>>>(Rm, S, dim, dsub, books, a.as<int32_t>(), dist.as<float>(), cnt.as<int>());
+      note_launch();
+      TRY(cudaMemcpyAsync(hcnt.data(), cnt.p, k * 4, cudaMemcpyDeviceToHost, s));
+      scan_kernel<<<1, 1024, 0, s>>>(cnt.as<int>(), k); note_launch();
+      TRY(cudaMemcpyAsync(fill.p, cnt.p, (k + 1) * 4, cudaMemcpyDeviceToDevice, s));
+      scatter_kernel<<<blocks_for(n, 256), 256, 0, s>>>(a.as<int32_t>(), n, fill.as<int>(), members.as<int32_t>());
+      note_launch();
+      pq_update_kernel<<<(unsigned)k, 32 * std::min(dsub, 8), 0, s>>>(Rm, S, dim, dsub, cnt.as<int>(),
+                                                                       members.as<int32_t>(), books);
+      note_launch();
+      TRY(cudaStreamSynchronize(s));
+      // empty entries, ascending within their sub-space: the rows farthest from
+      // their entries, ties to the lower row
+      for (int64_t j = 0; j < k; ++j) {
+        if (hcnt[j] != 0) continue;
+        const int64_t m = j / 256;
+        float* dm = dist.as<float>() + m * S;
+        TRY(cudaMemsetAsync(best.p, 0, 8, s));
+        farthest_kernel<<<blocks_for(S, 256), 256, 0, s>>>(dm, S, best.as<unsigned long long>());
+        note_launch();
+        unsigned long long key = 0;
+        TRY(cudaMemcpyAsync(&key, best.p, 8, cudaMemcpyDeviceToHost, s));
+        TRY(cudaStreamSynchronize(s));
+        if (key == 0) return fail(ANNS_ERR_INVALID_ARG, "more empty clusters than sample rows");
+        const int64_t row = (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
+        TRY(cudaMemcpyAsync(books + j * dsub, Rm + row * dim + m * dsub, dsub * 4, cudaMemcpyDeviceToDevice, s));
+        const float taken = -1.f;
+        TRY(cudaMemcpyAsync(dm + row, &taken, 4, cudaMemcpyHostToDevice, s));
+        TRY(cudaStreamSynchronize(s));
+      }
+    }
+  }
+  return ANNS_OK;
+}
+
 }  // namespace anns
 
 using namespace anns;
@@ -332,7 +466,7 @@ extern "C" int anns_train_index(const float* base, int64_t n, int64_t dim, const
   cudaStream_t s = nullptr;
   int rc = ANNS_OK;
   {
-    DevBuf Xown, rows, Xs, cent, books, R, Ra, Rd, res, Xm, lst, ldist, codes;
+    DevBuf Xown, rows, Xs, cent, books, R, Ra, Rd, res, lst, ldist, codes;
     const float* X = base;
     do {
       if (!on_device) {
@@ -360,8 +494,7 @@ extern "C" int anns_train_index(const float* base, int64_t n, int64_t dim, const
       int64_t S2 = 0;
       if ((rc = sample(n, t->pq_sample, t->seed + 1, rows.as<int64_t>(), &S2, s))) break;
       if (R.alloc((size_t)S2 * dim * 4) != cudaSuccess || Ra.alloc((size_t)S2 * 4) != cudaSuccess ||
-          Rd.alloc((size_t)S2 * 4) != cudaSuccess || res.alloc((size_t)S2 * dim * 4) != cudaSuccess ||
-          Xm.alloc((size_t)S2 * dsub * 4) != cudaSuccess) {
+          Rd.alloc((size_t)S2 * 4) != cudaSuccess || res.alloc((size_t)S2 * dim * 4) != cudaSuccess) {
         rc = fail(ANNS_ERR_OOM, "PQ sample");
         break;
       }
@@ -373,12 +506,7 @@ extern "C" int anns_train_index(const float* base, int64_t n, int64_t dim, const
       residual_kernel<<<blocks_for(S2 * dim, 256), 256, 0, s>>>(R.as<float>(), Ra.as<int32_t>(), cent.as<float>(),
                                                                  S2, dim, res.as<float>());
       note_launch();
-      for (int64_t m = 0; m < M && rc == ANNS_OK; ++m) {
-        gather_rows_kernel<<<blocks_for(S2 * dsub, 256), 256, 0, s>>>(res.as<float>(), dim, nullptr, S2, m * dsub,
-                                                                       dsub, Xm.as<float>());
-        note_launch();
-        rc = kmeans(Xm.as<float>(), S2, dsub, 256, t->pq_iters, books.as<float>() + m * 256 * dsub, s);
-      }
+      rc = kmeans_pq(res.as<float>(), S2, dim, M, t->pq_iters, books.as<float>(), s);
       if (rc) break;
       // encoding
       if (lst.alloc((size_t)n * 4) != cudaSuccess || ldist.alloc((size_t)n * 4) != cudaSuccess ||
