@@ -352,7 +352,7 @@ static bool nibble_possible(const anns_precision_policy& P) {
 }
 
 static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
-  return filter_supported(ix, P, nq, nprobe, k) && (!nibble_possible(P) || grouped_supported(ix, k));
+  return filter_supported(ix, P, nq, nprobe, k, use_grouped(ix, P, k)) && (!nibble_possible(P) || grouped_supported(ix, k));
 }
 
 // Whether the grouped kernels follow the filter: for the pairs on 1..4-bit
@@ -440,7 +440,8 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     if (P.cl_prec == ANNS_PREC_FP16) coarse_tc_operand(ix, ix.ws_tc, nq, &q16, &q16_rows);
     FilterResult r{};
     e = launch_search_filter(ix, Q, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
-                             ix.ws_bits, ix.ws_fl, q16, q16_rows, tables_for_all, di, dd, grouped ? part_i : nullptr,
+                             ix.ws_bits, ix.ws_fl, q16, q16_rows, tables_for_all,
+                             P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8, di, dd, grouped ? part_i : nullptr,
                              grouped ? part_d : nullptr, &r, s);
     if (e != cudaSuccess) return cuda_fail(e, "filter kernels");
     // queries with more candidates than fit (usually none): their FP32, 12- and

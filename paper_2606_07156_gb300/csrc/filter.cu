@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -53,6 +54,7 @@ constexpr int kPush = 64;          // staged candidates per epilogue warp
 // ring | per epilogue warp: constants of its 64 columns, staged candidates | barriers
 constexpr uint32_t kEpiBytes = 64 * 16 + kPush * 12;
 constexpr size_t kFilterSmem = 1024 + (size_t)kFStages * kFStage + kEpiWarps * kEpiBytes + 256;
+constexpr int kBatch = 4;          // quantised pairs a warp settles at a time
 constexpr int kPosBits = 25;       // candidate word: rank << 25 | position in the list
 constexpr int kTakeMax = 4096;
 constexpr size_t kFilterWorkspaceMax = (size_t)32 << 30;  // larger batches scan
@@ -139,16 +141,23 @@ struct PlanArgs {
   float* eps;              // [nq * nprobe], -1: the pair takes no part
   float* eps0;             // [nq * nprobe] eps without the quantiser's term
   int2* sel;               // [nq * nprobe] GEMM 1: vectors taken, where their bounds go
+  uint8_t* in2;            // [nq * nprobe] the pair takes part in GEMM 2
   int* ntake;              // [nq] bounds of the query
-  int *c1, *c2, *f1, *f2;  // [nlist] pairs per list in GEMM 1 and 2, fill cursors
-  int *g1, *g2, *i1, *i2;  // [nlist + 1] first slot and item of each list
-  float2 *k1, *k2;         // [slots] column constants
-  int2* d1;                // [slots] GEMM 1: (vectors taken, destination)
-  int* p2;                 // [slots] GEMM 2: pair of each slot
+  float* thr;              // [nq] T
+  uint8_t* alive;          // [nq * nprobe]
   const __half* q16;       // [nq x Dp] the queries' FP16 operand
-  __half *r1, *r2;         // [slots x Dp] its rows slot by slot
-  int* slot2;              // [nq * nprobe] slot of each pair, -1: none
-  FItem *it1, *it2;
+};
+
+// The pairs of one GEMM regrouped by list.
+struct PassArgs {
+  int *cnt, *fill;         // [nlist] pairs per list, fill cursors
+  int *s0, *i0;            // [nlist + 1] first slot and item of each list
+  float2* kc;              // [slots] column constants
+  int2* d1;                // GEMM 1: [slots] (vectors taken, destination)
+  int* pair;               // GEMM 2: [slots]
+  __half* rows;            // [slots x Dp] the queries' rows slot by slot
+  FItem* items;
+  int tiles;               // vector tiles of a list, at most
 };
 
 // eps of a pair: |D~ - d_rule| <= eps. u = 2^-24. With r = |y|max, e = |y~ - y|
@@ -180,9 +189,9 @@ __device__ __forceinline__ float quant_eps(int M, int b, float R) {
   return 1.01f * (float)M * R * (0.5f / (float)((1 << b) - 1) + 8.f * u);
 }
 
-// One block per query: eps of its pairs, the first `take` vectors of its probe
-// sequence for GEMM 1, and the pairs counted per list.
-__global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a) {
+// One block per query: eps of its pairs and the first `take` vectors of its
+// probe sequence for GEMM 1, those pairs counted per list.
+__global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a, const PassArgs p1) {
   __shared__ int len[ANNS_MAX_NPROBE];
   const int64_t q = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -217,10 +226,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a) {
       }
       float G;
       eps = pair_eps(a, qt, qd, a.stat[l], a.d2[p], G);
-      if (lane == 0) {
-        a.eps0[p] = eps;
-        atomicAdd(a.c2 + l, 1);
-      }
+      if (lane == 0) a.eps0[p] = eps;
       if (b > 0) eps += quant_eps(a.M, b, rmax * rmax * 1.0001f + 4.f * (a.dsub + 4) * 5.9604645e-8f * G);
     }
     if (lane == 0) {
@@ -245,7 +251,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a) {
       if (j < a.nprobe) {
         const int64_t p = q * a.nprobe + j;
         a.sel[p] = make_int2(t, (int)(q * a.take) + excl);
-        if (t > 0) atomicAdd(a.c1 + a.probes[p], 1);
+        if (t > 0) atomicAdd(p1.cnt + a.probes[p], 1);
       }
       base = __shfl_sync(kFull, incl, 31);
     }
@@ -253,25 +259,23 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a) {
   }
 }
 
-// One block: exclusive prefixes over the lists of the slots and the items of
-// both GEMMs (totals at [nlist]).
-__global__ void __launch_bounds__(1024) plan_scan_kernel(const PlanArgs a) {
-  __shared__ int part[4][32];
+// One block: exclusive prefixes over the lists of a pass's slots and items
+// (totals at [nlist]).
+__global__ void __launch_bounds__(1024) plan_scan_kernel(const int32_t* __restrict__ list_len, int nlist,
+                                                         const PassArgs w) {
+  __shared__ int part[2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int carry[4] = {0, 0, 0, 0};
-  int* out[4] = {a.g1, a.i1, a.g2, a.i2};
-  for (int base = 0; base < a.nlist; base += 1024) {
+  int carry[2] = {0, 0};
+  for (int base = 0; base < nlist; base += 1024) {
     const int l = base + threadIdx.x;
-    int v[4] = {0, 0, 0, 0}, x[4];
-    if (l < a.nlist) {
-      const int tiles = (a.list_len[l] + kTv - 1) / kTv;
-      v[0] = (a.c1[l] + 15) & ~15;
-      v[1] = (a.c1[l] + kGq - 1) / kGq * min(tiles, (a.take + kTv - 1) / kTv);
-      v[2] = (a.c2[l] + 15) & ~15;
-      v[3] = (a.c2[l] + kGq - 1) / kGq * tiles;
+    int v[2] = {0, 0}, x[2];
+    if (l < nlist) {
+      const int c = w.cnt[l];
+      v[0] = (c + 15) & ~15;
+      v[1] = (c + kGq - 1) / kGq * min((list_len[l] + kTv - 1) / kTv, w.tiles);
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2; ++i) {
       x[i] = v[i];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -281,7 +285,7 @@ __global__ void __launch_bounds__(1024) plan_scan_kernel(const PlanArgs a) {
       if (lane == 31) part[i][warp] = x[i];
     }
     __syncthreads();
-    if (warp < 4) {
+    if (warp < 2) {
       int p = part[warp][lane];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -292,71 +296,71 @@ __global__ void __launch_bounds__(1024) plan_scan_kernel(const PlanArgs a) {
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (l < a.nlist) out[i][l] = carry[i] + (warp ? part[i][warp - 1] : 0) + x[i] - v[i];
+    for (int i = 0; i < 2; ++i) {
+      if (l < nlist) (i ? w.i0 : w.s0)[l] = carry[i] + (warp ? part[i][warp - 1] : 0) + x[i] - v[i];
       carry[i] += part[i][31];
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) out[i][a.nlist] = carry[i];
+  if (threadIdx.x == 0) {
+    w.s0[nlist] = carry[0];
+    w.i0[nlist] = carry[1];
+  }
 }
 
-// The first `pair_blocks` blocks: each pair to a slot of its list, a warp per
-// pair, which also copies the query's FP16 row there: the GEMM then loads a
-// group's rows as plain TMA boxes. (Gathering them in the GEMM by tile::gather4
-// took 0.1 us per four rows, 7.6 us per 128-query tile where the whole tile now
-// takes under 2.) The other blocks: the items of each list (a warp per list),
-// vector tile by vector tile, so that a tile's groups follow one another.
-__global__ void __launch_bounds__(256) plan_scatter_kernel(const PlanArgs a, int pair_blocks) {
+// The first `pair_blocks` blocks: each pair of the pass to a slot of its list,
+// a warp per pair, which also copies the query's FP16 row there: the GEMM then
+// loads a group's rows as plain TMA boxes. (Gathering them in the GEMM by
+// tile::gather4 took 0.1 us per four rows, 7.6 us per tile of 128 queries.) The
+// other blocks: the items of each list (a warp per list), vector tile by vector
+// tile, so that a tile's groups follow one another.
+template <int PASS>
+__global__ void __launch_bounds__(256) plan_scatter_kernel(const PlanArgs a, const PassArgs w, int pair_blocks) {
   const int lane = threadIdx.x & 31;
   if ((int)blockIdx.x < pair_blocks) {
-    const int64_t p = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (p >= a.nq * a.nprobe) return;
-    const float eps = a.eps[p];
-    if (eps == -1.f) {
-      if (lane == 0) a.slot2[p] = -1;
-      return;
-    }
-    const int q = (int)(p / a.nprobe), l = a.probes[p];
-    const int2 t = a.sel[p];
-    int s1 = 0, s2 = 0;
-    if (lane == 0) {
-      const float m2s = -2.f * (a.qrows[2 * a.nq + q] * a.yscale);
-      s2 = a.g2[l] + atomicAdd(a.f2 + l, 1);
-      a.p2[s2] = (int)p;
-      a.slot2[p] = s2;
-      a.k2[s2].y = m2s;
-      if (t.x > 0) {
-        s1 = a.g1[l] + atomicAdd(a.f1 + l, 1);
-        a.k1[s1] = make_float2(__fadd_ru(a.d2[p], eps), m2s);
-        a.d1[s1] = t;
+    const int64_t p0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32;  // 32 pairs a warp
+    const int64_t pl = p0 + lane;
+    int2 t = make_int2(0, 0);
+    bool in = false;
+    if (pl < a.nq * a.nprobe) {
+      if constexpr (PASS == 1) {
+        t = a.sel[pl];
+        in = t.x > 0;
+      } else {
+        in = a.in2[pl] != 0;
       }
     }
-    s1 = __shfl_sync(kFull, s1, 0);
-    s2 = __shfl_sync(kFull, s2, 0);
-    const uint4* src = (const uint4*)(a.q16 + (size_t)q * a.Dp);
-    uint4* dst2 = (uint4*)(a.r2 + (size_t)s2 * a.Dp);
-    uint4* dst1 = (uint4*)(a.r1 + (size_t)s1 * a.Dp);
-    for (int i = lane; i < a.Dp / 8; i += 32) {
-      const uint4 v = __ldg(src + i);
-      dst2[i] = v;
-      if (t.x > 0) dst1[i] = v;
+    int slot = 0, q = 0;
+    if (in) {
+      q = (int)(pl / a.nprobe);
+      const int l = a.probes[pl];
+      const float m2s = -2.f * (a.qrows[2 * a.nq + q] * a.yscale), eps = a.eps[pl], d2 = a.d2[pl];
+      slot = w.s0[l] + atomicAdd(w.fill + l, 1);
+      if constexpr (PASS == 1) {
+        w.kc[slot] = make_float2(__fadd_ru(d2, eps), m2s);
+        w.d1[slot] = t;
+      } else {
+        // D~ - eps <= T  <=>  s_x - 2 dot <= T + eps - D2 (rounded upward)
+        w.kc[slot] = make_float2(__fadd_ru(__fadd_ru(a.thr[q], eps), -d2), m2s);
+        const int b = a.bits[pl];  // sign bit: only marked, a table of at most 4 bits
+        w.pair[slot] = (int)((uint32_t)pl | (b >= 1 && b <= 4 ? 0x80000000u : 0u));
+      }
+    }
+    for (unsigned left = __ballot_sync(kFull, in); left; left &= left - 1u) {
+      const int src = __ffs(left) - 1;
+      const int qq = __shfl_sync(kFull, q, src), ss = __shfl_sync(kFull, slot, src);
+      const uint4* from = (const uint4*)(a.q16 + (size_t)qq * a.Dp);
+      uint4* to = (uint4*)(w.rows + (size_t)ss * a.Dp);
+      for (int i = lane; i < a.Dp / 8; i += 32) to[i] = __ldg(from + i);
     }
   } else {
     const int l = ((int)blockIdx.x - pair_blocks) * 8 + (threadIdx.x >> 5);
     if (l >= a.nlist) return;
-    const int n_l = a.list_len[l], row = (int)(a.tile_off[l] * kTileVecs);
-#pragma unroll
-    for (int w = 0; w < 2; ++w) {
-      const int c = w ? a.c2[l] : a.c1[l], g0 = w ? a.g2[l] : a.g1[l], i0 = w ? a.i2[l] : a.i1[l];
-      const int ng = (c + kGq - 1) / kGq, n = (w ? a.i2[l + 1] : a.i1[l + 1]) - i0;
-      FItem* out = (w ? a.it2 : a.it1) + i0;
-      for (int i = lane; i < n; i += 32) {
-        const int t = i / ng, g = i % ng;
-        out[i] = FItem{row + t * kTv, min(kTv, n_l - t * kTv) | (min(kGq, c - g * kGq) << 16), g0 + g * kGq, t * kTv};
-      }
+    const int c = w.cnt[l], i0 = w.i0[l], n = w.i0[l + 1] - i0, ng = (c + kGq - 1) / kGq;
+    const int n_l = a.list_len[l], row = (int)(a.tile_off[l] * kTileVecs), s0 = w.s0[l];
+    for (int i = lane; i < n; i += 32) {
+      const int t = i / ng, g = i % ng;
+      w.items[i0 + i] = FItem{row + t * kTv, min(kTv, n_l - t * kTv) | (min(kGq, c - g * kGq) << 16), s0 + g * kGq, t * kTv};
     }
   }
 }
@@ -444,10 +448,11 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     // producer: chunk g goes to stage g % S; lane i brings 64 rows of vectors
     // (i < 4) or 32 of queries (i - 4 < 4)
     uint32_t g = 0;
-    FItem it = load_item(a.items + blockIdx.x), nx = it;
+    FItem it = load_item(a.items + blockIdx.x), nx = it, n2 = it;
+    if ((int)blockIdx.x + stride < nitems) nx = load_item(a.items + blockIdx.x + stride);
     for (int i = blockIdx.x; i < nitems && ok; i += stride) {
       const int nv = it.nv_cnt & 0xFFFF, cnt = it.nv_cnt >> 16, nbox = (nv + 63) >> 6, qbox = (cnt + 31) >> 5;
-      if (i + stride < nitems) nx = load_item(a.items + i + stride);
+      if (i + 2 * stride < nitems) n2 = load_item(a.items + i + 2 * stride);
       for (int k = 0; k < a.nK; ++k, ++g) {
         const uint32_t st = g % kFStages;
         if (g >= kFStages) {
@@ -463,6 +468,7 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
         if (b >= 0 && b < qbox) tma_load_2d(q_dst + b * 4096, &tmQ, k * kKE, it.slot0 + 32 * b, full0 + 8 * st);
       }
       it = nx;
+      nx = n2;
     }
     if (!ok) {
       if (lane == 0) {
@@ -480,10 +486,12 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     // MMA issuer: this CTA's n-th item accumulates into TMEM columns (n & 1) * 256 + 128 * half
     uint32_t g = 0;
     int n = 0;
-    FItem it = load_item(a.items + blockIdx.x);
+    FItem it = load_item(a.items + blockIdx.x), nx = it;
+    if ((int)blockIdx.x + stride < nitems) nx = load_item(a.items + blockIdx.x + stride);
     for (int i = blockIdx.x; i < nitems && ok; i += stride, ++n) {
       const int nv = it.nv_cnt & 0xFFFF, N = ((it.nv_cnt >> 16) + 15) & ~15;
-      if (i + stride < nitems) it = load_item(a.items + i + stride);
+      it = nx;
+      if (i + 2 * stride < nitems) nx = load_item(a.items + i + 2 * stride);
       const uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);  // FP16 operands, FP32 sums
       const int b = n & 1, use = n >> 1;
       if (use > 0) ok = mbar_wait(acce0 + 8 * b, (uint32_t)((use - 1) & 1), a.wait_limit, abort_flag);
@@ -522,7 +530,7 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     const int quad = warp & 3, half = ((warp - 2) >> 2) & 1, par = (warp - 2) >> 3, r0 = half * 128 + quad * 32;
     unsigned char* mine = epi + (warp - 2) * kEpiBytes;
     float2* ck = (float2*)mine;                       // constants of the warp's columns: chunk c0 at (c0 / 64) * 32
-    int2* cd = (int2*)(mine + 64 * 8);                // GEMM 1: (taken, destination); GEMM 2: (pair, marked only)
+    int2* cd = (int2*)(mine + 64 * 8);                // GEMM 1: (taken, destination); GEMM 2: pair (sign bit: only marked)
     int* sp = (int*)(mine + 64 * 16);                 // staged candidates: pair, position, D~ - D2
     int* spos = sp + kPush;
     float* sv = (float*)(spos + kPush);
@@ -545,22 +553,24 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     auto push = [&](uint32_t mask, int j0, uint32_t tcol, const float2* kc, const int2* dc, float s, int pos) {
       for (uint32_t cols = __reduce_or_sync(kFull, mask); cols; cols &= cols - 1u) {
         const int j = __ffs(cols) - 1;
-        const int2 d = dc[j0 + j];
-        if (lane == 0) a.alive[d.x] = 1;
-        if (d.y) continue;
+        const int d = dc[j0 + j].x;
+        if (lane == 0) a.alive[d & 0x7FFFFFFF] = 1;
+        if (d < 0) continue;
         const unsigned who = __ballot_sync(kFull, mask >> j & 1u);
         const float t = fmaf(tc_ld1(tcol + j0 + j), kc[j0 + j].y, s);
         if (staged > kPush - 32) flush();
         if (mask >> j & 1u) {
           const int e = staged + __popc(who & ((1u << lane) - 1u));
-          sp[e] = d.x;
+          sp[e] = d;
           spos[e] = pos;
           sv[e] = t;
         }
         staged += __popc(who);
       }
     };
-    FItem nx = load_item(a.items + blockIdx.x);
+    // the next item's columns are requested while this one is drained, its item
+    // one step earlier: a round trip to L2 each, as long as a short tile
+    FItem nx = load_item(a.items + blockIdx.x), n2 = nx;
     float2 nk[2] = {};
     int2 nd[2] = {};
     float ns = 0.f;
@@ -576,13 +586,13 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
           if constexpr (MODE == 1) {
             nd[c] = __ldg(a.gd + s);
           } else {
-            const int p = __ldg(a.gp + s), b = a.bits[p];
-            nd[c] = make_int2(p, b >= 1 && b <= 4);
+            nd[c].x = __ldg(a.gp + s);
           }
         }
       }
     };
     load_cols(nx);
+    if ((int)blockIdx.x + stride < nitems) n2 = load_item(a.items + blockIdx.x + stride);
     int n = 0;
     for (int i = blockIdx.x; i < nitems; i += stride, ++n) {
       const FItem it = nx;
@@ -595,7 +605,9 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
         cd[lane + 32 * c] = nd[c];
       }
       __syncwarp();
-      if (i + stride < nitems) nx = load_item(a.items + i + stride);
+      nx = n2;
+      if (i + 2 * stride < nitems) n2 = load_item(a.items + i + 2 * stride);
+      if (i + stride < nitems) load_cols(nx);
       // every lane waits; the warp goes on only together (tcgen05.ld is .sync.aligned)
       const bool got = mbar_wait(accf0 + 8 * b, (uint32_t)((n >> 1) & 1), a.wait_limit, abort_flag);
       if (!__all_sync(kFull, got)) {
@@ -603,7 +615,6 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
         break;
       }
       tc_fence_after();
-      if (i + stride < nitems) load_cols(nx);
       if (r0 < nv) {
         const int pos = it.pos0 + r;
         for (int c0 = 32 * par; c0 < cnt; c0 += 64) {
@@ -696,30 +707,62 @@ __device__ __forceinline__ float warp_kth(const uint32_t (&key)[VPT], int n, int
   return __uint_as_float(hi);
 }
 
-// One warp per query: T, and the column constants of the query's pairs in
-// GEMM 2: D~ - eps <= T  <=>  s_x - 2 dot <= T + eps - D2 (rounded upward).
+// Which of a query's pairs GEMM 2 takes (lanes over the probe ranks), given T:
+//  - none of a pair that no vector can reach T from: the vectors lie within r =
+//    |y|max of the centroid, so d >= (sqrt(D2) - r)^2 (with slack for the FP32
+//    rule's rounding of D2);
+//  - not a pair on a table of at most 4 bits about half of whose vectors would
+//    pass (T + eps above the list's expected mean distance, D2 plus the mean of
+//    s_x - 2 dot over GEMM 1's vectors): it is scanned anyway.
+__device__ __forceinline__ void classify_pairs(const PlanArgs& a, const PassArgs& p2, int64_t q, float T, float mean_t,
+                                               int first, int step) {
+  for (int j = first; j < a.nprobe; j += step) {
+    const int64_t p = q * a.nprobe + j;
+    const float eps = a.eps[p];
+    bool in = eps != -1.f;
+    if (in) {
+      const float d2 = a.d2[p];
+      const int l = a.probes[p], b = a.bits[p];
+      const float away = sqrtf(d2) * (1.f - (2e-5f + 1.3e-7f * (float)a.dim)) - a.stat[l].x;
+      if (away > 0.f && away * away * 0.99999f > __fadd_ru(T, eps)) {
+        in = false;
+      } else if (b >= 1 && b <= 4 && T + eps > d2 + mean_t) {
+        a.alive[p] = 1;
+        in = false;
+      }
+      if (in) atomicAdd(p2.cnt + l, 1);
+    }
+    a.in2[p] = in ? 1 : 0;
+  }
+}
+
+// One warp per query: T from GEMM 1's bounds, then the pairs of GEMM 2.
 // take <= 32 VPT.
 template <int VPT>
-__global__ void __launch_bounds__(128) threshold_kernel(const PlanArgs a, const float* __restrict__ ub,
-                                                        float* __restrict__ thr) {
+__global__ void __launch_bounds__(128) threshold_kernel(const PlanArgs a, const PassArgs p2,
+                                                        const float* __restrict__ ub) {
   const int64_t q = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (q >= a.nq) return;
   const int n = a.ntake[q], kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
-  if (n == 0) return;  // no pair takes part
   uint32_t key[VPT];
+  float sum = 0.f;
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
     const int e = lane + 32 * i;
-    key[i] = e < n ? bound_key(ub[q * a.take + e]) : 0xFFFFFFFFu;
+    key[i] = 0xFFFFFFFFu;
+    if (e < n) {
+      const float u = ub[q * a.take + e];
+      key[i] = bound_key(u);
+      sum += u;
+    }
   }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
   const float T = warp_kth<VPT>(key, n, kq);
-  if (lane == 0) thr[q] = T;
-  for (int j = lane; j < a.nprobe; j += 32) {
-    const int64_t p = q * a.nprobe + j;
-    const int s2 = a.slot2[p];
-    if (s2 >= 0) a.k2[s2].x = __fadd_ru(__fadd_ru(T, a.eps[p]), -a.d2[p]);
-  }
+  if (lane == 0) a.thr[q] = T;
+  const float mean_t = n > 0 ? sum / (float)n - (a.d2[q * a.nprobe] + a.eps[q * a.nprobe]) : 0.f;
+  classify_pairs(a, p2, q, T, mean_t, lane, 32);
 }
 
 // ---------------------------------------------------------------- final
@@ -784,8 +827,8 @@ __device__ __forceinline__ void each_entry(const FinalArgs& a, const float* qs, 
 }
 
 constexpr int kFinalThreads = 256, kFinalWarps = kFinalThreads / 32;
-size_t final_smem(int64_t dim, int64_t Mp, int fin) {
-  return (size_t)fin * 20 + (size_t)((dim + 3) & ~int64_t(3)) * 4 + (size_t)kFinalWarps * Mp * 4;
+size_t final_smem(int64_t dim, int64_t Mp, int fin, int batch) {
+  return (size_t)fin * 20 + (size_t)((dim + 3) & ~int64_t(3)) * 4 + (size_t)kFinalWarps * batch * Mp * 4;
 }
 
 // Minimum and maximum over the warp (NaN ignored like fminf, fmaxf).
@@ -798,6 +841,104 @@ __device__ __forceinline__ float redux_max(float v) {
   float r;
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
   return r;
+}
+
+// Row statistics of the tables of n <= N quantised pairs of a query (one warp):
+// the row minima to bias[u * Mp + m], and the largest row range of each. One
+// pair: two of its rows in flight; four: a row of each, which share the row of 2
+// Q_q. What bounds this is L2 reads (1 KB a row and pair, P_l and partly 2 Q_q
+// also from HBM) and their latency.
+template <int N>
+__device__ __forceinline__ void pair_stats(const float* const (&P)[N], int n, const float* qt, int M, int Mp,
+                                           float* bias, float (&range)[N]) {
+  constexpr int R = N == 1 ? 2 : 1;
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int u = 0; u < N; ++u) range[u] = 0.f;
+  for (int m0 = 0; m0 < M; m0 += R) {
+    float qr[R][8], pr[N][R][8];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int m = min(m0 + r, M - 1);
+      ldg_row8(qt + m * kKsub, lane, qr[r]);
+#pragma unroll
+      for (int u = 0; u < N; ++u)
+        if (u < n) ldg_row8(P[u] + m * kKsub, lane, pr[u][r]);
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+      if (u >= n) break;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float lo = sub_rn(pr[u][r][0], qr[r][0]), hi = lo;
+#pragma unroll
+        for (int e = 1; e < 8; ++e) {
+          const float t = sub_rn(pr[u][r][e], qr[r][e]);
+          lo = fminf(lo, t);
+          hi = fmaxf(hi, t);
+        }
+        lo = redux_min(lo);
+        // max over entries of fl32(t - lo) = fl32(max t - lo): rounding is monotone
+        range[u] = fmaxf(range[u], sub_rn(redux_max(hi), lo));
+        if (lane == 0) bias[u * Mp + min(m0 + r, M - 1)] = lo;
+      }
+    }
+  }
+  __syncwarp();
+}
+
+// A warp's batch of pairs, in shared memory.
+template <int N>
+struct PairBatch {
+  int j[N], l[N], c0[N + 1];  // rank, list, first candidate of the batch's list (prefix)
+  float s32[N], delta[N], B32[N], reach[N];
+};
+
+__device__ __forceinline__ const uint8_t* code_of(const FinalArgs& a, int l, uint32_t pos) {
+  return a.codes + (((size_t)a.tile_off[l] + pos / kTileVecs) * a.nchunk) * kTileChunkBytes + (pos % kTileVecs) * kChunkBytes;
+}
+
+// The FP32 rule's distance of a vector, and the quantised rule's.
+template <int DS>
+__device__ __forceinline__ float exact_f32(const FinalArgs& a, const float* qs, const float* P, const uint8_t* code,
+                                           float d2) {
+  float acc = 0.f;
+  each_entry<DS, false>(a, qs, nullptr, P, code, [&](int, float t) { acc = add_rn(acc, t); });
+  return add_rn(d2, acc);
+}
+__device__ __forceinline__ float exact_quant(const FinalArgs& a, const float* qt, const float* P, const uint8_t* code,
+                                             const float* bias, float s32, float delta, float B32) {
+  int S = 0;
+  each_entry<0, true>(a, nullptr, qt, P, code, [&](int m, float t) {
+    // rint of a value in [0, 2^22): the low bits of fl32(x + 1.5 * 2^23)
+    S += (int)(__float_as_uint(add_rn(mul_rn(sub_rn(t, bias[m]), s32), 12582912.0f)) - 0x4B400000u);
+  });
+  return add_rn(mul_rn(delta, __int2float_rn(S)), B32);
+}
+
+// The statistics and scales of the n pairs in bt (ranks bt.j, lists bt.l): one
+// warp; ranges returned for the callers' bounds.
+template <int N>
+__device__ __forceinline__ void settle_pairs(const FinalArgs& a, int64_t row, int n, const float* qt, float* bias,
+                                             PairBatch<N>& bt, float (&range)[N]) {
+  const int lane = threadIdx.x & 31;
+  const float* P[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) P[u] = a.ltab + (size_t)bt.l[u < n ? u : 0] * a.Mp * kKsub;
+  pair_stats<N>(P, n, qt, a.M, a.Mp, bias, range);
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    if (u >= n) break;
+    const int64_t p = row + bt.j[u];
+    const float B32 = warp_exact_sum(bias + u * a.Mp, a.M, a.d2[p], true);
+    if (lane == 0) {
+      const float L = (float)((1 << a.bits[p]) - 1);
+      bt.s32[u] = range[u] > 0.f ? __fdiv_rn(L, range[u]) : 0.f;
+      bt.delta[u] = range[u] > 0.f ? __fdiv_rn(range[u], L) : 0.f;
+      bt.B32[u] = B32;
+    }
+  }
+  __syncwarp();
 }
 
 // warp_kth over n keys of f(e), e < n (one warp).
@@ -863,18 +1004,18 @@ __device__ __forceinline__ float block_kth(const uint32_t (&key)[VPT], int kq, i
 
 // One block per query: the candidates that can still be in the top-k, their
 // distances by the exact rules, and their ranks by (distance, id). FP32 pairs
-// take a thread per candidate. Quantised pairs take a warp per pair, in probe
-// order: the row statistics of its table (two rows of P_l and 2 Q_q in flight;
-// no block barrier, so the warps' loads overlap), then its candidates, whose
-// bound now uses the pair's true range; every finished pair lowers T to the
-// k-th exact distance so far, and a pair none of whose candidates reaches T is
-// skipped. `cap` <= VPT * kFinalThreads.
-template <int VPT, int DS>
-__global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a) {
+// take a thread per candidate. Quantised pairs are settled by warps, four at a
+// time in probe order and without block barriers: the row statistics of their
+// tables, then their candidates, whose bounds now use the pairs' true ranges;
+// every finished batch lowers T to the k-th exact distance so far, and a pair
+// none of whose candidates reaches T is skipped. `cap` <= VPT * kFinalThreads.
+template <int VPT, int DS, int BATCH>
+__global__ void __launch_bounds__(kFinalThreads, BATCH == 1 ? 4 : 2) final_kernel(const FinalArgs a) {
   __shared__ int wsum[2][32];
   __shared__ float kj[ANNS_MAX_NPROBE], tj[ANNS_MAX_NPROBE];
   __shared__ int coff[ANNS_MAX_NPROBE + 1], cfill[ANNS_MAX_NPROBE];
-  __shared__ int nvalid, next_pair;
+  __shared__ int nvalid, next_pair, npairs_s;
+  __shared__ PairBatch<BATCH> batch[kFinalWarps];
   __shared__ int T_s;  // T's bits (T >= 0: they order like the value)
   int64_t* cid = (int64_t*)anns_dyn_smem;
   float* cdist = (float*)(cid + a.fin);        // D~ - D2
@@ -883,7 +1024,7 @@ __global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a)
   float* qs = (float*)(cjp + a.fin);
   const int64_t q = blockIdx.x, row = q * a.nprobe;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  float* bias = qs + ((a.dim + 3) & ~int64_t(3)) + warp * a.Mp;
+  float* bias = qs + ((a.dim + 3) & ~int64_t(3)) + warp * BATCH * a.Mp;
   const int kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
   const int nc = a.ntake[q] > 0 ? a.qcnt[q] : 0;
   auto leave = [&]() {  // to the scanning kernels
@@ -946,9 +1087,10 @@ __global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a)
   }
   __syncthreads();
   if (warp == 0) {
-    int base = 0;
+    int base = 0, np = 0;
     for (int j0 = 0; j0 < a.nprobe; j0 += 32) {
       const int j = j0 + lane, v = j < a.nprobe ? cfill[j] : 0;
+      np += __popc(__ballot_sync(kFull, v > 0));
       int x = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -961,7 +1103,10 @@ __global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a)
       }
       base += __shfl_sync(kFull, x, 31);
     }
-    if (lane == 0) coff[a.nprobe] = base;
+    if (lane == 0) {
+      coff[a.nprobe] = base;
+      npairs_s = np;
+    }
   }
   __syncthreads();
   const int ns = coff[a.nprobe];
@@ -982,9 +1127,6 @@ __global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a)
   }
   __syncthreads();
   const float* qt = a.qt + (size_t)q * a.Mp * kKsub;
-  auto code_of = [&](int l, uint32_t pos) {
-    return a.codes + (((size_t)a.tile_off[l] + pos / kTileVecs) * a.nchunk) * kTileChunkBytes + (pos % kTileVecs) * kChunkBytes;
-  };
   // ids, and the distances of the FP32 pairs
   for (int i = tid; i < ns; i += kFinalThreads) {
     const uint32_t w = cjp[i], pos = w & kPosMask;
@@ -992,77 +1134,67 @@ __global__ void __launch_bounds__(kFinalThreads) final_kernel(const FinalArgs a)
     const int l = a.probes[p];
     cid[i] = a.ids[a.vec_off[l] + pos];
     if (a.bits[p]) continue;
-    float acc = 0.f;
-    each_entry<DS, false>(a, qs, qt, a.ltab + (size_t)l * a.Mp * kKsub, code_of(l, pos),
-                          [&](int, float t) { acc = add_rn(acc, t); });
-    cex[i] = add_rn(a.d2[p], acc);
+    cex[i] = exact_f32<DS>(a, qs, a.ltab + (size_t)l * a.Mp * kKsub, code_of(a, l, pos), a.d2[p]);
   }
   if (a.quantised) {
     __syncthreads();
-    for (;;) {
-      int j = 0;
-      if (lane == 0) j = atomicAdd(&next_pair, 1);
-      j = __shfl_sync(kFull, j, 0);
-      if (j >= a.nprobe) break;
-      const int c0 = coff[j], c1 = coff[j + 1];
-      if (c0 == c1) continue;
-      const int64_t p = row + j;
-      const int b = a.bits[p];
-      if (b == 0) continue;
-      const float d2 = a.d2[p];
-      float T = __int_as_float(*(volatile int*)&T_s);
-      bool near = false;
-      const float t0 = __fadd_ru(__fadd_ru(T, a.eps[p]), -d2);
-      for (int i = c0 + lane; i < c1; i += 32) near = near || !(cdist[i] > t0);
-      if (!__any_sync(kFull, near)) continue;  // out of reach
-      const int l = a.probes[p];
-      const float* P = a.ltab + (size_t)l * a.Mp * kKsub;
-      float range = 0.f;
-      for (int m0 = 0; m0 < a.M; m0 += 2) {
-        const int m1 = min(m0 + 1, a.M - 1);
-        float pr[2][8], qr[2][8];
-        ldg_row8(P + m0 * kKsub, lane, pr[0]);
-        ldg_row8(qt + m0 * kKsub, lane, qr[0]);
-        ldg_row8(P + m1 * kKsub, lane, pr[1]);
-        ldg_row8(qt + m1 * kKsub, lane, qr[1]);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          float lo = sub_rn(pr[u][0], qr[u][0]), hi = lo;
-#pragma unroll
-          for (int e = 1; e < 8; ++e) {
-            const float t = sub_rn(pr[u][e], qr[u][e]);
-            lo = fminf(lo, t);
-            hi = fmaxf(hi, t);
-          }
-          lo = redux_min(lo);
-          // max over entries of fl32(t - lo) = fl32(max t - lo): rounding is monotone
-          range = fmaxf(range, sub_rn(redux_max(hi), lo));
-          if (lane == 0) bias[u ? m1 : m0] = lo;
+    PairBatch<BATCH>& bt = batch[warp];
+    const int most = min(BATCH, max(1, npairs_s / (2 * kFinalWarps)));  // few pairs: spread over the warps
+    for (bool more = true; more;) {
+      // the next pairs, in probe order, with a candidate within reach of T
+      int n = 0;
+      while (n < most) {
+        int j = 0;
+        if (lane == 0) j = atomicAdd(&next_pair, 1);
+        j = __shfl_sync(kFull, j, 0);
+        if (j >= a.nprobe) {
+          more = false;
+          break;
         }
+        const int c0 = coff[j], c1 = coff[j + 1];
+        if (c0 == c1 || a.bits[row + j] == 0) continue;
+        const float t0 = __fadd_ru(__fadd_ru(__int_as_float(*(volatile int*)&T_s), a.eps[row + j]), -a.d2[row + j]);
+        bool near = false;
+        for (int i = c0 + lane; i < c1; i += 32) near = near || !(cdist[i] > t0);
+        if (!__any_sync(kFull, near)) continue;
+        if (lane == 0) {
+          bt.j[n] = j;
+          bt.l[n] = a.probes[row + j];
+          bt.c0[n + 1] = c1 - c0;
+        }
+        ++n;
+      }
+      if (n == 0) break;
+      __syncwarp();
+      float range[BATCH];
+      settle_pairs<BATCH>(a, row, n, qt, bias, bt, range);
+      const float T = __int_as_float(*(volatile int*)&T_s);
+      if (lane == 0) {
+        int at = 0;
+        for (int u = 0; u < n; ++u) {  // the pair's true range now bounds its candidates
+          const int64_t p = row + bt.j[u];
+          bt.reach[u] = __fadd_ru(__fadd_ru(T, a.eps0[p] + quant_eps(a.M, a.bits[p], range[u] * 1.0001f)), -a.d2[p]);
+          const int c = bt.c0[u + 1];
+          bt.c0[u] = at;
+          at += c;
+        }
+        bt.c0[n] = at;
       }
       __syncwarp();
-      const float B32 = warp_exact_sum(bias, a.M, d2, true);
-      const float Lf = (float)((1 << b) - 1);
-      const float s32 = range > 0.f ? __fdiv_rn(Lf, range) : 0.f, delta = range > 0.f ? __fdiv_rn(range, Lf) : 0.f;
-      T = __int_as_float(*(volatile int*)&T_s);
-      const float t1 = __fadd_ru(__fadd_ru(T, a.eps0[p] + quant_eps(a.M, b, range * 1.0001f)), -d2);
       bool lower = false;
-      for (int i = c0 + lane; i < c1; i += 32) {
-        if (cdist[i] > t1) continue;
-        int S = 0;
-        each_entry<DS, true>(a, qs, qt, P, code_of(l, cjp[i] & kPosMask), [&](int m, float t) {
-          // rint of a value in [0, 2^22): the low bits of fl32(x + 1.5 * 2^23)
-          S += (int)(__float_as_uint(add_rn(mul_rn(sub_rn(t, bias[m]), s32), 12582912.0f)) - 0x4B400000u);
-        });
-        const float d = add_rn(mul_rn(delta, __int2float_rn(S)), B32);
+      for (int e = lane; e < bt.c0[n]; e += 32) {  // the batch's candidates, one per lane
+        int u = 0;
+        while (e >= bt.c0[u + 1]) ++u;
+        const int i = coff[bt.j[u]] + e - bt.c0[u];
+        if (cdist[i] > bt.reach[u]) continue;
+        const float d = exact_quant(a, qt, a.ltab + (size_t)bt.l[u] * a.Mp * kKsub, code_of(a, bt.l[u], cjp[i] & kPosMask),
+                                    bias + u * a.Mp, bt.s32[u], bt.delta[u], bt.B32[u]);
         *(volatile float*)&cex[i] = d;  // other warps may read it: +inf or d, either is a valid bound
         lower = lower || d < T;
       }
       __syncwarp();
       if (__any_sync(kFull, lower)) {
-        const float Tn = warp_kth_of(ns, kq, [&](int e) {
-          return bound_key(*(volatile float*)&cex[e]);
-        });
+        const float Tn = warp_kth_of(ns, kq, [&](int e) { return bound_key(*(volatile float*)&cex[e]); });
         if (lane == 0) atomicMin(&T_s, (int)bound_key(Tn));
       }
     }
@@ -1162,12 +1294,7 @@ __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArg
     const int64_t p = row + (w >> kPosBits);
     const int l = a.probes[p];
     cid[i] = a.ids[a.vec_off[l] + pos];
-    const uint8_t* code = a.codes + (((size_t)a.tile_off[l] + pos / kTileVecs) * a.nchunk) * kTileChunkBytes +
-                          (pos % kTileVecs) * kChunkBytes;
-    float acc = 0.f;
-    each_entry<DS, false>(a, qs, nullptr, a.ltab + (size_t)l * a.Mp * kKsub, code,
-                          [&](int, float t) { acc = add_rn(acc, t); });
-    const float d = add_rn(a.d2[p], acc);
+    const float d = exact_f32<DS>(a, qs, a.ltab + (size_t)l * a.Mp * kKsub, code_of(a, l, pos), a.d2[p]);
     cex[i] = d;
     valid += d < INFINITY ? 1 : 0;
   }
@@ -1195,6 +1322,137 @@ __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArg
   }
 }
 
+// threshold_kernel for batches with quantised tables: the bounds of such pairs
+// are wide by the quantiser's term on either side (2 eps between D~ - eps and
+// T), so T comes from the exact distances of the vectors with the kq smallest
+// bounds instead. One block per query, a warp per pair.
+constexpr int kTWarps = 4, kExact = 512;
+size_t threshold_smem(int take, int64_t dim, int64_t Mp) {
+  return (size_t)take * 4 + (size_t)((dim + 3) & ~int64_t(3)) * 4 + (size_t)kTWarps * Mp * 4;
+}
+template <int DS>
+__global__ void __launch_bounds__(kTWarps * 32) threshold_exact_kernel(const PlanArgs a, const PassArgs p2,
+                                                                       const FinalArgs f, const float* __restrict__ ub) {
+  __shared__ uint32_t dex[kExact];
+  __shared__ int wsum[2][kTWarps], ndex;
+  __shared__ float wmean[kTWarps], T_s;
+  __shared__ PairBatch<1> batch[kTWarps];
+  __shared__ int hits[kTWarps][64];
+  uint32_t* key = (uint32_t*)anns_dyn_smem;
+  float* qs = (float*)(key + a.take);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* bias = qs + ((a.dim + 3) & ~int64_t(3)) + warp * f.Mp;
+  const int64_t q = blockIdx.x, row = q * a.nprobe;
+  const int n = a.ntake[q], kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
+  if (tid == 0) ndex = 0;
+  for (int d = tid; d < a.dim; d += kTWarps * 32) qs[d] = a.Q[q * a.dim + d];
+  float sum = 0.f;
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  for (int e = tid; e < n; e += kTWarps * 32) {
+    const float u = ub[q * a.take + e];
+    const uint32_t k = bound_key(u);
+    key[e] = k;
+    lo = min(lo, k);
+    hi = max(hi, k);
+    sum += u;
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+  lo = __reduce_min_sync(kFull, lo);
+  hi = __reduce_max_sync(kFull, hi);
+  if (lane == 0) {
+    wmean[warp] = sum;
+    wsum[0][warp] = (int)lo;
+    wsum[1][warp] = (int)hi;
+  }
+  __syncthreads();
+  sum = 0.f;
+  for (int w = 0; w < kTWarps; ++w) {
+    lo = min(lo, (uint32_t)wsum[0][w]);
+    hi = max(hi, (uint32_t)wsum[1][w]);
+    sum += wmean[w];
+  }
+  __syncthreads();
+  if (n < kq) hi = 0x7F800000u;
+  for (int step = 0; n >= kq && hi - lo > 255u; ++step) {
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    int c = 0;
+    for (int e = tid; e < n; e += kTWarps * 32) c += key[e] <= mid ? 1 : 0;
+    c = __reduce_add_sync(kFull, c);
+    if (lane == 0) wsum[step & 1][warp] = c;
+    __syncthreads();
+    int t = 0;
+    for (int w = 0; w < kTWarps; ++w) t += wsum[step & 1][w];
+    if (t >= kq) hi = mid;
+    else lo = mid + 1u;
+  }
+  // the exact distances of the vectors whose bounds are <= hi
+  const float* qt = f.qt + (size_t)q * f.Mp * kKsub;
+  auto keep = [&](float d) {
+    const int at = atomicAdd(&ndex, 1);
+    if (at < kExact) dex[at] = bound_key(d);
+  };
+  PairBatch<1>& bt = batch[warp];
+  const bool some = n >= kq && hi < 0x7F800000u;
+  for (int j = warp; some && j < a.nprobe; j += kTWarps) {
+    const int64_t p = row + j;
+    const int2 t = a.sel[p];
+    if (t.x == 0) continue;
+    const int e0 = t.y - (int)(q * a.take), l = a.probes[p], b = a.bits[p];
+    const float* P = f.ltab + (size_t)l * f.Mp * kKsub;
+    bool settled = false;
+    // 32 of the pair's vectors at a time (one by one as they come, a few lanes
+    // of a warp would wait out the whole chain of table reads)
+    auto settle = [&](int c) {
+      if (b > 0 && !settled) {
+        if (lane == 0) {
+          bt.j[0] = j;
+          bt.l[0] = l;
+        }
+        __syncwarp();
+        float range[1];
+        settle_pairs<1>(f, row, 1, qt, bias, bt, range);
+        settled = true;
+      }
+      if (lane < c) {
+        const uint8_t* code = code_of(f, l, (uint32_t)(hits[warp][lane] - e0));
+        keep(b > 0 ? exact_quant(f, qt, P, code, bias, bt.s32[0], bt.delta[0], bt.B32[0])
+                   : exact_f32<DS>(f, qs, P, code, a.d2[p]));
+      }
+      __syncwarp();
+    };
+    int c = 0;
+    for (int eb = e0; eb < e0 + t.x; eb += 32) {
+      const int e = eb + lane;
+      const bool hit = e < e0 + t.x && key[e] <= hi;
+      const unsigned m = __ballot_sync(kFull, hit);
+      if (hit) hits[warp][c + __popc(m & ((1u << lane) - 1u))] = e;
+      c += __popc(m);
+      __syncwarp();
+      if (c >= 32) {
+        settle(32);
+        c -= 32;
+        const int rest = lane < c ? hits[warp][32 + lane] : 0;
+        __syncwarp();
+        if (lane < c) hits[warp][lane] = rest;
+        __syncwarp();
+      }
+    }
+    if (c > 0) settle(c);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const float T = warp_kth_of(min(ndex, kExact), kq, [&](int e) { return dex[e]; });
+    if (lane == 0) {
+      T_s = fminf(T, __uint_as_float(hi));
+      a.thr[q] = T_s;
+    }
+  }
+  __syncthreads();
+  const float mean_t = n > 0 ? sum / (float)n - (a.d2[row] + a.eps[row]) : 0.f;
+  classify_pairs(a, p2, q, T_s, mean_t, tid, kTWarps * 32);
+}
+
 // ---------------------------------------------------------------- host side
 
 struct FilterWork {
@@ -1205,20 +1463,26 @@ struct FilterWork {
     bytes += (n * sizeof(T) + 255) & ~size_t(255);
     return p;
   }
-  int *c1, *c2, *f1, *f2, *qcnt, *nover;
-  uint8_t *alive, *overflag;
-  int *g1, *g2, *i1, *i2, *ntake, *slot2, *p2;
+  int *qcnt, *nover;
+  uint8_t *alive, *overflag, *in2;
+  int* ntake;
   float *eps, *eps0, *thr, *ub, *qrows;
-  int2 *sel, *d1;
-  float2 *k1, *k2;
-  FItem *it1, *it2;
+  int2* sel;
+  PassArgs p1{}, p2{};
   uint2* cand;
   int32_t* over;
   void* Qf;
-  __half *r1, *r2;
 };
 
-int filter_take(int k) { return k <= 16 ? 1024 : k <= 64 ? 2048 : kTakeMax; }
+// Vectors of GEMM 1 per query: more of them lower T and with it the candidates
+// of GEMM 2. While the index's rows sit in L2 the second pass over them is cheap
+// (SIFT-shaped, 1024 -> 2048: GEMM 1 35 -> 56 us, GEMM 2 545 -> 454 us); rows
+// read from HBM make GEMM 1 cost as much as it saves (Deep-shaped, 1024 -> 2048:
+// 132 -> 253 us for 32 us less in GEMM 2).
+int filter_take(const Index& ix, int k) {
+  const bool in_l2 = (double)ix.ntiles * kTileVecs * ix.fl_w * 2.0 <= 256e6;
+  return k <= 16 ? (in_l2 ? 2048 : 1024) : k <= 32 ? 2048 : kTakeMax;
+}
 int filter_fin(int k) { return k <= 32 ? 1024 : 2048; }
 int filter_cap(int k) { return k <= 32 ? 2048 : 4096; }
 
@@ -1234,29 +1498,43 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
   FilterWork w;
   w.base = base;
   const int64_t P = nq * nprobe, G = max_slots(ix, P), L = ix.nlist, Dp = coarse_tc_dp(ix, ANNS_PREC_FP16);
-  const int64_t tiles = (ix.max_list + kTv - 1) / kTv, t1 = std::min<int64_t>(tiles, (filter_take(k) + kTv - 1) / kTv);
-  w.c1 = w.take<int>(L); w.c2 = w.take<int>(L); w.f1 = w.take<int>(L); w.f2 = w.take<int>(L);
+  const int64_t tiles = (ix.max_list + kTv - 1) / kTv, t1 = std::min<int64_t>(tiles, (filter_take(ix, k) + kTv - 1) / kTv);
+  for (PassArgs* p : {&w.p1, &w.p2}) {
+    p->cnt = w.take<int>(L);
+    p->fill = w.take<int>(L);
+  }
   w.qcnt = w.take<int>(nq); w.nover = w.take<int>(1); w.alive = w.take<uint8_t>(P);
   w.overflag = w.take<uint8_t>(nq);
   w.zero_bytes = w.bytes;
-  w.g1 = w.take<int>(L + 1); w.g2 = w.take<int>(L + 1); w.i1 = w.take<int>(L + 1); w.i2 = w.take<int>(L + 1);
-  w.ntake = w.take<int>(nq); w.slot2 = w.take<int>(P);
-  w.p2 = w.take<int>(G);
-  w.eps = w.take<float>(P); w.eps0 = w.take<float>(P); w.thr = w.take<float>(nq); w.ub = w.take<float>(nq * filter_take(k));
-  w.sel = w.take<int2>(P); w.d1 = w.take<int2>(G);
-  w.k1 = w.take<float2>(G); w.k2 = w.take<float2>(G);
-  w.it1 = w.take<FItem>(max_items(ix, P, nq, t1)); w.it2 = w.take<FItem>(max_items(ix, P, nq, tiles));
+  for (PassArgs* p : {&w.p1, &w.p2}) {
+    p->tiles = (int)(p == &w.p1 ? t1 : tiles);
+    p->s0 = w.take<int>(L + 1);
+    p->i0 = w.take<int>(L + 1);
+    p->kc = w.take<float2>(G);
+    if (p == &w.p1) p->d1 = w.take<int2>(G);
+    else p->pair = w.take<int>(G);
+    p->rows = w.take<__half>(G * Dp);
+    p->items = w.take<FItem>(max_items(ix, P, nq, p->tiles));
+  }
+  w.ntake = w.take<int>(nq); w.in2 = w.take<uint8_t>(P);
+  w.eps = w.take<float>(P); w.eps0 = w.take<float>(P); w.thr = w.take<float>(nq); w.ub = w.take<float>(nq * filter_take(ix, k));
+  w.sel = w.take<int2>(P);
   w.cand = w.take<uint2>(nq * filter_cap(k));
   w.over = w.take<int32_t>(nq);
   w.qrows = w.take<float>(3 * nq);
-  w.Qf = w.take<__half>(nq * Dp); w.r1 = w.take<__half>(G * Dp); w.r2 = w.take<__half>(G * Dp);
+  w.Qf = w.take<__half>(nq * Dp);
   return w;
 }
 
+// Four pairs to a warp where a query has candidates in most of many probes (k
+// and nprobe large: embedding-shaped, 60 of 64 pairs, 8.4 -> 5.2 ms); else one,
+// which keeps more blocks resident (SIFT-shaped, about 10 pairs: 0.92 ms
+// against 1.74; uneven GIST-shaped 2.5 against 3.6).
 template <int VPT>
 cudaError_t run_final_ds(const FinalArgs& a, cudaStream_t s) {
+  const int batch = a.k >= 64 && a.nprobe >= 48 && !a.npq ? kBatch : 1;
   auto go = [&](auto kern) {
-    const size_t sm = final_smem(a.dim, a.Mp, a.fin);
+    const size_t sm = final_smem(a.dim, a.Mp, a.fin, batch);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)a.nq, kFinalThreads, sm, s>>>(a);
@@ -1264,10 +1542,10 @@ cudaError_t run_final_ds(const FinalArgs& a, cudaStream_t s) {
     return cudaGetLastError();
   };
   switch (a.dsub) {
-    case 2: return go(final_kernel<VPT, 2>);
-    case 4: return go(final_kernel<VPT, 4>);
-    case 8: return go(final_kernel<VPT, 8>);
-    default: return go(final_kernel<VPT, 0>);
+    case 2: return batch == 1 ? go(final_kernel<VPT, 2, 1>) : go(final_kernel<VPT, 2, kBatch>);
+    case 4: return batch == 1 ? go(final_kernel<VPT, 4, 1>) : go(final_kernel<VPT, 4, kBatch>);
+    case 8: return batch == 1 ? go(final_kernel<VPT, 8, 1>) : go(final_kernel<VPT, 8, kBatch>);
+    default: return batch == 1 ? go(final_kernel<VPT, 0, 1>) : go(final_kernel<VPT, 0, kBatch>);
   }
 }
 
@@ -1385,18 +1663,23 @@ void free_filter(Index& ix) {
   ix.fl_w = 0;
 }
 
-bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
+bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
+                      bool grouped_otherwise) {
   if (ix.fl_w == 0 || (ix.opt_kernel != ANNS_KERNEL_AUTO && ix.opt_kernel != ANNS_KERNEL_SPLIT)) return false;
   if (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits < 5) return false;  // every pair would be scanned anyway
-  // A search of a few short lists is over before the filter's dozen launches
-  // (about 100 us) are: a block scans a pair in about Mp (256 + list) / 2000 us,
-  // some 400 queries at a time (one query, 8 lists of 312, M = 16: 54 us
-  // scanned, 87 us filtered; 777 queries, 19 lists of 150, M = 20, 12 bits: 530
-  // and 200 us).
+  const int64_t pairs = nq * nprobe;
+  // Small searches are over before the filter's fifteen launches (100 us; 250 us
+  // with the grouped kernels behind them) are. Query-major, a block scans a pair
+  // in about Mp (256 + list) / 2000 us, some 400 queries at a time (one query, 8
+  // lists of 312, M = 16: 54 us scanned, 87 us filtered; 777 queries, 19 lists
+  // of 150, M = 20, 12 bits: 530 and 200 us). The grouped kernels spread a small
+  // batch over the GPU and take about 4.6e9 look-ups a millisecond (77 queries,
+  // 64 lists of 1094, M = 48: 304 us grouped, 364 us filtered).
+  const double lookups = (double)pairs * (double)ix.Mp * ((double)ix.n / (double)ix.nlist + 512.0);
   const double scan_us = (double)nprobe * (double)ix.Mp * (256.0 + (double)ix.n / (double)ix.nlist) / 2000.0 *
                          std::max(1.0, (double)nq / 400.0);
-  if (scan_us < 100.0) return false;
-  const int64_t pairs = nq * nprobe, tiles = (ix.max_list + kTv - 1) / kTv;
+  if (grouped_otherwise ? lookups < 2e9 : scan_us < 100.0) return false;
+  const int64_t tiles = (ix.max_list + kTv - 1) / kTv;
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))
     return false;
@@ -1410,10 +1693,10 @@ size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k) {
 cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* qt, int64_t nq, int nprobe,
                                  const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
                                  const float* probe_d2, const uint8_t* bits, void* ws, const void* q16,
-                                 const float* q16_rows, bool quantised, int64_t* ids_out, float* dists_out,
+                                 const float* q16_rows, bool quantised, bool exact_threshold, int64_t* ids_out, float* dists_out,
                                  int64_t* over_i, float* over_d, FilterResult* out, cudaStream_t s) {
   FilterWork w = filter_work(ix, nq, nprobe, k, (char*)ws);
-  cudaError_t e = cudaMemsetAsync(w.c1, 0, w.zero_bytes, s);
+  cudaError_t e = cudaMemsetAsync(w.base, 0, w.zero_bytes, s);
   if (e == cudaSuccess && !q16) {
     e = launch_center_fp16(ix, Q, nq, w.Qf, w.qrows, s);
     q16 = w.Qf;
@@ -1423,42 +1706,34 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   const int Dp = coarse_tc_dp(ix, ANNS_PREC_FP16);
   PlanArgs p{};
   p.nq = nq; p.dim = ix.dim; p.nprobe = nprobe; p.k = k; p.M = (int)ix.M; p.dsub = (int)ix.dsub; p.Dp = Dp;
-  p.take = filter_take(k); p.nlist = (int)ix.nlist; p.npq = nprobe_per_q; p.kpq = k_per_q; p.probes = probes;
+  p.take = filter_take(ix, k); p.nlist = (int)ix.nlist; p.npq = nprobe_per_q; p.kpq = k_per_q; p.probes = probes;
   p.d2 = probe_d2; p.bits = bits; p.list_len = ix.list_len; p.tile_off = ix.tile_off; p.Q = Q; p.C = ix.centroids;
   p.ym = ix.fl_ym; p.stat = (const float4*)ix.fl_stat; p.qrows = q16_rows; p.mu_norm = ix.fl_mu;
-  p.yscale = ix.fl_yscale; p.eps = w.eps; p.eps0 = w.eps0; p.sel = w.sel; p.ntake = w.ntake; p.c1 = w.c1; p.c2 = w.c2; p.f1 = w.f1;
-  p.f2 = w.f2; p.g1 = w.g1; p.g2 = w.g2; p.i1 = w.i1; p.i2 = w.i2; p.q16 = (const __half*)q16; p.r1 = w.r1; p.r2 = w.r2; p.k1 = w.k1; p.k2 = w.k2;
-  p.d1 = w.d1; p.p2 = w.p2; p.slot2 = w.slot2; p.it1 = w.it1; p.it2 = w.it2;
-  plan_kernel<<<(unsigned)nq, 128, 0, s>>>(p); note_launch();
-  plan_scan_kernel<<<1, 1024, 0, s>>>(p); note_launch();
-  const int64_t P = nq * nprobe;
-  const int pair_blocks = (int)((P + 7) / 8);
-  plan_scatter_kernel<<<(unsigned)(pair_blocks + (ix.nlist + 7) / 8), 256, 0, s>>>(p, pair_blocks); note_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  CUtensorMap tmY, tmQ1, tmQ2;
+  p.yscale = ix.fl_yscale; p.eps = w.eps; p.eps0 = w.eps0; p.sel = w.sel; p.in2 = w.in2; p.ntake = w.ntake;
+  p.thr = w.thr; p.alive = w.alive; p.q16 = (const __half*)q16;
+  const int64_t P = nq * nprobe, slots = max_slots(ix, P);
+  const int pair_blocks = (int)((P + 255) / 256);
+  const unsigned scatter_grid = (unsigned)(pair_blocks + (ix.nlist + 7) / 8);
+  CUtensorMap tmY, tmQ;
   e = make_tmap(&tmY, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ix.fl_y, ix.ntiles * kTileVecs, ix.fl_w, kKE, 64);
-  const int64_t slots = max_slots(ix, P);
-  if (e == cudaSuccess) e = make_tmap(&tmQ1, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w.r1, slots, Dp, kKE, 32);
-  if (e == cudaSuccess) e = make_tmap(&tmQ2, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w.r2, slots, Dp, kKE, 32);
   if (e != cudaSuccess) return e;
-  const int64_t tiles = (ix.max_list + kTv - 1) / kTv, t1 = std::min<int64_t>(tiles, (p.take + kTv - 1) / kTv);
   GemmArgs g{};
   g.sx = ix.fl_s; g.nK = Dp / kKE; g.ksteps = (int)((ix.dim + 15) / 16); g.status = ix.dev_status;
   g.wait_limit = ix.opt_wait_cycles > 0 ? ix.opt_wait_cycles : kWaitCycles;
-  g.nprobe = nprobe; g.bits = bits;
-  g.items = w.it1; g.nitems = w.i1 + ix.nlist; g.gk = w.k1; g.gd = w.d1; g.ub = w.ub;
-  if ((e = run_gemm<1>(ix, tmY, tmQ1, g, max_items(ix, P, nq, t1), s)) != cudaSuccess) return e;
-  const unsigned tb = (unsigned)((nq + 3) / 4);
-  switch (p.take / 32) {
-    case 32: threshold_kernel<32><<<tb, 128, 0, s>>>(p, w.ub, w.thr); break;
-    case 64: threshold_kernel<64><<<tb, 128, 0, s>>>(p, w.ub, w.thr); break;
-    default: threshold_kernel<128><<<tb, 128, 0, s>>>(p, w.ub, w.thr); break;
-  }
-  note_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  g.items = w.it2; g.nitems = w.i2 + ix.nlist; g.gk = w.k2; g.gp = w.p2; g.qcnt = w.qcnt; g.cand = w.cand;
-  g.cap = filter_cap(k); g.alive = w.alive;
-  if ((e = run_gemm<2>(ix, tmY, tmQ2, g, max_items(ix, P, nq, tiles), s)) != cudaSuccess) return e;
+  g.nprobe = nprobe; g.bits = bits; g.ub = w.ub; g.qcnt = w.qcnt; g.cand = w.cand; g.cap = filter_cap(k);
+  g.alive = w.alive;
+  auto pass = [&](auto mode, const PassArgs& w1) {
+    constexpr int MODE = decltype(mode)::value;
+    plan_scan_kernel<<<1, 1024, 0, s>>>(ix.list_len, (int)ix.nlist, w1); note_launch();
+    plan_scatter_kernel<MODE><<<scatter_grid, 256, 0, s>>>(p, w1, pair_blocks); note_launch();
+    cudaError_t e1 = cudaGetLastError();
+    if (e1 == cudaSuccess) e1 = make_tmap(&tmQ, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w1.rows, slots, Dp, kKE, 32);
+    if (e1 != cudaSuccess) return e1;
+    g.items = w1.items; g.nitems = w1.i0 + ix.nlist; g.gk = w1.kc; g.gd = w1.d1; g.gp = w1.pair;
+    return run_gemm<MODE>(ix, tmY, tmQ, g, max_items(ix, P, nq, w1.tiles), s);
+  };
+  plan_kernel<<<(unsigned)nq, 128, 0, s>>>(p, w.p1); note_launch();
+  if ((e = pass(std::integral_constant<int, 1>{}, w.p1)) != cudaSuccess) return e;
   FinalArgs f{};
   f.nq = nq; f.dim = ix.dim; f.nprobe = nprobe; f.k = k; f.M = (int)ix.M; f.Mp = (int)ix.Mp; f.nchunk = (int)ix.nchunk;
   f.dsub = (int)ix.dsub; f.cap = g.cap; f.fin = filter_fin(k); f.npq = nprobe_per_q; f.kpq = k_per_q; f.probes = probes; f.d2 = probe_d2;
@@ -1466,6 +1741,33 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   f.books = ix.codebooks; f.ltab = ix.ltab; f.qt = qt; f.codes = ix.codes; f.ids = ix.ids; f.tile_off = ix.tile_off;
   f.vec_off = ix.vec_off; f.over = w.over; f.nover = w.nover; f.ids_out = ids_out; f.dists_out = dists_out;
   f.overflag = w.overflag; f.over_i = over_i; f.over_d = over_d;
+  if (exact_threshold) {
+    auto go = [&](auto kern) {
+      const size_t sm = threshold_smem(p.take, ix.dim, ix.Mp);
+      const cudaError_t e1 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e1 != cudaSuccess) return e1;
+      kern<<<(unsigned)nq, kTWarps * 32, sm, s>>>(p, w.p2, f, w.ub);
+      note_launch();
+      return cudaGetLastError();
+    };
+    switch (ix.dsub) {
+      case 2: e = go(threshold_exact_kernel<2>); break;
+      case 4: e = go(threshold_exact_kernel<4>); break;
+      case 8: e = go(threshold_exact_kernel<8>); break;
+      default: e = go(threshold_exact_kernel<0>); break;
+    }
+  } else {
+    const unsigned tb = (unsigned)((nq + 3) / 4);
+    switch (p.take / 32) {
+    case 32: threshold_kernel<32><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
+      case 64: threshold_kernel<64><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
+      default: threshold_kernel<128><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
+    }
+    note_launch();
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  if ((e = pass(std::integral_constant<int, 2>{}, w.p2)) != cudaSuccess) return e;
   if (quantised) {
     e = f.cap == 2048 ? run_final_ds<8>(f, s) : run_final_ds<16>(f, s);
   } else {

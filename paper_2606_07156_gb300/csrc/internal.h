@@ -267,7 +267,9 @@ cudaError_t launch_scan_pairs(const Index& ix, const float* Q, const float* qt, 
 // Tensor-core filter in front of the exact rules (filter.cu).
 int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<float>& books);
 void free_filter(Index& ix);
-bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k);
+// Whether the filter serves the call; grouped_otherwise: the grouped kernels would.
+bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
+                      bool grouped_otherwise);
 size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k);
 // What the filter leaves: queries for the scanning kernel (their number on the
 // device) and the pairs on tables of at most 4 bits that are worth a scan.
@@ -280,11 +282,13 @@ struct FilterResult {
 // The top-k over the pairs that are not on 1..4-bit tables, per query, except
 // for the queries in out->over, which get padding in over_i / over_d (if
 // given). `quantised`: some pairs are on 5..16-bit tables (qt then holds the
-// query tables); q16 and q16_rows are the queries' FP16 operand if it exists.
+// query tables); `exact_threshold`: the nearest ones are, so that the k-th
+// distance is better bounded by exact distances than by upper bounds; q16 and q16_rows are the queries' FP16 operand if it exists.
 cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* qt, int64_t nq, int nprobe,
                                  const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
                                  const float* probe_d2, const uint8_t* bits, void* ws, const void* q16,
-                                 const float* q16_rows, bool quantised, int64_t* ids_out, float* dists_out,
+                                 const float* q16_rows, bool quantised, bool exact_threshold, int64_t* ids_out,
+                                 float* dists_out,
                                  int64_t* over_i, float* over_d, FilterResult* out, cudaStream_t s);
 
 // Index training (train.cu): Lloyd k-means of the S rows of X [S x dim]

@@ -35,6 +35,7 @@ def make_index(amp, dim, M, sizes, seed, spread=0.35):
     codes = r.integers(0, 256, (len(lo), M)).astype(np.uint8)
     ids = r.permutation(10 * len(lo))[:len(lo)].astype(np.int64)
     g = amp.Index(cent, books, codes, lo, ids=ids, device=0)
+    g.set_kernel("split")  # filtered at these sizes whatever the tables (automatic: small quantised batches are grouped)
     return r, g, ivfpq.Index(cent, books, codes, lo, ids)
 
 
@@ -97,6 +98,7 @@ def test_queries_left_to_the_scan(amp):
     codes[lo == 0] = 7
     codes[lo == 2] = 9
     g = amp.Index(cent, books, codes, lo, device=0)
+    g.set_kernel("split")
     o = ivfpq.Index(cent, books, codes, lo)
     Q = (cent[r.integers(0, 6, 40)] + 0.1 * r.standard_normal((40, 32))).astype(np.float32)
     Q[3] = cent[0]
@@ -126,6 +128,7 @@ def test_scales(amp):
         lo = r.integers(0, 12, 20000).astype(np.int32)
         codes = r.integers(0, 256, (20000, 12)).astype(np.uint8)
         g = amp.Index(cent, books, codes, lo, device=0)
+        g.set_kernel("split")
         o = ivfpq.Index(cent, books, codes, lo)
         Q = (cent[r.integers(0, 12, 33)] + 0.4 * scale * r.standard_normal((33, 48))).astype(np.float32)
         try:
