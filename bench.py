@@ -488,7 +488,7 @@ def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray):
     """Names of the profile stages (anns_profile) for the search that ran, and
     the candidates for the roofline's dominant kernel: (label, source file, ms
     per step, algorithmic code bytes). `kernel` is the autotuner's choice
-    ("split", "grouped", ...; None: the automatic one), `st_ms` the stage
+    ("split", "grouped", "automatic" (filtered), ...; None: the one without a trial), `st_ms` the stage
     times, `bits` and `pb` the pairs' table widths and code bytes [nq, nprobe].
     The split search runs its wide pairs (stage 3) and then every 1..8-bit pair
     (stage 4); the grouped search runs every rank-0 pair and the wide pairs in
@@ -504,6 +504,11 @@ def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray):
              st_ms[3], int(pb[~narrow].sum())),
             ("search_kernel (split search, narrow pass: 1..8-bit byte tables; two-pass build + scan + top-k)",
              "search.cu", st_ms[4], int(pb[narrow].sum()))]
+    if kernel == "automatic":
+        names = STAGES_CL + ("filtered_search (plan + two GEMM passes + exact distances)", "grouped_kernel_5to8bit (unsettled)",
+                             "grouped_kernel_4bit_nibble (pairs with candidates)", "grouped_merge")
+        return names, [("filter_gemm_kernel (filtered search: all of plan, GEMM passes and exact distances)", "filter.cu",
+                        st_ms[3], int(pb.sum()))]
     names = STAGES_CL + ("search_before_grouped (invert + query-major)", "grouped_kernel_5to8bit",
                          "grouped_kernel_4bit_nibble", "grouped_merge")
     if not (st_ms[4] > 0.0 or st_ms[5] > 0.0):
@@ -643,8 +648,8 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
     # picks on this batch (kernel, query order, grouped work-order chunk);
     # the others in the automatic one
     KN = {abi.KERNEL_BASIC: "query-major", abi.KERNEL_LIST_MAJOR: "list-major", abi.KERNEL_GROUPED: "grouped",
-          abi.KERNEL_SPLIT: "split"}
-    SN = {abi.SCHED_NATURAL: "natural", abi.SCHED_LPT: "longest-first"}
+          abi.KERNEL_SPLIT: "split", abi.KERNEL_AUTO: "automatic"}
+    SN = {abi.SCHED_AUTO: "automatic", abi.SCHED_NATURAL: "natural", abi.SCHED_LPT: "longest-first"}
     tuned = None
     if not args.no_autotune:
         trials = index.autotune(Q, nprobe, k, adaptive, reps=2)

@@ -207,7 +207,8 @@ enum { ANNS_PREC_FP32 = 0, ANNS_PREC_BF16 = 1, ANNS_PREC_FP8E4M3 = 2, ANNS_PREC_
 typedef struct {
   int32_t lut_mode;        /* ANNS_LUT_* */
   int32_t fixed_bits;      /* 4, 6, 8, 12 or 16 (FIXED_BITS) */
-  int32_t cl_prec;         /* coarse distances: ANNS_PREC_FP32, or a tensor-core GEMM
+  int32_t cl_prec;         /* coarse distances: ANNS_PREC_FP32 (large batches may go
+                              through the FP16 GEMM below: same output), or a GEMM
                               on centred operands scaled per row by a power of two,
                               in ANNS_PREC_BF16, ANNS_PREC_FP16 or ANNS_PREC_FP8E4M3
                               with FP32 accumulation, then every list within the
@@ -329,8 +330,9 @@ int anns_scan_pairs(anns_index* index, const float* queries, int64_t nq,
  *   0 CL distances, 1 CL selection (the tensor-core CL: the whole stage in 1),
  *   2 precision choice plus the per-query tables, 3 the search kernels up to
  *   the grouped kernels (the whole LUT + scan + top-k for the query-major and
- *   list-major kernels; pair regrouping plus the query-major pass for the
- *   grouped search; the wide pass of the split search), 4 the grouped kernel
+ *   list-major kernels; the filter and its exact distances; pair regrouping
+ *   plus the query-major pass for the grouped search; the wide pass of the split
+ *   search), 4 the grouped kernel
  *   of the 5..8-bit tables (of all narrow tables without nibble packing; the
  *   narrow pass of the split search), 5 the grouped kernel of the 4-bit
  *   tables packed eight to a word, 6 the grouped search's per-query merge
@@ -358,8 +360,16 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
 
 /* Index options.
  *  ANNS_OPT_KERNEL: which search kernel anns_search launches.
- *    ANNS_KERNEL_AUTO (default): grouped when the policy can choose tables of
- *      at most 8 bits (k <= 128), else query-major.
+ *    ANNS_KERNEL_AUTO (default): filtered when the batch is large enough: a
+ *      tensor-core GEMM of the lists' decoded vectors (held in FP16, 2 * dim
+ *      bytes a vector, where that is at most a quarter of the free device
+ *      memory when the index is built) with the queries bounds every distance,
+ *      and only the vectors that can reach a query's top-k are evaluated by the
+ *      exact rules; pairs on tables of at most 4 bits with such vectors, and
+ *      queries with too many, are scanned by the kernels below. Else grouped
+ *      when the policy can choose tables of at most 8 bits (k <= 128) and the
+ *      batch is not very small, else query-major (several blocks a query for a
+ *      few queries).
  *    ANNS_KERNEL_BASIC: query-major, one block per query walking its probes.
  *    ANNS_KERNEL_GROUPED: the pairs on 1..8-bit tables taken four per list,
  *      their byte tables interleaved so that one shared-memory gather serves
@@ -372,7 +382,8 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
  *    ANNS_KERNEL_SPLIT: query-major in two passes split by table width: the
  *      FP32 and 12/16-bit pairs into a per-query partial top-k, then the
  *      1..8-bit pairs with byte tables only (no FP32 table in shared memory,
- *      so more blocks per SM), bounded by and merged with the partial.
+ *      so more blocks per SM), bounded by and merged with the partial. Large
+ *      batches are filtered first, as with ANNS_KERNEL_AUTO.
  *  ANNS_OPT_SCHEDULE: the order in which the query-major kernel takes queries
  *    (the greedy load scheduling of Section 4.3, applied to queries).
  *    ANNS_SCHED_AUTO (default): longest first when nprobe_per_q is given (an
@@ -387,12 +398,12 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
  *    the list tables and codes fit in the other half, else one chunk.
  *    Values >= 1 fix the chunk.
  *  ANNS_OPT_WAIT_CYCLES: the limit, in SM clock cycles, of each wait inside
- *    the tensor-core CL kernel's main loop (its mbarrier waits on TMA copies,
- *    stage releases and the accumulator). 0 (default) = 2e9 cycles (about
+ *    the main loops of the tensor-core kernels, CL and filter (their mbarrier
+ *    waits on TMA copies, stage releases and the accumulator). 0 (default) = 2e9 cycles (about
  *    one second). A wait that runs out makes the kernel record a timeout in
  *    the index's status word (anns_sync_status), wait with the long limit for
  *    the copies and MMAs it has issued, free its tensor memory and return;
- *    the coarse stage's output is then invalid. Small values serve tests of
+ *    the call's output is then invalid. Small values serve tests of
  *    this failure path.
  *  ANNS_OPT_NIBBLE: 1 (default) = in the grouped search (k <= 32), the pairs
  *    on tables of at most 4 bits are taken eight per list, their levels
@@ -425,8 +436,9 @@ int anns_graph_launch(anns_graph* graph, void* cuda_stream);
 void anns_graph_free(anns_graph* graph);
 
 /* Autotuner: times every available configuration on the given batch (reps
- * timed searches each, after one untimed): the query-major kernel in query
- * order and longest first, the list-major kernel, and the grouped kernel in
+ * timed searches each, after one untimed): the automatic choice (filtered for
+ * a large batch), the query-major kernel in query order and longest first, the
+ * split search in both, the list-major kernel, and the grouped kernel in
  * both query orders with its automatic work order and with query chunks of
  * a half and a quarter of the batch (when >= 256 queries). Installs the
  * fastest as the index's options and reports all of them (at most cap, in

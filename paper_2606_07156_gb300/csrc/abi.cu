@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "predictor.cuh"
+#include "select_small.cuh"
 
 namespace anns {
 namespace {
@@ -53,14 +54,16 @@ __device__ __forceinline__ uint8_t eq2_bits(const float f[5], const float th[4])
 // levels), 12 and 16 -> FP32 (a 16-bit table gathers as slowly as FP32).
 __device__ __forceinline__ uint8_t gpu_width(uint8_t b) { return b == 6 ? 8 : (b == 12 || b == 16) ? 0 : b; }
 
-__global__ void policy_kernel(const PolicyArgs p) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= p.nq * p.nprobe) return;
-  const int64_t q = idx / p.nprobe;
-  const int j = (int)(idx % p.nprobe);
+// The width of pair (q, j) and its features. WARP: called by a whole warp, whose
+// lanes share the MLP (a thread's 2300 dependent operations are 25 us however
+// few pairs there are).
+template <bool WARP>
+__device__ __forceinline__ uint8_t choose_bits(const PolicyArgs& p, int64_t q, int j, float f[5]) {
+  const int64_t idx = q * p.nprobe + j;
   const int np = p.npq ? min(max(p.npq[q], 0), p.nprobe) : p.nprobe;
   const int l = p.probes[idx];
-  float f[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) f[i] = 0.f;
   uint8_t b = 0;
   if (j < np && l >= 0) {
     switch (p.mode) {
@@ -74,15 +77,104 @@ __global__ void policy_kernel(const PolicyArgs p) {
         break;
       case ANNS_LUT_MLP:
         features_of(p, q, j, np, f);
-        b = mlp_decide(*(const MlpParams16*)p.mlp, f, p.margin);
+        b = WARP ? mlp_decide_warp(*(const MlpParams16*)p.mlp, f, p.margin)
+                 : mlp_decide(*(const MlpParams16*)p.mlp, f, p.margin);
         if (p.width_map) b = gpu_width(b);
         break;
     }
   }
+  return b;
+}
+
+__device__ __forceinline__ void write_bits(const PolicyArgs& p, int64_t idx, uint8_t b, const float f[5]) {
   p.bits[idx] = b;
   if (p.feat) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) p.feat[idx * 5 + i] = f[i];
+  }
+}
+
+template <bool WARP>
+__global__ void policy_kernel(const PolicyArgs p) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, idx = WARP ? t >> 5 : t;
+  if (idx >= p.nq * p.nprobe) return;
+  float f[5];
+  const uint8_t b = choose_bits<WARP>(p, idx / p.nprobe, (int)(idx % p.nprobe), f);
+  if (WARP && (threadIdx.x & 31) != 0) return;
+  write_bits(p, idx, b, f);
+}
+
+// The stages before the scan in one launch, for a few queries on a small index:
+// coarse distances (FP32 rule), the probes, the widths and the query's table, a
+// block per query. Four launches of a few microseconds each otherwise.
+struct FrontArgs {
+  const float* Q; const float* C; const float* books;
+  int nlist, dim, M, Mp, dsub;
+  int32_t* probes; float* probe_d2; float* qt;
+  PolicyArgs pol;
+};
+template <int R>
+__global__ void __launch_bounds__(kSmallThreads) front_kernel(const FrontArgs a) {
+  __shared__ SelectSmem sm;
+  float* qv = (float*)anns_dyn_smem;           // [dim rounded up to 4]
+  float* row = qv + ((a.dim + 3) & ~3);        // [nlist]
+  const int64_t q = blockIdx.x;
+  const int tid = threadIdx.x, np_max = a.pol.nprobe;
+  for (int d = tid; d < a.dim; d += kSmallThreads) qv[d] = a.Q[q * a.dim + d];
+  __syncthreads();
+  for (int l = tid; l < a.nlist; l += kSmallThreads) {
+    const float* c = a.C + (int64_t)l * a.dim;
+    float acc = 0.f;
+    if (a.dim % 4 == 0) {
+#pragma unroll 8
+      for (int i = 0; i < a.dim; i += 4) {
+        const float4 v = __ldg((const float4*)(c + i));
+        float e = sub_rn(qv[i], v.x);
+        acc = add_rn(acc, mul_rn(e, e));
+        e = sub_rn(qv[i + 1], v.y);
+        acc = add_rn(acc, mul_rn(e, e));
+        e = sub_rn(qv[i + 2], v.z);
+        acc = add_rn(acc, mul_rn(e, e));
+        e = sub_rn(qv[i + 3], v.w);
+        acc = add_rn(acc, mul_rn(e, e));
+      }
+    } else {
+#pragma unroll 8
+      for (int i = 0; i < a.dim; ++i) {
+        const float e = sub_rn(qv[i], __ldg(c + i));
+        acc = add_rn(acc, mul_rn(e, e));
+      }
+    }
+    row[l] = acc;
+  }
+  __syncthreads();
+  const int np = a.pol.npq ? min(max(a.pol.npq[q], 0), np_max) : np_max;
+  select_small<R>(row, a.nlist, np_max, np, a.probes + q * np_max, a.probe_d2 + q * np_max, sm);
+  __syncthreads();
+  if (a.pol.mode == ANNS_LUT_MLP) {
+    for (int j = tid >> 5; j < np_max; j += kSmallThreads / 32) {
+      float f[5];
+      const uint8_t b = choose_bits<true>(a.pol, q, j, f);
+      if ((tid & 31) == 0) write_bits(a.pol, q * np_max + j, b, f);
+    }
+  } else {
+    for (int j = tid; j < np_max; j += kSmallThreads) {
+      float f[5];
+      const uint8_t b = choose_bits<false>(a.pol, q, j, f);
+      write_bits(a.pol, q * np_max + j, b, f);
+    }
+  }
+  // 2 Q_q by the rule of tables.cu, two rows of 256 entries at a time
+  float* out = a.qt + q * (int64_t)a.Mp * kKsub;
+  const int c = tid & 255;
+#pragma unroll 4
+  for (int m = tid >> 8; m < a.Mp; m += kSmallThreads / 256) {
+    float acc = 0.f;
+    if (m < a.M) {
+      const float* y = a.books + ((size_t)m * kKsub + c) * a.dsub;
+      for (int j = 0; j < a.dsub; ++j) acc = add_rn(acc, mul_rn(qv[m * a.dsub + j], __ldg(y + j)));
+    }
+    out[m * kKsub + c] = mul_rn(2.f, acc);
   }
 }
 
@@ -248,11 +340,9 @@ cudaEvent_t* next_profile_slot(Index& ix) {
   return ev;
 }
 
-}  // namespace
-
-int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq, int nprobe,
-                  const int32_t* nprobe_per_q, const int32_t* probes, const float* probe_d2,
-                  uint8_t* bits, float* feat, cudaStream_t s) {
+PolicyArgs policy_args(const Index& ix, const anns_precision_policy& pol, int64_t nq, int nprobe,
+                       const int32_t* nprobe_per_q, const int32_t* probes, const float* probe_d2, uint8_t* bits,
+                       float* feat) {
   PolicyArgs p{};
   p.nq = nq; p.nprobe = nprobe; p.npq = nprobe_per_q; p.probes = probes; p.probe_d2 = probe_d2;
   p.list_len = ix.list_len; p.radius = ix.radius; p.mode = pol.lut_mode;
@@ -261,6 +351,40 @@ int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq,
   p.margin = pol.fallback_margin; p.pair_bits = pol.pair_bits; p.mlp = ix.mlp_dev;
   p.width_map = pol.width_map;
   p.bits = bits; p.feat = feat;
+  return p;
+}
+
+// One launch for a few queries on an index whose centroids a block reads in
+// about a microsecond (half a megabyte).
+bool front_fits(const Index& ix, const anns_precision_policy& P, int64_t nq) {
+  return ix.opt_kernel == ANNS_KERNEL_AUTO && P.cl_prec == ANNS_PREC_FP32 && P.lut_mode != ANNS_LUT_SVR && nq <= 64 &&
+         ix.nlist <= 2048 && ix.nlist * ix.dim <= 131072 && ix.dim <= 4096;
+}
+
+cudaError_t launch_front(const Index& ix, const anns_precision_policy& P, const float* Q, int64_t nq, int nprobe,
+                         const int32_t* nprobe_per_q, float* feat, cudaStream_t s) {
+  FrontArgs a{};
+  a.Q = Q; a.C = ix.centroids; a.books = ix.codebooks; a.nlist = (int)ix.nlist; a.dim = (int)ix.dim; a.M = (int)ix.M;
+  a.Mp = (int)ix.Mp; a.dsub = (int)ix.dsub; a.probes = ix.ws_probes; a.probe_d2 = ix.ws_probe_d2; a.qt = ix.ws_qt;
+  a.pol = policy_args(ix, P, nq, nprobe, nprobe_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits, feat);
+  const size_t smem = (size_t)((ix.dim + 3) & ~int64_t(3)) * 4 + (size_t)ix.nlist * 4;  // at most 24 KB
+  const unsigned g = (unsigned)nq;
+  switch ((nprobe + 31) / 32) {
+    case 1: front_kernel<1><<<g, kSmallThreads, smem, s>>>(a); break;
+    case 2: front_kernel<2><<<g, kSmallThreads, smem, s>>>(a); break;
+    case 3: front_kernel<3><<<g, kSmallThreads, smem, s>>>(a); break;
+    default: front_kernel<4><<<g, kSmallThreads, smem, s>>>(a); break;
+  }
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq, int nprobe,
+                  const int32_t* nprobe_per_q, const int32_t* probes, const float* probe_d2,
+                  uint8_t* bits, float* feat, cudaStream_t s) {
+  const PolicyArgs p = policy_args(ix, pol, nq, nprobe, nprobe_per_q, probes, probe_d2, bits, feat);
   const int64_t n = nq * nprobe;
   if (pol.lut_mode == ANNS_LUT_SVR) {
     SvrArgs m{};
@@ -271,7 +395,9 @@ int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq,
     if (e != cudaSuccess) return cuda_fail(e, "svr policy kernel attribute");
     svr_policy_kernel<<<(unsigned)((n + 255) / 256), 256, smem, s>>>(p, m); note_launch();
   } else {
-    policy_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p); note_launch();
+    if (pol.lut_mode == ANNS_LUT_MLP && n <= 16384) policy_kernel<true><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(p);
+    else policy_kernel<false><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p);
+    note_launch();
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "policy kernel");
@@ -319,11 +445,29 @@ int anns::check_search_args(anns_index* ix, const float* Q, int64_t nq, int32_t 
 
 namespace anns {
 
+// The operand format the coarse stage runs in (FP32: the CUDA cores).
+static int coarse_route(const Index& ix, int cl_prec, int64_t nq) {
+  return cl_prec == ANNS_PREC_FP32 && coarse_fp32_by_tc(ix, nq) ? ANNS_PREC_FP16 : cl_prec;
+}
+
+// A batch of few pairs whose policy the grouped kernels would serve, but that
+// the query-major kernel with several blocks a query finishes sooner: the pairs
+// form no groups, and the regrouping, two grouped kernels and merge are some
+// 200 us of latency. A block scans a pair in about Mp (256 + list) / 6500 us
+// with the GPU full (304 blocks). (16 queries, 32 lists of 2441, M = 48, mixed
+// widths: 285 us grouped, 140 us so)
+static bool small_mixed(const Index& ix, int64_t nq, int nprobe) {
+  const double pair_us = (double)ix.Mp * (256.0 + (double)ix.n / (double)ix.nlist) / 6500.0;
+  return ix.opt_kernel == ANNS_KERNEL_AUTO && ix.opt_schedule == ANNS_SCHED_AUTO && search_split(nq, nprobe, 1) > 1 &&
+         std::ceil((double)nq * nprobe / 304.0) * pair_us < 120.0;
+}
+
 // The grouped kernel (narrow pairs packed four to a word): on request, or by
-// default for a policy that can choose 1..8-bit tables, when k <= 128.
-static bool use_grouped(const Index& ix, const anns_precision_policy& P, int k) {
+// default for a policy that can choose 1..8-bit tables, when k <= 128 and the
+// batch is large enough for groups.
+static bool use_grouped(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
   if (ix.opt_kernel == ANNS_KERNEL_GROUPED) return grouped_supported(ix, k);
-  if (ix.opt_kernel != ANNS_KERNEL_AUTO) return false;
+  if (ix.opt_kernel != ANNS_KERNEL_AUTO || small_mixed(ix, nq, nprobe)) return false;
   const bool narrow_possible = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
                                P.lut_mode == ANNS_LUT_EXPLICIT || P.lut_mode == ANNS_LUT_SVR ||
                                (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8);
@@ -351,8 +495,15 @@ static bool nibble_possible(const anns_precision_policy& P) {
          P.lut_mode == ANNS_LUT_SVR;
 }
 
-static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
-  return filter_supported(ix, P, nq, nprobe, k, use_grouped(ix, P, k)) && (!nibble_possible(P) || grouped_supported(ix, k));
+// Blocks per query of the automatic query-major search (all queries of such a
+// batch run at once: their order does not matter).
+static int split_of(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
+  return ix.opt_kernel == ANNS_KERNEL_AUTO && ix.opt_schedule == ANNS_SCHED_AUTO && !use_grouped(ix, P, nq, nprobe, k)
+             ? search_split(nq, nprobe, k) : 1;
+}
+
+static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven) {
+  return filter_supported(ix, P, nq, nprobe, k, use_grouped(ix, P, nq, nprobe, k), uneven) && (!nibble_possible(P) || grouped_supported(ix, k));
 }
 
 // Whether the grouped kernels follow the filter: for the pairs on 1..4-bit
@@ -369,7 +520,7 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
                    const int32_t* nprobe_per_q) {
   int rc = ensure_workspace(ix, nq, nprobe);
   if (rc) return rc;
-  if (use_filter(ix, P, nq, nprobe, k)) {
+  if (use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr)) {
     if ((rc = grow(&ix.ws_fl, &ix.ws_fl_cap, filter_workspace_bytes(ix, nq, nprobe, k)))) return rc;
     if (grouped_after_filter(ix, P, k)) {
       ListWork w{};
@@ -377,19 +528,22 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
       if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
     }
   } else {
-    if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, k)) {
+    if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, nq, nprobe, k)) {
       ListWork w{};
       const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
       if ((rc = list_workspace(ix, nq, nprobe, k, w, qchunk))) return rc;
     }
-    if (use_grouped(ix, P, k) || ix.opt_kernel == ANNS_KERNEL_SPLIT) {
+    if (use_grouped(ix, P, nq, nprobe, k) || ix.opt_kernel == ANNS_KERNEL_SPLIT) {
       if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
     }
-    if (ix.opt_kernel != ANNS_KERNEL_LIST_MAJOR && use_lpt(ix, nprobe_per_q)) {
+    const int split = split_of(ix, P, nq, nprobe, k);
+    if (split > 1) {
+      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq * split, k)))) return rc;
+    } else if (ix.opt_kernel != ANNS_KERNEL_LIST_MAJOR && use_lpt(ix, nprobe_per_q)) {
       if ((rc = grow(&ix.ws_sched, &ix.ws_sched_cap, lpt_workspace_bytes(nq)))) return rc;
     }
   }
-  if (coarse_tc_format(P.cl_prec)) {
+  if (coarse_route(ix, P.cl_prec, nq) != ANNS_PREC_FP32) {
     if ((rc = grow(&ix.ws_tc, &ix.ws_tc_cap, coarse_tc_workspace_bytes(ix, nq)))) return rc;
   }
   return ANNS_OK;
@@ -406,9 +560,17 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
   ix.ws_tc_valid = coarse_tc_format(P.cl_prec);
   ix.ws_tc_prec = P.cl_prec;
   ix.ws_tc_nq = nq;
-  if (ix.ws_tc_valid) {
+  const int cl = coarse_route(ix, P.cl_prec, nq);
+  const bool want_feat = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
+                         P.lut_mode == ANNS_LUT_SVR;
+  const bool filter = use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  const bool front = !filter && front_fits(ix, P, nq);
+  if (front) {
+    e = launch_front(ix, P, Q, nq, nprobe, nprobe_per_q, want_feat ? ix.ws_feat : nullptr, s);
     if (ev) cudaEventRecord(ev[1], s);
-    e = launch_coarse_tc(ix, P.cl_prec, Q, nq, nprobe, nprobe_per_q, ix.ws_tc, ix.ws_d2, ix.ws_probes,
+  } else if (cl != ANNS_PREC_FP32) {
+    if (ev) cudaEventRecord(ev[1], s);
+    e = launch_coarse_tc(ix, cl, Q, nq, nprobe, nprobe_per_q, ix.ws_tc, ix.ws_d2, ix.ws_probes,
                          ix.ws_probe_d2, s);
   } else {
     e = launch_coarse(ix, Q, nq, nprobe, nprobe_per_q, ix.ws_d2, ix.ws_probes, ix.ws_probe_d2, s,
@@ -416,15 +578,13 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
   }
   if (e != cudaSuccess) return cuda_fail(e, "coarse kernels");
   if (ev) cudaEventRecord(ev[2], s);
-  const bool want_feat = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
-                         P.lut_mode == ANNS_LUT_SVR;
-  if ((rc = launch_policy(ix, P, nq, nprobe, nprobe_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits,
+  if (!front &&
+      (rc = launch_policy(ix, P, nq, nprobe, nprobe_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits,
                           want_feat ? ix.ws_feat : nullptr, s)))
     return rc;
-  const bool filter = use_filter(ix, P, nq, nprobe, k);
   // the filtered search forms the few FP32 entries it needs itself
   const bool tables_for_all = !filter || P.lut_mode != ANNS_LUT_PLAIN_FP32;
-  e = tables_for_all ? launch_query_tables(ix, Q, nq, ix.ws_qt, s) : cudaSuccess;
+  e = tables_for_all && !front ? launch_query_tables(ix, Q, nq, ix.ws_qt, s) : cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(e, "query tables");
   if (filter) {
     if (ev) cudaEventRecord(ev[3], s);
@@ -437,7 +597,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     float* dd = nib ? part_d : dists_out;
     void* q16 = nullptr;
     float* q16_rows = nullptr;
-    if (P.cl_prec == ANNS_PREC_FP16) coarse_tc_operand(ix, ix.ws_tc, nq, &q16, &q16_rows);
+    if (cl == ANNS_PREC_FP16) coarse_tc_operand(ix, ix.ws_tc, nq, &q16, &q16_rows);
     FilterResult r{};
     e = launch_search_filter(ix, Q, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
                              ix.ws_bits, ix.ws_fl, q16, q16_rows, tables_for_all,
@@ -479,7 +639,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     if (ev) cudaEventRecord(ev[3], s);
     e = launch_search_lists(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
                             ix.ws_bits, tbytes, w, ids_out, dists_out, s);
-  } else if (use_grouped(ix, P, k)) {
+  } else if (use_grouped(ix, P, nq, nprobe, k)) {
     ListWork w{};
     if ((rc = list_workspace(ix, nq, nprobe, k, w, grouped_qchunk(ix, nq)))) return rc;
     // longest-first order of the query-major pass, over the pairs it scans
@@ -496,8 +656,9 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     if (e == cudaSuccess && ev) cudaEventRecord(ev[7], s);
     return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "search kernel");
   } else {
+    const int split = split_of(ix, P, nq, nprobe, k);
     const int32_t* order = nullptr;
-    if (use_lpt(ix, nprobe_per_q)) {
+    if (split == 1 && use_lpt(ix, nprobe_per_q)) {
       e = launch_lpt_order(ix, ix.ws_probes, nprobe_per_q, nq, nprobe, ix.ws_sched, s, ix.ws_bits, false);
       if (e != cudaSuccess) return cuda_fail(e, "schedule kernels");
       order = lpt_order_ptr(ix.ws_sched, nq);
@@ -523,8 +684,16 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     const int tables = P.lut_mode == ANNS_LUT_PLAIN_FP32 ? QM_TABLES_FP32
                        : P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8 ? QM_TABLES_NARROW
                                                                                  : QM_TABLES_ALL;
-    e = launch_search(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
-                      ix.ws_bits, order, ids_out, dists_out, s, 0, tables);
+    if (split > 1) {
+      float* part_d = (float*)ix.ws_grp;
+      int64_t* part_i = (int64_t*)((char*)ix.ws_grp + (((size_t)nq * split * k * 4 + 255) & ~size_t(255)));
+      e = launch_search(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2, ix.ws_bits,
+                        nullptr, part_i, part_d, s, 0, tables, nullptr, nullptr, nullptr, split);
+      if (e == cudaSuccess) e = launch_merge_split(part_d, part_i, split, k_per_q, nq, k, ids_out, dists_out, s);
+    } else {
+      e = launch_search(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
+                        ix.ws_bits, order, ids_out, dists_out, s, 0, tables);
+    }
   }
   if (e != cudaSuccess) return cuda_fail(e, "search kernel");
   if (ev)
@@ -586,9 +755,10 @@ extern "C" int anns_locate(anns_index* ix, const float* Q, int64_t nq, int32_t n
   ix->ws_tc_valid = coarse_tc_format(cl_prec);
   ix->ws_tc_prec = cl_prec;
   ix->ws_tc_nq = nq;
-  if (ix->ws_tc_valid) {
+  const int cl = coarse_route(*ix, cl_prec, nq);
+  if (cl != ANNS_PREC_FP32) {
     if ((rc = grow(&ix->ws_tc, &ix->ws_tc_cap, coarse_tc_workspace_bytes(*ix, nq)))) return rc;
-    e = launch_coarse_tc(*ix, cl_prec, Q, nq, nprobe, nprobe_per_q, ix->ws_tc, ix->ws_d2, probes_out, probe_d2_out,
+    e = launch_coarse_tc(*ix, cl, Q, nq, nprobe, nprobe_per_q, ix->ws_tc, ix->ws_d2, probes_out, probe_d2_out,
                          s);
   } else {
     e = launch_coarse(*ix, Q, nq, nprobe, nprobe_per_q, ix->ws_d2, probes_out, probe_d2_out, s);

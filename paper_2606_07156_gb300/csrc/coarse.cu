@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "select_small.cuh"
 
 namespace anns {
 namespace {
@@ -68,6 +69,42 @@ __global__ void __launch_bounds__(256) coarse_d2_kernel(const float* __restrict_
     }
   }
   }
+}
+
+// The same distances for a few queries: one thread per (query, list), its row
+// read directly with 16-byte loads (dim % 4 == 0). The tiled kernel's 64-query
+// tile is then mostly empty and its chain of staged chunks is all latency (one
+// query, 64 lists, D = 128: 16 us).
+__global__ void __launch_bounds__(128) coarse_d2_small_kernel(const float* __restrict__ Q, const float* __restrict__ C,
+                                                              int64_t nlist, int dim, float* __restrict__ d2) {
+  const int64_t q = blockIdx.y, l = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (l >= nlist) return;
+  const float4* c = (const float4*)(C + l * dim);
+  const float* x = Q + q * dim;
+  float acc = 0.f;
+#pragma unroll 8
+  for (int i = 0; i < dim / 4; ++i) {
+    const float4 v = __ldg(c + i);
+    float e = sub_rn(__ldg(x + 4 * i), v.x);
+    acc = add_rn(acc, mul_rn(e, e));
+    e = sub_rn(__ldg(x + 4 * i + 1), v.y);
+    acc = add_rn(acc, mul_rn(e, e));
+    e = sub_rn(__ldg(x + 4 * i + 2), v.z);
+    acc = add_rn(acc, mul_rn(e, e));
+    e = sub_rn(__ldg(x + 4 * i + 3), v.w);
+    acc = add_rn(acc, mul_rn(e, e));
+  }
+  d2[q * nlist + l] = acc;
+}
+
+template <int R>
+__global__ void __launch_bounds__(kSmallThreads) coarse_select_small_kernel(
+    const float* __restrict__ d2, int64_t nlist, int nprobe, const int32_t* __restrict__ npq,
+    int32_t* __restrict__ probes, float* __restrict__ probe_d2) {
+  __shared__ SelectSmem sm;
+  const int64_t q = blockIdx.x;
+  const int np = npq ? min(max(npq[q], 0), nprobe) : nprobe;
+  select_small<R>(d2 + q * nlist, nlist, nprobe, np, probes + q * nprobe, probe_d2 + q * nprobe, sm);
 }
 
 // One warp per query: the nprobe_q smallest (D2, list id). D2 >= 0, so the
@@ -165,9 +202,35 @@ __global__ void __launch_bounds__(256) coarse_select_kernel(const float* __restr
 
 }  // namespace
 
+// A batch whose (query, list) pairs fill the GPU at most a few times over.
+static bool small_batch(const Index& ix, int64_t nq) { return nq <= 64 && nq * ix.nlist <= (1 << 18); }
+
 cudaError_t launch_coarse(const Index& ix, const float* Q, int64_t nq, int nprobe,
                           const int32_t* nprobe_per_q, float* d2, int32_t* probes,
                           float* probe_d2, cudaStream_t s, cudaEvent_t between) {
+  if (small_batch(ix, nq)) {
+    const bool v4 = ix.dim % 4 == 0 && ((uintptr_t)ix.centroids & 15u) == 0;
+    if (v4) {
+      coarse_d2_small_kernel<<<dim3((unsigned)((ix.nlist + 127) / 128), (unsigned)nq), 128, 0, s>>>(
+          Q, ix.centroids, ix.nlist, (int)ix.dim, d2);
+    } else {
+      coarse_d2_kernel<<<dim3((unsigned)((ix.nlist + kTL - 1) / kTL), (unsigned)((nq + kTQ - 1) / kTQ)), 256, 0, s>>>(
+          Q, ix.centroids, nq, ix.nlist, ix.dim, d2);
+    }
+    note_launch();
+    if (between) cudaEventRecord(between, s);
+    auto go = [&](auto kern) {
+      kern<<<(unsigned)nq, kSmallThreads, 0, s>>>(d2, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2);
+    };
+    switch ((nprobe + 31) / 32) {
+      case 1: go(coarse_select_small_kernel<1>); break;
+      case 2: go(coarse_select_small_kernel<2>); break;
+      case 3: go(coarse_select_small_kernel<3>); break;
+      default: go(coarse_select_small_kernel<4>); break;
+    }
+    note_launch();
+    return cudaGetLastError();
+  }
   dim3 g1((unsigned)((ix.nlist + kTL - 1) / kTL), (unsigned)std::min<int64_t>((nq + kTQ - 1) / kTQ, 65535));
   coarse_d2_kernel<<<g1, 256, 0, s>>>(Q, ix.centroids, nq, ix.nlist, ix.dim, d2); note_launch();
   if (between) cudaEventRecord(between, s);

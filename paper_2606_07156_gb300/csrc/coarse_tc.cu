@@ -22,13 +22,13 @@
 //    -> coalesced rows of D~), so that a tile's epilogue overlaps the next
 //    tile's MMAs.
 // 3. Error bound per pair: |D~ - D2| <= eps(D~, rows), D2 the FP32-rule
-//    distance (derivation at rerank_bound). T = the nprobe-th smallest of the
-//    upper bounds D~ + eps (rounded up by at most 255 units of its last place:
-//    a radix select that stops at bins of 256); every list of the FP32
-//    top-nprobe has D~ - eps <= T, so those candidates are re-ranked with the
+//    distance (derivation at rerank_bound). From the nprobe-th
+//    smallest D~ and the largest eps of any list follows a limit of D~ that no
+//    list of the FP32 top-nprobe exceeds (candidate_limit; rerank_stream_kernel
+//    uses each list's own eps); the lists below are re-ranked with the
 //    FP32 rule itself (same operation order as coarse.cu) and the nprobe
 //    smallest (D2, l) kept: identical output to the plain path. The re-rank
-//    runs in three kernels: a select kernel per query (bounds, T, the
+//    runs in three kernels: a select kernel per query (the limit, the
 //    candidate list, up to kCap of them to the workspace as work items of 32),
 //    a distance kernel whose warps walk every query's items, and a merge
 //    kernel (one warp per query); indexes whose keys do not fit in shared
@@ -367,6 +367,7 @@ struct RerankArgs {
   int32_t* probes;
   float* probe_d2;
   int* ncand;
+  float cn_max, cd_max;  // the centroids' largest norm and rounding error
 };
 
 constexpr int kRWarps = 8, kRThreads = kRWarps * 32;
@@ -446,63 +447,6 @@ __device__ __forceinline__ float batch_d2_any(const float* __restrict__ C, const
   return acc;
 }
 
-// An upper bound, within 2^8 - 1 units of the last place, of the np-th
-// smallest of keys[0..n) (1 <= np <= n), all in [kmin, kmax] <= +inf: radix
-// levels of 8 bits over key - kmin, the first level's shift fitted to the
-// range, each level counting only the keys inside the bin chosen before, until
-// the bins are at most 2^8 keys wide; the top of the last bin chosen.
-__device__ uint32_t block_select(const uint32_t* keys, int64_t n, int np, uint32_t kmin, uint32_t kmax, int* hist,
-                                 uint32_t* sh) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int shift = 0;
-  while (((kmax - kmin) >> shift) > 255u) ++shift;
-  uint32_t lo = 0;                        // relative start of the current range
-  uint32_t span_m1 = kmax - kmin;         // its length - 1 (keys <= 0x7F800000: no overflow)
-  int need = np;
-  for (;;) {
-    for (int i = tid; i < 256; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
-    for (int64_t l = tid; l < n; l += blockDim.x) {
-      const uint32_t rel = keys[l] - kmin - lo;   // wraps below lo: outside the range
-      if (rel <= span_m1) atomicAdd(&hist[rel >> shift], 1);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      int c[8], run = 0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) { c[i] = hist[lane * 8 + i]; run += c[i]; }
-      int incl = run;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int excl = incl - run;
-      int pick = -1, below = 0;
-      if (excl < need && need <= incl) {
-        int acc = excl;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (pick < 0 && acc + c[i] >= need) { pick = lane * 8 + i; below = acc; }
-          acc += c[i];
-        }
-      }
-      const unsigned who = __ballot_sync(kFull, pick >= 0);
-      const int src = who ? __ffs(who) - 1 : 0;
-      pick = __shfl_sync(kFull, pick, src);
-      below = __shfl_sync(kFull, below, src);
-      if (lane == 0) { sh[0] = who ? (uint32_t)pick : 255u; sh[1] = who ? (uint32_t)below : 0u; }
-    }
-    __syncthreads();
-    lo += sh[0] << shift;
-    need -= (int)sh[1];
-    span_m1 = (1u << shift) - 1u;
-    if (shift <= 8) break;
-    shift = shift >= 16 ? shift - 8 : 8;
-  }
-  return min(kmin + lo + span_m1, 0x7F800000u);  // the last bin may reach past +inf's key
-}
-
 // Candidate lists of the split re-rank: up to kCap candidates per query in
 // the workspace, their distances computed by rerank_dist_kernel (one warp per
 // 32 candidates, over all queries at once) and merged by rerank_merge_kernel.
@@ -531,33 +475,59 @@ __device__ __forceinline__ void write_probes(const RerankArgs& a, int64_t q, int
   }
 }
 
-// One block per query, every list's upper key and lower bound held in shared
-// memory.
-// A: eps, the key of D~ + eps and the lower bound D~ - eps of every list, and
-//    the keys' range.
-// B: T >= the np-th smallest key, within 255 units of the last place
-//    (block_select).
-// C: the candidates, D~ - eps <= T, appended to a block-wide list.
+// X with D~ - eps > T for every list with D~ > X, given T0 = a bound of the
+// np-th smallest D~ and E(x) = the largest eps of any list at D~ = x
+// (rerank_bound grows with each of its distance and centroid arguments): the
+// np lists with D~ <= T0 have FP32-rule distances of at most T = T0 + E(T0),
+// so every list of the FP32 top-np has D~ - E(D~) <= T. x - E(x) is convex (E
+// is a square root plus a linear term), so it stays above T beyond a point
+// where it is above and rising. +inf (every list a candidate) where no such
+// point is found or a value is not finite.
+__device__ __forceinline__ float candidate_limit(const RerankArgs& a, float T0, float qn, float qd) {
+  auto E = [&](float x) { return rerank_bound(x, qn, qd, a.cn_max, a.cd_max, a.kef, a.kfp); };
+  const float T = __fadd_ru(T0, E(T0));
+  float x = __fadd_ru(T, E(T));
+  for (int i = 0; i < 12; ++i) {
+    x = __fadd_ru(T, 1.01f * E(x)) * 1.000001f;
+    const float y = 1.01f * x + 1e-30f;
+    if (x - E(x) > T * 1.0000002f && y - E(y) > x - E(x)) return x;
+  }
+  return INFINITY;
+}
+
+// One block per query, its row of D~ in registers (VPT values a thread; VPT =
+// 0: in shared memory).
+// A: T0 >= the np-th smallest D~ (negative values count as 0, NaN as +inf), from
+//    the np-th smallest of the threads' minima (one value a thread to bisect
+//    over instead of VPT; about 15 % more lists lie below it) and then among
+//    the values up to that, within 2^10 units of the last place; from T0 the
+//    limit X of the candidates' D~ (candidate_limit).
+// B: the candidates, D~ <= X, appended to a block-wide list.
+// 20000 queries, 8192 lists, nprobe 64: 462 us, bound by issue and barriers; 728
+// us when each list's own bound was formed (25 operations a list) for a radix
+// select over the upper bounds. The shared bound keeps a few more candidates.
 // Then, with at most kCap candidates, the list goes to the workspace with one
 // work item per 32 candidates; otherwise the block computes their FP32-rule
 // distances itself, 32 per warp batch (batches dealt round-robin to the
 // warps), each warp keeping its top-np by (D2, l), the warps' lists merged at
 // the end. Queries with np = 0 get their padding here.
-// Dynamic shared memory: qs [dim rounded up to 4] | keys [nlist rounded up to
-// 4] (then the candidate list) | lower [nlist], whose space then holds the
-// warps' staging tiles [8][1056].
-template <int R, bool V4>
+// Dynamic shared memory: qs [dim rounded up to 4] | candidate list [nlist
+// rounded up to 4] | the warps' staging tiles [8][1056]; VPT = 0: qs | D~, later
+// the tiles | candidate list.
+template <int R, bool V4, int VPT>
 __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs a, RerankSplit sp) {
-  __shared__ int hist[256];
   __shared__ uint32_t sh[2];
   __shared__ int total;
   __shared__ uint32_t kr[2][kRWarps];
+  constexpr int kNear = 512;
+  __shared__ uint32_t near_keys[kNear];
   const int dq = (a.dim + 3) & ~3;
   const int64_t nl4 = (a.nlist + 3) & ~3;
   float* qs = (float*)anns_dyn_smem;
-  uint32_t* keys = (uint32_t*)(qs + dq);
-  float* lower = (float*)(keys + nl4);
-  float* tiles = lower;
+  float* vals = qs + dq;
+  const int64_t tile_floats = (int64_t)kRWarps * kRTile, first = VPT > 0 || nl4 > tile_floats ? nl4 : tile_floats;
+  int32_t* cand = (int32_t*)(VPT > 0 ? vals : vals + first);
+  float* tiles = VPT > 0 ? vals + nl4 : vals;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t q = blockIdx.x, nlist = a.nlist;
   const int np = a.npq ? min(max(a.npq[q], 0), a.nprobe) : a.nprobe;
@@ -571,61 +541,94 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
   const float* row = a.dt + q * nlist;
   const float qn = a.qrows[q], qd = a.qrows[a.nq + q];
   if (threadIdx.x == 0) total = 0;
-  // A: eight lists per thread per round, all their loads issued before any
-  // use (D~ streams from HBM once)
-  uint32_t kmin = 0xFFFFFFFFu, kmax = 0;
-  for (int64_t b0 = threadIdx.x; b0 < nlist; b0 += 8 * kRThreads) {
-    float d[8], cn[8], cd[8];
+  float d[VPT ? VPT : 1];
+  const int nl = (int)nlist;
+  auto each = [&](auto f) {  // f(list, D~) over this thread's lists
+    if constexpr (VPT > 0) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t l = b0 + j * kRThreads;
-      const bool in = l < nlist;
-      d[j] = in ? row[l] : 0.f;
-      cn[j] = in ? a.crows[l] : 0.f;
-      cd[j] = in ? a.crows[nlist + l] : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int64_t l = b0 + j * kRThreads;
-      if (l < nlist) {
-        const float b = rerank_bound(d[j], qn, qd, cn[j], cd[j], a.kef, a.kfp);
-        const uint32_t k = upper_key(d[j] + b);
-        keys[l] = k;
-        lower[l] = d[j] - b;
-        kmin = min(kmin, k);
-        kmax = max(kmax, k);
+      for (int j = 0; j < VPT; ++j) {
+        const int l = threadIdx.x + j * kRThreads;
+        if (l < nl) f(l, d[j]);
       }
+    } else {
+      for (int l = threadIdx.x; l < nl; l += kRThreads) f(l, vals[l]);
     }
-  }
+  };
+  if constexpr (VPT > 0) {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    kmin = min(kmin, __shfl_xor_sync(kFull, kmin, o));
-    kmax = max(kmax, __shfl_xor_sync(kFull, kmax, o));
+    for (int j = 0; j < VPT; ++j) {
+      const int l = threadIdx.x + j * kRThreads;
+      d[j] = l < nl ? row[l] : INFINITY;
+    }
+  } else {
+    for (int l = threadIdx.x; l < nl; l += kRThreads) vals[l] = row[l];  // read back by this thread only
   }
-  if (lane == 0) { kr[0][warp] = kmin; kr[1][warp] = kmax; }
+  // the np-th smallest of the threads' minima: at least np lists lie at or
+  // below it, and few more (a thread without lists, or with none but NaN: +inf)
+  float least = INFINITY;
+  each([&](int, float v) { least = fminf(least, v); });
+  const uint32_t mine = upper_key(least);
+  uint32_t lo = __reduce_min_sync(kFull, mine), hi = 0x7F800000u;
+  if (lane == 0) kr[0][warp] = lo;
   __syncthreads();
-  kmin = 0xFFFFFFFFu;
-  kmax = 0;
-  for (int w = 0; w < kRWarps; ++w) {
-    kmin = min(kmin, kr[0][w]);
-    kmax = max(kmax, kr[1][w]);
+  for (int w = 0; w < kRWarps; ++w) lo = min(lo, kr[0][w]);
+  const uint32_t lowest = lo;
+  while (hi - lo > 4095u) {  // count(mine <= hi) >= np throughout, or hi = +inf
+    const uint32_t mid = lo + ((hi - lo) >> 1);
+    if (__syncthreads_count(mine <= mid) >= np) hi = mid;
+    else lo = mid + 1u;
   }
-  // B
-  const float T = __uint_as_float(block_select(keys, nlist, np, kmin, kmax, hist, sh));
-  __syncthreads();  // keys are free: they become the candidate list
-  // C
-  int32_t* cand = (int32_t*)keys;
-  for (int64_t b0 = (int64_t)warp * 32; b0 < nlist; b0 += kRThreads) {
-    const int64_t l = b0 + lane;
-    const bool c = l < nlist && !(lower[l] > T);
-    const unsigned m = __ballot_sync(kFull, c);
-    if (m) {
-      int at = 0;
-      if (lane == 0) at = atomicAdd(&total, __popc(m));
-      at = __shfl_sync(kFull, at, 0);
-      if (c) cand[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)l;
+  // the values up to it, and the np-th smallest of them
+  {
+    const float U = __uint_as_float(hi);
+    each([&](int, float v) {
+      if (v <= U) {
+        const int at = atomicAdd(&total, 1);
+        if (at < kNear) near_keys[at] = upper_key(v);
+      }
+    });
+  }
+  __syncthreads();
+  const int nn = total;
+  __syncthreads();
+  if (threadIdx.x == 0) total = 0;
+  if (nn <= kNear) {
+    if (warp == 0) {
+      uint32_t l2 = lowest, h2 = hi;
+      while (h2 - l2 > 1023u) {
+        const uint32_t mid = l2 + ((h2 - l2) >> 1);
+        int c = 0;
+        for (int i = lane; i < nn; i += 32) c += near_keys[i] <= mid ? 1 : 0;
+        if ((int)__reduce_add_sync(kFull, c) >= np) h2 = mid;
+        else l2 = mid + 1u;
+      }
+      if (lane == 0) sh[0] = h2;
+    }
+    __syncthreads();
+    hi = sh[0];
+  } else {  // many equal values, or fewer lists than threads: over all of them
+    lo = lowest;
+    hi = 0x7F800000u;
+    for (int step = 0; hi - lo > 1023u; ++step) {
+      const uint32_t mid = lo + ((hi - lo) >> 1);
+      const float midf = __uint_as_float(mid);
+      int c = 0;
+      each([&](int, float v) { c += v <= midf ? 1 : 0; });  // a NaN never counts
+      c = __reduce_add_sync(kFull, c);
+      if (lane == 0) kr[step & 1][warp] = (uint32_t)c;
+      __syncthreads();
+      int t = 0;
+      for (int w = 0; w < kRWarps; ++w) t += (int)kr[step & 1][w];
+      if (t >= np) hi = mid;
+      else lo = mid + 1u;
     }
   }
+  const float X = candidate_limit(a, __uint_as_float(hi), qn, qd);
+  __syncthreads();
+  // B
+  each([&](int l, float v) {
+    if (!(v > X)) cand[atomicAdd(&total, 1)] = l;
+  });
   __syncthreads();
   const int nc_all = total;
   if (threadIdx.x == 0 && a.ncand) a.ncand[q] = nc_all;
@@ -637,7 +640,7 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
     if (threadIdx.x < nb) sp.items[sh[0] + threadIdx.x] = make_int2((int)q, threadIdx.x);
     return;
   }
-  // D, in the block: the query itself and the staging tiles (over `lower`)
+  // C, in the block: the query itself and the staging tiles
   for (int d = threadIdx.x; d < dq; d += kRThreads) qs[d] = d < a.dim ? a.Q[q * a.dim + d] : 0.f;
   __syncthreads();
   float thd = INFINITY;
@@ -645,9 +648,9 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
   float* tile = tiles + warp * kRTile;
   for (int b0 = warp * 32; b0 < nc_all; b0 += kRWarps * 32) {
     const int nc = min(32, nc_all - b0);
-    const float d = V4 ? batch_d2_v4(a.C, qs, a.dim, cand + b0, nc, tile)
-                       : batch_d2_any(a.C, qs, a.dim, cand + b0, nc, tile);
-    top.offer(lane < nc, d, lane < nc ? cand[b0 + lane] : 0, np, thd, thi);
+    const float dc = V4 ? batch_d2_v4(a.C, qs, a.dim, cand + b0, nc, tile)
+                        : batch_d2_any(a.C, qs, a.dim, cand + b0, nc, tile);
+    top.offer(lane < nc, dc, lane < nc ? cand[b0 + lane] : 0, np, thd, thi);
   }
   __syncthreads();  // tiles are free: they hold the warps' lists
   float* md = tiles;
@@ -844,11 +847,13 @@ constexpr int kFmts[3] = {ANNS_PREC_BF16, ANNS_PREC_FP16, ANNS_PREC_FP8E4M3};
 int fmt_slot(int prec) { return prec == ANNS_PREC_BF16 ? 0 : prec == ANNS_PREC_FP16 ? 1 : 2; }
 int fmt_elem(int prec) { return prec == ANNS_PREC_FP8E4M3 ? 1 : 2; }
 
-// Dynamic shared memory of the select kernel for this index: qs | keys |
-// lower (or the tiles).
+// Dynamic shared memory of the select kernel for this index: qs | the
+// candidate list | tiles, and D~ where it does not fit in registers.
+constexpr int kRegLists = 32 * kRThreads;
 size_t rerank_smem(const Index& ix) {
   const size_t nl4 = (size_t)((ix.nlist + 3) & ~3);
-  return (size_t)((ix.dim + 3) & ~3) * 4 + nl4 * 4 + std::max(nl4 * 4, (size_t)kRWarps * kRTile * 4);
+  const size_t tiles = (size_t)kRWarps * kRTile * 4;
+  return (size_t)((ix.dim + 3) & ~3) * 4 + nl4 * 4 + (ix.nlist > kRegLists ? std::max(nl4 * 4, tiles) : tiles);
 }
 constexpr size_t kRerankSmemMax = 200 * 1024;  // beyond it: the streaming re-rank
 
@@ -873,6 +878,18 @@ cudaError_t center_any(int prec, const float* X, int64_t n, int dim, int Dp, con
 
 bool coarse_tc_format(int prec) {
   return prec == ANNS_PREC_BF16 || prec == ANNS_PREC_FP16 || prec == ANNS_PREC_FP8E4M3;
+}
+
+// The GEMM and the exact re-rank give the FP32 rule's probes and distances bit
+// for bit, so a large FP32 coarse stage takes them: its own kernel does three
+// FP32 operations a dimension on the CUDA cores. Below about 3e8 of them, or
+// with too few queries or lists for the GEMM's tiles, its two launches are
+// faster than the fast path's six. (10000 queries x 4096 lists x 96: 622 us on
+// the CUDA cores, 323 us so; 4096 x 1024 x 960: 581 and 265 us; 10000 x 1024 x
+// 128: 203 and 120 us.)
+bool coarse_fp32_by_tc(const Index& ix, int64_t nq) {
+  return nq >= 256 && ix.nlist >= 256 && rerank_smem(ix) <= kRerankSmemMax &&
+         (double)nq * (double)ix.nlist * (double)ix.dim >= 3e8;
 }
 
 int coarse_tc_dp(const Index& ix, int prec) {
@@ -900,7 +917,18 @@ int prepare_coarse_tc(Index& ix, const std::vector<float>& cent) {
   for (int f = 0; f < 3 && e == cudaSuccess; ++f)
     e = center_any(kFmts[f], ix.centroids, ix.nlist, (int)ix.dim, coarse_tc_dp(ix, kFmts[f]), ix.tc_mu, ix.tc_c[f],
                    ix.tc_crows[f], 0);
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  std::vector<float> rows(2 * (size_t)ix.nlist);
+  for (int f = 0; f < 3 && e == cudaSuccess; ++f) {  // the largest norm and rounding error (a NaN stays)
+    e = cudaMemcpy(rows.data(), ix.tc_crows[f], rows.size() * sizeof(float), cudaMemcpyDeviceToHost);
+    for (int i = 0; i < 2; ++i) {
+      float most = 0.f;
+      for (int64_t l = 0; l < ix.nlist; ++l) {
+        const float v = rows[i * ix.nlist + l];
+        if (v > most || v != v) most = v;
+      }
+      ix.tc_cmax[f][i] = most;
+    }
+  }
   return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "coarse fast-path setup");
 }
 
@@ -970,7 +998,7 @@ cudaError_t launch_coarse_tc(const Index& ix, int prec, const float* Q, int64_t 
   if (e != cudaSuccess) return e;
   RerankArgs a{Q, ix.centroids, dt, qrows, ix.tc_crows[f], nq, ix.nlist, (int)ix.dim,
                (float)((2.0 * Dp + 8.0) * 5.9604644775390625e-8 * 1.01), (float)((ix.dim + 2) * 5.9604644775390625e-8),
-               nprobe, nprobe_per_q, probes, probe_d2, ncand};
+               nprobe, nprobe_per_q, probes, probe_d2, ncand, ix.tc_cmax[f][0], ix.tc_cmax[f][1]};
   char* after = (char*)ws + tc_operand_bytes(ix, nq) + tc_small_bytes(nq);
   RerankSplit sp{(int32_t*)after, (float*)(after + (size_t)nq * kCap * 4), (int2*)(after + (size_t)nq * kCap * 8),
                  (int*)(ncand + nq)};
@@ -993,8 +1021,18 @@ cudaError_t launch_coarse_tc(const Index& ix, int prec, const float* Q, int64_t 
     if (smem > kRerankSmemMax) return run(rerank_stream_kernel<RR>, g, kRThreads, (size_t)ix.dim * 4, a);
     cudaError_t e2 = cudaMemsetAsync(sp.nitems, 0, sizeof(int), s);
     if (e2 == cudaSuccess)
-      e2 = v4 ? run(rerank_select_kernel<RR, true>, g, kRThreads, smem, a, sp)
-              : run(rerank_select_kernel<RR, false>, g, kRThreads, smem, a, sp);
+      e2 = [&] {
+        auto sel = [&](auto v_tag) {
+          constexpr int V = decltype(v_tag)::value;
+          return v4 ? run(rerank_select_kernel<RR, true, V>, g, kRThreads, smem, a, sp)
+                    : run(rerank_select_kernel<RR, false, V>, g, kRThreads, smem, a, sp);
+        };
+        const int64_t per = (ix.nlist + kRThreads - 1) / kRThreads;
+        return per <= 4    ? sel(std::integral_constant<int, 4>{})
+               : per <= 16 ? sel(std::integral_constant<int, 16>{})
+               : per <= 32 ? sel(std::integral_constant<int, 32>{})
+                           : sel(std::integral_constant<int, 0>{});
+      }();
     // the distance kernel's grid: every block resident at once (the warps
     // stride over the item list)
     auto dist = [&](auto kern) {

@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(256) decode_kernel(const uint8_t* __restrict__
 struct PlanArgs {
   int64_t nq, dim;
   int nprobe, k, M, dsub, Dp, take, nlist;
+  int v4;                  // 16-byte loads of Q and the centroids, dsub a multiple of 4
   const int32_t* npq; const int32_t* kpq;
   const int32_t* probes; const float* d2; const uint8_t* bits; const int32_t* list_len;
   const int64_t* tile_off;
@@ -211,9 +212,17 @@ __global__ void __launch_bounds__(128) plan_kernel(const PlanArgs a, const PassA
         const float* cv = a.C + (int64_t)l * a.dim;
         for (int m = lane; m < a.M; m += 32) {
           float s = 0.f;
-          for (int i = 0; i < a.dsub; ++i) {
-            const float e = qv[m * a.dsub + i] - cv[m * a.dsub + i];
-            s += e * e;
+          if (a.v4) {
+            for (int i = 0; i < a.dsub; i += 4) {
+              const float4 x = __ldg((const float4*)(qv + m * a.dsub + i)), c = __ldg((const float4*)(cv + m * a.dsub + i));
+              const float e0 = x.x - c.x, e1 = x.y - c.y, e2 = x.z - c.z, e3 = x.w - c.w;
+              s += e0 * e0 + e1 * e1 + (e2 * e2 + e3 * e3);
+            }
+          } else {
+            for (int i = 0; i < a.dsub; ++i) {
+              const float e = qv[m * a.dsub + i] - cv[m * a.dsub + i];
+              s += e * e;
+            }
           }
           const float v = sqrtf(s) * 1.0001f + a.ym[m];
           rmax = v > rmax || v != v ? v : rmax;  // a NaN stays
@@ -551,11 +560,14 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     // that reads a column again from TMEM (unrolled over the registers it is 32
     // copies of the push, and their instruction fetches cost ten times the work).
     auto push = [&](uint32_t mask, int j0, uint32_t tcol, const float2* kc, const int2* dc, float s, int pos) {
-      for (uint32_t cols = __reduce_or_sync(kFull, mask); cols; cols &= cols - 1u) {
+      uint32_t cols = __reduce_or_sync(kFull, mask);
+      const int dl = dc[j0 + (lane & 7)].x;  // lane j < 8: column j's pair
+      const bool hit = lane < 8 && (cols >> lane & 1u);
+      if (hit) a.alive[dl & 0x7FFFFFFF] = 1;
+      cols = __ballot_sync(kFull, hit && dl >= 0);  // the others are only marked
+      for (; cols; cols &= cols - 1u) {
         const int j = __ffs(cols) - 1;
         const int d = dc[j0 + j].x;
-        if (lane == 0) a.alive[d & 0x7FFFFFFF] = 1;
-        if (d < 0) continue;
         const unsigned who = __ballot_sync(kFull, mask >> j & 1u);
         const float t = fmaf(tc_ld1(tcol + j0 + j), kc[j0 + j].y, s);
         if (staged > kPush - 32) flush();
@@ -1664,21 +1676,26 @@ void free_filter(Index& ix) {
 }
 
 bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
-                      bool grouped_otherwise) {
+                      bool grouped_otherwise, bool uneven) {
   if (ix.fl_w == 0 || (ix.opt_kernel != ANNS_KERNEL_AUTO && ix.opt_kernel != ANNS_KERNEL_SPLIT)) return false;
   if (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits < 5) return false;  // every pair would be scanned anyway
   const int64_t pairs = nq * nprobe;
   // Small searches are over before the filter's fifteen launches (100 us; 250 us
   // with the grouped kernels behind them) are. Query-major, a block scans a pair
-  // in about Mp (256 + list) / 2000 us, some 400 queries at a time (one query, 8
-  // lists of 312, M = 16: 54 us scanned, 87 us filtered; 777 queries, 19 lists
-  // of 150, M = 20, 12 bits: 530 and 200 us). The grouped kernels spread a small
-  // batch over the GPU and take about 4.6e9 look-ups a millisecond (77 queries,
-  // 64 lists of 1094, M = 48: 304 us grouped, 364 us filtered).
-  const double lookups = (double)pairs * (double)ix.Mp * ((double)ix.n / (double)ix.nlist + 512.0);
-  const double scan_us = (double)nprobe * (double)ix.Mp * (256.0 + (double)ix.n / (double)ix.nlist) / 2000.0 *
-                         std::max(1.0, (double)nq / 400.0);
-  if (grouped_otherwise ? lookups < 2e9 : scan_us < 100.0) return false;
+  // in about Mp (256 + list) / 2000 us, some 400 blocks at a time (777 queries,
+  // 19 lists of 150, M = 20, 12 bits: 530 us scanned, 200 us filtered), and
+  // lists of k > 32 entries add some 8 us a pair and 60 us for their merge (3
+  // queries, 27 lists of 692, M = 24, k = 128: 413 and 199 us). The grouped
+  // kernels take about 4.6e9 look-ups a millisecond (77 queries, 64 lists of
+  // 1094, M = 48: 304 us grouped, 364 us filtered), ten times less with k > 32
+  // (39 queries, 11 lists of 608, M = 64, k = 128: 1345 us).
+  const double probes = uneven ? nprobe / 6.0 : nprobe;  // their number per query is on the device
+  const int split = ix.opt_kernel == ANNS_KERNEL_AUTO ? search_split(nq, nprobe, k) : 1;
+  const double scan_us = std::max(1.0, probes / split) * (double)ix.Mp *
+                         (256.0 + (double)ix.n / (double)ix.nlist) / 2000.0 * std::max(1.0, (double)nq * split / 400.0) +
+                         (k > 32 ? 60.0 + 8.0 * probes : 0.0);
+  const double lookups = probes * (double)nq * (double)ix.Mp * ((double)ix.n / (double)ix.nlist + 512.0);
+  if (grouped_otherwise ? lookups < (k > 32 ? 2e7 : 2e9) : scan_us < 100.0) return false;
   const int64_t tiles = (ix.max_list + kTv - 1) / kTv;
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))
@@ -1706,7 +1723,7 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   const int Dp = coarse_tc_dp(ix, ANNS_PREC_FP16);
   PlanArgs p{};
   p.nq = nq; p.dim = ix.dim; p.nprobe = nprobe; p.k = k; p.M = (int)ix.M; p.dsub = (int)ix.dsub; p.Dp = Dp;
-  p.take = filter_take(ix, k); p.nlist = (int)ix.nlist; p.npq = nprobe_per_q; p.kpq = k_per_q; p.probes = probes;
+  p.v4 = ix.dsub % 4 == 0 && ((uintptr_t)Q & 15u) == 0; p.take = filter_take(ix, k); p.nlist = (int)ix.nlist; p.npq = nprobe_per_q; p.kpq = k_per_q; p.probes = probes;
   p.d2 = probe_d2; p.bits = bits; p.list_len = ix.list_len; p.tile_off = ix.tile_off; p.Q = Q; p.C = ix.centroids;
   p.ym = ix.fl_ym; p.stat = (const float4*)ix.fl_stat; p.qrows = q16_rows; p.mu_norm = ix.fl_mu;
   p.yscale = ix.fl_yscale; p.eps = w.eps; p.eps0 = w.eps0; p.sel = w.sel; p.in2 = w.in2; p.ntake = w.ntake;

@@ -53,6 +53,7 @@ struct Index {
   float* tc_mu = nullptr;
   void* tc_c[3] = {};
   float* tc_crows[3] = {};
+  float tc_cmax[3][2] = {};     // the largest of each row (cn, cd) of tc_crows
   int* dev_status = nullptr;
   // tensor-core filter (filter.cu): decoded residuals in FP16 [ntiles*32][fl_w]
   // (fl_w = 0: not available), s_x [ntiles*32], per list (largest |y|, largest
@@ -144,6 +145,9 @@ cudaError_t launch_coarse(const Index& ix, const float* Q, int64_t nq, int nprob
 // CL fast path: tensor-core distances with BF16, FP16 or FP8 E4M3 operands
 // (ANNS_PREC_*), then the exact re-rank (coarse_tc.cu).
 bool coarse_tc_format(int prec);
+// Whether a coarse stage asked for by the FP32 rule goes through the FP16 fast
+// path (same output).
+bool coarse_fp32_by_tc(const Index& ix, int64_t nq);
 int coarse_tc_dp(const Index& ix, int prec);
 int prepare_coarse_tc(Index& ix, const std::vector<float>& cent);
 size_t coarse_tc_workspace_bytes(const Index& ix, int64_t nq);
@@ -168,7 +172,8 @@ int launch_policy(const Index& ix, const anns_precision_policy& pol, int64_t nq,
 // table: fewer bytes of shared memory per block, more blocks per SM).
 enum { QM_TABLES_ALL = 0, QM_TABLES_FP32 = 1, QM_TABLES_NARROW = 2 };
 // RC + LC + quantise + DC + TS for every query; `order` (NULL = 0..nq-1) is
-// the order in which blocks take the queries; with `count` (device) only its
+// the order in which blocks take the queries; split > 1: that many blocks a
+// query, row q * split + i of the results for its part i; with `count` (device) only its
 // first *count entries run. skip_narrow 1 leaves out the 1..8-bit pairs of
 // probe rank >= 1, 2 those of every rank, 3 the 1..4-bit pairs of every rank. With
 // QM_TABLES_NARROW only the 1..8-bit pairs are scanned, and part_d / part_i
@@ -179,7 +184,13 @@ cudaError_t launch_search(const Index& ix, const float* qt, int64_t nq, int npro
                           const int32_t* probes, const float* probe_d2, const uint8_t* bits,
                           const int32_t* order, int64_t* ids_out, float* dists_out, cudaStream_t s,
                           int skip_narrow = 0, int tables = QM_TABLES_ALL, const float* part_d = nullptr,
-                          const int64_t* part_i = nullptr, const int* count = nullptr);
+                          const int64_t* part_i = nullptr, const int* count = nullptr, int split = 1);
+// Blocks per query of a batch too small to fill the GPU with one each (a query
+// alone scans its probes one after the other: 8 lists of 312, M = 16, 37 us;
+// k <= 32), and the merge of their partial results, rows q * split + i.
+int search_split(int64_t nq, int nprobe, int k);
+cudaError_t launch_merge_split(const float* part_d, const int64_t* part_i, int split, const int32_t* k_per_q, int64_t nq,
+                               int k, int64_t* ids_out, float* dists_out, cudaStream_t s);
 // Longest-first query order (schedule.cu) into a workspace of
 // lpt_workspace_bytes(nq); the order is at lpt_order_ptr(ws, nq).
 size_t lpt_workspace_bytes(int64_t nq);
@@ -269,7 +280,7 @@ int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<
 void free_filter(Index& ix);
 // Whether the filter serves the call; grouped_otherwise: the grouped kernels would.
 bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
-                      bool grouped_otherwise);
+                      bool grouped_otherwise, bool uneven);
 size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k);
 // What the filter leaves: queries for the scanning kernel (their number on the
 // device) and the pairs on tables of at most 4 bits that are worth a scan.

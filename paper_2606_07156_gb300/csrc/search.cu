@@ -429,6 +429,7 @@ struct SearchArgs {
   // kernels take them); 2: of every rank (the narrow pass takes them); 3: the
   // pairs on 1..4-bit tables (the grouped kernels take the ones worth a scan)
   int skip_narrow;
+  int split;  // blocks per query: block i of a query takes every split-th of its pairs, result row q * split + i
   int ids32;  // every id fits in int32 (the 128-entry lists then hold 32-bit ids)
   int64_t* ids_out; float* dists_out;
   // kModeNarrow: the query's top-k over its other pairs ([nq * k], padding
@@ -437,11 +438,11 @@ struct SearchArgs {
   SmemLayout lay;
 };
 
-// End of a query: the warps' lists are merged into warp 0, which writes the
-// query's k results (padding id -1, distance +inf). Ends with a barrier.
+// End of a query: the warps' lists are merged into warp 0, which writes row
+// `out` of the results, k of them (padding id -1, distance +inf). Ends with a barrier.
 template <int R, typename IdT>
 __device__ __forceinline__ void merge_and_write(const SearchArgs& a, Smem& s, WarpTopK<R, IdT>& top,
-                                                int64_t q, int kq, float& thd, IdT& thi) {
+                                                int64_t q, int64_t out, int kq, float& thd, IdT& thi) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (a.part_d && kq > 0) {
     // the top-k of the query's other pairs joins warp 0's list
@@ -472,8 +473,8 @@ __device__ __forceinline__ void merge_and_write(const SearchArgs& a, Smem& s, Wa
       const int e = r * 32 + lane;
       if (e < a.k) {
         const bool ok = e < kq && top.d[r] != INFINITY;
-        a.ids_out[q * a.k + e] = ok ? (int64_t)top.id[r] : -1;
-        a.dists_out[q * a.k + e] = ok ? top.d[r] : INFINITY;
+        a.ids_out[out * a.k + e] = ok ? (int64_t)top.id[r] : -1;
+        a.dists_out[out * a.k + e] = ok ? top.d[r] : INFINITY;
       }
     }
   }
@@ -503,7 +504,9 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tstride = (int64_t)a.Mp * kKsub;
   const int64_t nq = a.count ? *a.count : a.nq;
-  for (int64_t qi = blockIdx.x; qi < nq; qi += gridDim.x) {
+  for (int64_t bi = blockIdx.x; bi < nq * a.split; bi += gridDim.x) {
+    const int64_t qi = a.split > 1 ? bi / a.split : bi;
+    const int part = a.split > 1 ? (int)(bi - qi * a.split) : 0;
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
     const int np = a.npq ? min(max(a.npq[q], 0), a.nprobe) : a.nprobe;
     const int kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
@@ -539,10 +542,12 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
                                               : !(narrow && (a.skip_narrow == 2 || (a.skip_narrow == 1 && j >= 1) ||
                                                              (a.skip_narrow == 3 && b <= 4))));
         const unsigned m = __ballot_sync(kFull, use);
-        if (use) s.plist[base + __popc(m & ((1u << lane) - 1u))] = make_int4(l, n_l, b, __float_as_int(d2));
+        const int at = base + __popc(m & ((1u << lane) - 1u));
+        if (use && (a.split == 1 || at % a.split == part))
+          s.plist[a.split == 1 ? at : at / a.split] = make_int4(l, n_l, b, __float_as_int(d2));
         base += __popc(m);
       }
-      if (lane == 0) *s.npairs = base;
+      if (lane == 0) *s.npairs = a.split == 1 ? base : (base - part + a.split - 1) / a.split;
     }
     __syncthreads();
     const int npairs = *s.npairs;
@@ -623,7 +628,48 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
         __syncthreads();  // the next pair overwrites the LUT
       }
     }
-    merge_and_write<R, IdT>(a, s, top, q, kq, thd, thi);
+    merge_and_write<R, IdT>(a, s, top, q, a.split > 1 ? bi : q, kq, thd, thi);
+  }
+}
+
+// The k <= 32 smallest (d, id) of a query's `split` partial results, one block
+// per query: each candidate's rank among all of them (at most 32 x 32; offered
+// one by one to a warp's sorted list, 320 candidates took 19 us).
+constexpr int kSplitMax = 32;
+__global__ void __launch_bounds__(256) merge_split_kernel(const float* __restrict__ part_d,
+                                                          const int64_t* __restrict__ part_i, int split,
+                                                          const int32_t* __restrict__ kpq, int k,
+                                                          int64_t* __restrict__ ids_out, float* __restrict__ dists_out) {
+  __shared__ float cd[kSplitMax * 32];
+  __shared__ int64_t ci[kSplitMax * 32];
+  __shared__ int total;
+  const int64_t q = blockIdx.x;
+  const int kq = kpq ? min(max(kpq[q], 0), k) : k;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < split * k; e += blockDim.x) {
+    const float d = part_d[q * split * k + e];
+    if (e % k < kq && d < INFINITY) {
+      const int at = atomicAdd(&total, 1);
+      cd[at] = d;
+      ci[at] = part_i[q * split * k + e];
+    }
+  }
+  __syncthreads();
+  const int n = total;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const float d = cd[i];
+    const int64_t id = ci[i];
+    int rank = 0;
+    for (int e = 0; e < n; ++e) rank += key_less(cd[e], ci[e], d, id) || (cd[e] == d && ci[e] == id && e < i) ? 1 : 0;
+    if (rank < kq) {
+      ids_out[q * k + rank] = id;
+      dists_out[q * k + rank] = d;
+    }
+  }
+  for (int e = min(n, kq) + (int)threadIdx.x; e < k; e += blockDim.x) {
+    ids_out[q * k + e] = -1;
+    dists_out[q * k + e] = INFINITY;
   }
 }
 
@@ -711,6 +757,7 @@ SearchArgs make_args(const Index& ix, const float* Q, const float* qt, int R, in
   a.list_len = ix.list_len; a.vec_off = ix.vec_off; a.tile_off = ix.tile_off;
   a.M = (int)ix.M; a.Mp = (int)ix.Mp;
   a.lay = SmemLayout(ix.Mp, R, mode);
+  a.split = 1;
   return a;
 }
 
@@ -727,7 +774,7 @@ template <typename K>
 cudaError_t launch_query_major(K kern, const SearchArgs& a, cudaStream_t s) {
   cudaError_t e = prep(kern, a.lay.total);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::min<int64_t>(a.nq, a.count ? 1024 : 1 << 30);
+  const unsigned grid = (unsigned)std::min<int64_t>(a.nq * a.split, a.count ? 1024 : 1 << 30);
   kern<<<grid, kThreads, a.lay.total, s>>>(a); note_launch();
   return cudaGetLastError();
 }
@@ -772,13 +819,15 @@ cudaError_t launch_search(const Index& ix, const float* qt, int64_t nq, int npro
                           const int32_t* nprobe_per_q, int k, const int32_t* k_per_q,
                           const int32_t* probes, const float* probe_d2, const uint8_t* bits,
                           const int32_t* order, int64_t* ids_out, float* dists_out, cudaStream_t s,
-                          int skip_narrow, int tables, const float* part_d, const int64_t* part_i, const int* count) {
+                          int skip_narrow, int tables, const float* part_d, const int64_t* part_i, const int* count,
+                          int split) {
   const int R = k <= 32 ? 1 : 4;
   const int mode = tables == QM_TABLES_FP32 ? kModeFp32 : tables == QM_TABLES_NARROW ? kModeNarrow : kModeFull;
   SearchArgs a = make_args(ix, nullptr, qt, R, mode);
   a.nq = nq; a.nprobe = nprobe; a.k = k; a.npq = nprobe_per_q; a.kpq = k_per_q;
   a.probes = probes; a.probe_d2 = probe_d2; a.bits = bits; a.order = order; a.count = count;
   a.skip_narrow = skip_narrow;
+  a.split = split;
   a.ids32 = ix.ids32 ? 1 : 0;
   a.ids_out = ids_out; a.dists_out = dists_out;
   a.part_d = mode == kModeNarrow ? part_d : nullptr;
@@ -793,6 +842,19 @@ cudaError_t launch_search(const Index& ix, const float* qt, int64_t nq, int npro
     case 7: return run_search_r<7>(a, R, mode, s);
     default: return run_search_r<8>(a, R, mode, s);
   }
+}
+
+int search_split(int64_t nq, int nprobe, int k) {
+  if (k > 32) return 1;  // the parts' lists and their merge would cost what the split saves
+  const int64_t per = std::min<int64_t>(std::min<int64_t>(kSplitMax, nprobe), 608 / std::max<int64_t>(nq, 1));
+  return per >= 2 ? (int)per : 1;
+}
+
+cudaError_t launch_merge_split(const float* part_d, const int64_t* part_i, int split, const int32_t* k_per_q, int64_t nq,
+                               int k, int64_t* ids_out, float* dists_out, cudaStream_t s) {
+  merge_split_kernel<<<(unsigned)nq, 256, 0, s>>>(part_d, part_i, split, k_per_q, k, ids_out, dists_out);
+  note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t launch_compute_luts(const Index& ix, const float* Q, const float* qt, int64_t nq,

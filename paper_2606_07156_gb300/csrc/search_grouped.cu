@@ -747,18 +747,26 @@ __global__ void __launch_bounds__(256) merge_grouped_kernel(
       const int64_t id = in ? qm_i[q * k + e] : -1;
       top.offer(in && id >= 0, d, id, kq, thd, thi);
     }
-  for (int j = 0; kq > 0 && j < np; ++j) {
-    const int64_t pid = q * nprobe + j;
-    const int b = bits[pid];
-    if (j < jmin || probes[pid] < 0 || b < 1 || b > 8) continue;
-    if (alive && !(alive[pid] && (b <= 4 || over[q]))) continue;
+  for (int j0 = 0; kq > 0 && j0 < np; j0 += 32) {
+    // the pairs with a partial result, 32 probe ranks at a time (one by one,
+    // their loads are a dependent chain per rank)
+    bool use = false;
+    if (j0 + lane < np) {
+      const int64_t pid = q * nprobe + j0 + lane;
+      const int b = bits[pid];
+      use = j0 + lane >= jmin && probes[pid] >= 0 && b >= 1 && b <= 8 &&
+            (!alive || (alive[pid] && (b <= 4 || over[q])));
+    }
+    for (unsigned left = __ballot_sync(kFull, use); left; left &= left - 1u) {
+      const int64_t pid = q * nprobe + j0 + __ffs(left) - 1;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int e = r * 32 + lane;
-      const bool in = e < kq;
-      const float d = in ? part_d[pid * k + e] : INFINITY;
-      const int64_t id = in ? part_i[pid * k + e] : -1;
-      top.offer(in && id >= 0, d, id, kq, thd, thi);
+      for (int r = 0; r < R; ++r) {
+        const int e = r * 32 + lane;
+        const bool in = e < kq;
+        const float d = in ? part_d[pid * k + e] : INFINITY;
+        const int64_t id = in ? part_i[pid * k + e] : -1;
+        top.offer(in && id >= 0, d, id, kq, thd, thi);
+      }
     }
   }
 #pragma unroll

@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) query_table_kernel(const float* __restric
     const float* qv = Q + q * dim;
     float* out = qt + q * (int64_t)Mp * kKsub;
     if constexpr (DS > 0) {
-      for (int m0 = 0; m0 < Mp; m0 += 4) {
+      for (int m0 = blockIdx.y * 4; m0 < Mp; m0 += 4 * gridDim.y) {
         float y[4][DS], x[4][DS];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) query_table_kernel(const float* __restric
         }
       }
     } else {
-      for (int m = 0; m < Mp; ++m) {
+      for (int m = blockIdx.y; m < Mp; m += gridDim.y) {
         float acc = 0.f;
         if (m < M) {
           const float* x = qv + m * dsub;
@@ -85,7 +85,8 @@ cudaError_t launch_query_tables(const Index& ix, const float* Q, int64_t nq, flo
   static_assert(kKsub == 256, "one thread per codebook entry");
   // the queries of a list (its length on the device): usually none or few
   const int64_t grid = std::min<int64_t>(nq, list ? 1024 : (int64_t)1 << 30);
-  const unsigned g = (unsigned)grid;
+  // few queries: their rows spread over more blocks (one query, Mp = 16: 6 us in one block)
+  const dim3 g((unsigned)grid, grid <= 64 && !list ? (unsigned)((ix.Mp + 3) / 4) : 1u);
   const int dim = (int)ix.dim, M = (int)ix.M, Mp = (int)ix.Mp, ds = (int)ix.dsub;
   switch (ds) {
     case 2: query_table_kernel<2><<<g, 256, 0, s>>>(Q, ix.codebooks, nq, dim, M, Mp, ds, qt, list, count); break;
