@@ -5,9 +5,9 @@
 #include <cmath>
 #include <cstring>
 #include <string>
-#include <thread>
 #include <vector>
 
+#include "common.cuh"
 #include "internal.h"
 
 namespace anns {
@@ -64,9 +64,8 @@ static void free_index(anns_index* ix) {
 
 }  // namespace anns
 
-using namespace anns;
-
-namespace {
+namespace anns {
+namespace index_build {
 
 template <typename T>
 int fetch(const T* src, size_t count, bool on_device, std::vector<T>& dst, const char* what) {
@@ -93,42 +92,116 @@ int upload(T** dst, const T* src, size_t count, const char* what) {
   return ANNS_OK;
 }
 
+// A device buffer of one call.
+struct Temp {
+  void* p = nullptr;
+  ~Temp() { if (p) cudaFree(p); }
+};
+
 // P_l[m][c] = fl32(yn[m][c] + fl32(2 * <c_lm, y_mc>)) with both inner products
-// accumulated in FP32, j ascending, one rounding per operation; rows M..Mp-1 zero.
-void list_tables(const std::vector<float>& cent, const std::vector<float>& books, int64_t nlist,
-                 int64_t dim, int64_t M, int64_t Mp, std::vector<float>& out) {
-  const int64_t dsub = dim / M;
-  std::vector<float> yn((size_t)M * ANNS_KSUB);
-  for (int64_t e = 0; e < M * ANNS_KSUB; ++e) {
-    float acc = 0.f;
-    for (int64_t j = 0; j < dsub; ++j) {
-      const float y = books[(size_t)e * dsub + j];
-      const float sq = y * y;
-      acc = acc + sq;
+// accumulated in FP32, j ascending, one rounding per operation; rows M..Mp-1
+// zero. Block = list, thread = entry c of every row.
+__global__ void __launch_bounds__(256) list_tables_kernel(const float* __restrict__ cent, const float* __restrict__ books,
+                                                          int64_t dim, int M, int Mp, int dsub, float* __restrict__ out) {
+  const int64_t l = blockIdx.x;
+  const int c = threadIdx.x;
+  const float* cl = cent + l * dim;
+  for (int m = 0; m < Mp; ++m) {
+    float v = 0.f;
+    if (m < M) {
+      const float* y = books + ((size_t)m * ANNS_KSUB + c) * dsub;
+      float yn = 0.f, acc = 0.f;
+      for (int j = 0; j < dsub; ++j) {
+        yn = add_rn(yn, mul_rn(y[j], y[j]));
+        acc = add_rn(acc, mul_rn(cl[m * dsub + j], y[j]));
+      }
+      v = add_rn(yn, mul_rn(2.f, acc));
     }
-    yn[e] = acc;
+    out[((size_t)l * Mp + m) * ANNS_KSUB + c] = v;
   }
-  out.assign((size_t)nlist * Mp * ANNS_KSUB, 0.f);
-  auto work = [&](int64_t l0, int64_t l1) {
-    for (int64_t l = l0; l < l1; ++l)
-      for (int64_t m = 0; m < M; ++m)
-        for (int c = 0; c < ANNS_KSUB; ++c) {
-          float acc = 0.f;
-          for (int64_t j = 0; j < dsub; ++j) {
-            const float pr = cent[(size_t)l * dim + m * dsub + j] * books[((size_t)m * ANNS_KSUB + c) * dsub + j];
-            acc = acc + pr;
-          }
-          const float two = 2.f * acc;
-          out[((size_t)l * Mp + m) * ANNS_KSUB + c] = yn[(size_t)m * ANNS_KSUB + c] + two;
-        }
-  };
-  const int64_t nt = std::max<int64_t>(1, std::min<int64_t>(std::thread::hardware_concurrency(), nlist));
-  std::vector<std::thread> th;
-  for (int64_t t = 0; t < nt; ++t) th.emplace_back(work, nlist * t / nt, nlist * (t + 1) / nt);
-  for (auto& x : th) x.join();
 }
 
-}  // namespace
+// Vector i's codes to its place slot[i] = tile * 32 + lane in the
+// warp-interleaved tiles, a thread per 16-byte chunk.
+__global__ void pack_codes_kernel(const uint8_t* __restrict__ codes, const int64_t* __restrict__ slot, int64_t n, int M,
+                                  int nchunk, uint8_t* __restrict__ packed) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n * nchunk) return;
+  const int64_t i = t / nchunk;
+  const int c = (int)(t - i * nchunk);
+  const uint8_t* src = codes + i * M + c * kChunkBytes;
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int b = 0; b < kChunkBytes; ++b)
+    if (c * kChunkBytes + b < M) w[b >> 2] |= (uint32_t)src[b] << (8 * (b & 3));
+  const int64_t s = slot[i];
+  *(uint4*)(packed + ((s / kTileVecs) * nchunk + c) * kTileChunkBytes + (s % kTileVecs) * kChunkBytes) =
+      make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Per list the largest squared residual norm: per member the FP64 sum of its
+// entries' squared norms, m ascending. Non-negative doubles order like their
+// bit patterns; a NaN never counts.
+__global__ void radius_kernel(const uint8_t* __restrict__ codes, const int32_t* __restrict__ list_of, int64_t n, int M,
+                              const double* __restrict__ yn2, unsigned long long* __restrict__ rmax2) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double s = 0.0;
+  for (int m = 0; m < M; ++m) s = __dadd_rn(s, yn2[m * ANNS_KSUB + codes[i * M + m]]);
+  if (s == s) atomicMax(rmax2 + list_of[i], (unsigned long long)__double_as_longlong(s));
+}
+
+// The parts of the index that the GPU forms: code tiles, list tables and
+// covering radii (on one host thread the tiles and radii took about 2 ns a code
+// byte, the tables a few ns an entry). The codes are read where they are, or
+// from a copy on the device.
+int pack_index(Index& ix, const anns_build_desc* d, const std::vector<int64_t>& slot, const std::vector<int32_t>& list_of,
+               const std::vector<double>& yn2) {
+  const int64_t n = ix.n;
+  const size_t code_bytes = std::max<size_t>((size_t)ix.ntiles * ix.nchunk * kTileChunkBytes, 16);
+  Temp codes, slots, lists, norms, rmax;
+  cudaError_t e = cudaMalloc((void**)&ix.codes, code_bytes);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&ix.ltab, (size_t)ix.nlist * ix.Mp * kKsub * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&slots.p, std::max<size_t>(n * 8, 16));
+  if (e == cudaSuccess) e = cudaMalloc(&lists.p, std::max<size_t>(n * 4, 16));
+  if (e == cudaSuccess) e = cudaMalloc(&norms.p, yn2.size() * 8);
+  if (e == cudaSuccess) e = cudaMalloc(&rmax.p, (size_t)ix.nlist * 8);
+  const uint8_t* src = d->codes;
+  if (e == cudaSuccess && !d->on_device && n > 0) {
+    e = cudaMalloc(&codes.p, (size_t)n * ix.M);
+    if (e == cudaSuccess) e = cudaMemcpy(codes.p, d->codes, (size_t)n * ix.M, cudaMemcpyHostToDevice);
+    src = (const uint8_t*)codes.p;
+  }
+  if (e == cudaSuccess) e = cudaMemset(ix.codes, 0, code_bytes);
+  if (e == cudaSuccess) e = cudaMemset(rmax.p, 0, (size_t)ix.nlist * 8);
+  if (e == cudaSuccess) e = cudaMemcpy(norms.p, yn2.data(), yn2.size() * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && n > 0) e = cudaMemcpy(slots.p, slot.data(), n * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && n > 0) e = cudaMemcpy(lists.p, list_of.data(), n * 4, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return cuda_fail(e, "index arrays");
+  if (n > 0) {
+    pack_codes_kernel<<<(unsigned)((n * ix.nchunk + 255) / 256), 256>>>(src, (const int64_t*)slots.p, n, (int)ix.M,
+                                                                        (int)ix.nchunk, ix.codes);
+    note_launch();
+    radius_kernel<<<(unsigned)((n + 255) / 256), 256>>>(src, (const int32_t*)lists.p, n, (int)ix.M,
+                                                        (const double*)norms.p, (unsigned long long*)rmax.p);
+    note_launch();
+  }
+  list_tables_kernel<<<(unsigned)ix.nlist, 256>>>(ix.centroids, ix.codebooks, ix.dim, (int)ix.M, (int)ix.Mp, (int)ix.dsub,
+                                                  ix.ltab);
+  note_launch();
+  e = cudaGetLastError();
+  std::vector<double> r2(ix.nlist);
+  if (e == cudaSuccess) e = cudaMemcpy(r2.data(), rmax.p, (size_t)ix.nlist * 8, cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "index kernels");
+  for (int64_t l = 0; l < ix.nlist; ++l) ix.h_radius[l] = (float)std::sqrt(r2[l]);
+  return ANNS_OK;
+}
+
+}  // namespace index_build
+}  // namespace anns
+
+using namespace anns;
+using namespace anns::index_build;
 
 extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index** out) {
   set_error("");
@@ -155,13 +228,11 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
   const int64_t Mp = (M + 15) / 16 * 16, nchunk = Mp / 16;
   const bool dev = d->on_device != 0;
   std::vector<float> cent, books;
-  std::vector<uint8_t> codes;
   std::vector<int32_t> list_of;
   std::vector<int64_t> uids;
   int rc;
   if ((rc = fetch(d->centroids, (size_t)(nlist * dim), dev, cent, "copy centroids")) ||
       (rc = fetch(d->codebooks, (size_t)(M * ANNS_KSUB * dsub), dev, books, "copy codebooks")) ||
-      (rc = fetch(d->codes, (size_t)(n * M), dev, codes, "copy codes")) ||
       (rc = fetch(d->list_of, (size_t)n, dev, list_of, "copy list_of"))) {
     cudaSetDevice(prev);
     return rc;
@@ -187,10 +258,19 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
     max_list = std::max(max_list, cnt[l]);
   }
   const int64_t ntiles = toff[nlist];
-  std::vector<uint8_t> packed((size_t)ntiles * nchunk * kTileChunkBytes, 0);
+  // places in the tiles and ids in list order, members in array order
   std::vector<int64_t> pids(n);
-  std::vector<int64_t> fill(nlist, 0);
-  // ||y_{m,c}||^2 in FP64 with j ascending; per member the sum over m ascending.
+  std::vector<int64_t> slot(n);
+  {
+    std::vector<int64_t> fill(nlist, 0);
+    for (int64_t i = 0; i < n; ++i) {
+      const int32_t l = list_of[i];
+      const int64_t rank = fill[l]++;
+      slot[i] = toff[l] * kTileVecs + rank;
+      pids[voff[l] + rank] = d->ids ? uids[i] : i;
+    }
+  }
+  // ||y_{m,c}||^2 in FP64 with j ascending
   std::vector<double> yn2((size_t)M * ANNS_KSUB, 0.0);
   for (int64_t m = 0; m < M; ++m)
     for (int c = 0; c < ANNS_KSUB; ++c) {
@@ -202,21 +282,6 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
       }
       yn2[(size_t)m * ANNS_KSUB + c] = acc;
     }
-  std::vector<double> rmax2(nlist, 0.0);
-  for (int64_t i = 0; i < n; ++i) {
-    const int32_t l = list_of[i];
-    const int64_t rank = fill[l]++;
-    const int64_t tile = toff[l] + rank / kTileVecs;
-    const int lane = (int)(rank % kTileVecs);
-    const uint8_t* src = &codes[(size_t)i * M];
-    double rn2 = 0.0;
-    for (int64_t m = 0; m < M; ++m) {
-      packed[((size_t)tile * nchunk + m / 16) * kTileChunkBytes + lane * kChunkBytes + m % 16] = src[m];
-      rn2 = rn2 + yn2[(size_t)m * ANNS_KSUB + src[m]];
-    }
-    rmax2[l] = std::max(rmax2[l], rn2);
-    pids[voff[l] + rank] = d->ids ? uids[i] : i;
-  }
   anns_index* ix = new anns_index();
   ix->device = d->device;
   ix->n = n; ix->dim = dim; ix->nlist = nlist; ix->M = M; ix->dsub = dsub; ix->Mp = Mp;
@@ -229,18 +294,14 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
   for (int64_t l = 0; l < nlist; ++l) {
     ix->h_list_len64[l] = cnt[l];
     len32[l] = (int32_t)cnt[l];
-    ix->h_radius[l] = (float)std::sqrt(rmax2[l]);
   }
-  std::vector<float> ltab;
-  list_tables(cent, books, nlist, dim, M, Mp, ltab);
   std::vector<int32_t> order(nlist);
   for (int64_t l = 0; l < nlist; ++l) order[l] = (int32_t)l;
   std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return cnt[x] > cnt[y]; });
-  if ((rc = upload(&ix->ltab, ltab.data(), ltab.size(), "upload list tables")) ||
-      (rc = upload(&ix->order, order.data(), order.size(), "upload list order")) ||
+  if ((rc = upload(&ix->order, order.data(), order.size(), "upload list order")) ||
       (rc = upload(&ix->centroids, cent.data(), cent.size(), "upload centroids")) ||
       (rc = upload(&ix->codebooks, books.data(), books.size(), "upload codebooks")) ||
-      (rc = upload(&ix->codes, packed.data(), packed.size(), "upload codes")) ||
+      (rc = pack_index(*ix, d, slot, list_of, yn2)) ||
       (rc = upload(&ix->ids, pids.data(), pids.size(), "upload ids")) ||
       (rc = upload(&ix->list_len, len32.data(), len32.size(), "upload list_len")) ||
       (rc = upload(&ix->vec_off, voff.data(), voff.size(), "upload vec_off")) ||

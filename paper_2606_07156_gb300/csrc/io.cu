@@ -42,6 +42,25 @@ struct Reader {
   template <typename T> T val() { T v{}; get(&v, sizeof v); return v; }
 };
 
+// The codes of vector `row` (list order) from the warp-interleaved tiles: byte m
+// of vector v of list l sits in tile tile_off[l] + v / 32, chunk m / 16, lane
+// v % 32, byte m % 16.
+__global__ void unpack_codes_kernel(const uint8_t* __restrict__ packed, const int64_t* __restrict__ vec_off,
+                                    const int64_t* __restrict__ tile_off, int nlist, int64_t n, int M, int nchunk,
+                                    uint8_t* __restrict__ rows) {
+  const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (row >= n) return;
+  int lo = 0, hi = nlist - 1;  // the last list that starts at or before row
+  while (lo < hi) {
+    const int mid = lo + (hi - lo + 1) / 2;
+    if (vec_off[mid] <= row) lo = mid;
+    else hi = mid - 1;
+  }
+  const int64_t v = row - vec_off[lo];
+  const uint8_t* src = packed + (size_t)(tile_off[lo] + v / kTileVecs) * nchunk * kTileChunkBytes + (v % kTileVecs) * kChunkBytes;
+  for (int m = 0; m < M; ++m) rows[row * M + m] = src[(m >> 4) * kTileChunkBytes + (m & 15)];
+}
+
 uint64_t fnv1a(const uint8_t* p, size_t n) {
   uint64_t h = 0xcbf29ce484222325ull;
   for (size_t i = 0; i < n; ++i) { h ^= p[i]; h *= 0x100000001b3ull; }
@@ -66,21 +85,15 @@ extern "C" int anns_export_index(anns_index* ix, float* centroids, float* codebo
     e = cudaMemcpy(codebooks, ix->codebooks, (size_t)ix->M * ANNS_KSUB * dsub * 4, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && ids) e = cudaMemcpy(ids, ix->ids, (size_t)ix->n * 8, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && codes && ix->n > 0) {
-    // unpack the warp-interleaved tiles: byte m of vector v of list l sits in
-    // tile tile_off[l] + v / 32, chunk m / 16, lane v % 32, byte m % 16
-    std::vector<uint8_t> packed((size_t)ix->ntiles * ix->nchunk * kTileChunkBytes);
-    std::vector<int64_t> toff(ix->nlist + 1);
-    e = cudaMemcpy(packed.data(), ix->codes, packed.size(), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(toff.data(), ix->tile_off, toff.size() * 8, cudaMemcpyDeviceToHost);
+    uint8_t* rows = nullptr;
+    e = cudaMalloc((void**)&rows, (size_t)ix->n * ix->M);
     if (e == cudaSuccess) {
-      int64_t row = 0;
-      for (int64_t l = 0; l < ix->nlist; ++l)
-        for (int64_t v = 0; v < ix->h_list_len64[l]; ++v, ++row) {
-          const int64_t t = toff[l] + v / kTileVecs, lane = v % kTileVecs;
-          for (int64_t m = 0; m < ix->M; ++m)
-            codes[row * ix->M + m] = packed[((size_t)t * ix->nchunk + m / 16) * kTileChunkBytes +
-                                            lane * kChunkBytes + m % 16];
-        }
+      unpack_codes_kernel<<<(unsigned)((ix->n + 255) / 256), 256>>>(ix->codes, ix->vec_off, ix->tile_off, (int)ix->nlist,
+                                                                    ix->n, (int)ix->M, (int)ix->nchunk, rows);
+      note_launch();
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaMemcpy(codes, rows, (size_t)ix->n * ix->M, cudaMemcpyDeviceToHost);
+      cudaFree(rows);
     }
   }
   cudaSetDevice(prev);
