@@ -601,7 +601,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     FilterResult r{};
     e = launch_search_filter(ix, Q, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
                              ix.ws_bits, ix.ws_fl, q16, q16_rows, tables_for_all,
-                             P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8, di, dd, grouped ? part_i : nullptr,
+                             P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8, nib, di, dd, grouped ? part_i : nullptr,
                              grouped ? part_d : nullptr, &r, s);
     if (e != cudaSuccess) return cuda_fail(e, "filter kernels");
     // queries with more candidates than fit (usually none): their FP32, 12- and

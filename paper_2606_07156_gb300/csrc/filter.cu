@@ -789,6 +789,8 @@ struct FinalArgs {
   const int* qcnt; const uint2* cand;
   const float* Q; const float* books; const float* ltab; const float* qt;
   const uint8_t* codes; const int64_t* ids; const int64_t* tile_off; const int64_t* vec_off;
+  int fin_warp;
+  int32_t* quant_list; int* nquant;              // queries of a mixed batch for final_kernel, or null
   int32_t* over; int* nover; uint8_t* overflag;  // queries for the scanning kernels
   int64_t* over_i; float* over_d;                // their padding, or null
   int64_t* ids_out; float* dists_out;
@@ -1022,7 +1024,7 @@ __device__ __forceinline__ float block_kth(const uint32_t (&key)[VPT], int kq, i
 // every finished batch lowers T to the k-th exact distance so far, and a pair
 // none of whose candidates reaches T is skipped. `cap` <= VPT * kFinalThreads.
 template <int VPT, int DS, int BATCH>
-__global__ void __launch_bounds__(kFinalThreads, BATCH == 1 ? 4 : 2) final_kernel(const FinalArgs a) {
+__device__ __forceinline__ void final_query(const FinalArgs& a, const int64_t q) {
   __shared__ int wsum[2][32];
   __shared__ float kj[ANNS_MAX_NPROBE], tj[ANNS_MAX_NPROBE];
   __shared__ int coff[ANNS_MAX_NPROBE + 1], cfill[ANNS_MAX_NPROBE];
@@ -1034,7 +1036,7 @@ __global__ void __launch_bounds__(kFinalThreads, BATCH == 1 ? 4 : 2) final_kerne
   float* cex = cdist + a.fin;                  // the exact distance, +inf until it is known (and if it never is)
   uint32_t* cjp = (uint32_t*)(cex + a.fin);
   float* qs = (float*)(cjp + a.fin);
-  const int64_t q = blockIdx.x, row = q * a.nprobe;
+  const int64_t row = q * a.nprobe;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* bias = qs + ((a.dim + 3) & ~int64_t(3)) + warp * BATCH * a.Mp;
   const int kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
@@ -1236,9 +1238,25 @@ __global__ void __launch_bounds__(kFinalThreads, BATCH == 1 ? 4 : 2) final_kerne
   }
 }
 
-// final_kernel for batches without quantised tables: one warp per query (a few
-// dozen candidates and about k survivors leave most of a block idle, and its
-// barriers took half the time). `fin` as there.
+// Block = query; LIST: the blocks walk the *nquant queries of quant_list.
+template <int VPT, int DS, int BATCH, bool LIST>
+__global__ void __launch_bounds__(kFinalThreads, BATCH == 1 ? 4 : 2) final_kernel(const FinalArgs a) {
+  if constexpr (!LIST) {
+    final_query<VPT, DS, BATCH>(a, blockIdx.x);
+  } else {
+    const int n = *a.nquant;
+    for (int i = blockIdx.x; i < n; i += gridDim.x) {
+      final_query<VPT, DS, BATCH>(a, a.quant_list[i]);
+      __syncthreads();  // the next query overwrites the shared state
+    }
+  }
+}
+
+// final_kernel for queries without quantised candidates: one warp per query (a
+// few dozen candidates and about k survivors leave most of a block idle, and its
+// barriers took half the time). `fin` as there, `fin_warp` of them here. With
+// quant_list, a query that has quantised survivors, or too many, goes on to
+// final_kernel through that list.
 constexpr int kFWarps = 4;
 template <int DS>
 __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArgs a) {
@@ -1246,17 +1264,17 @@ __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArg
   const int64_t q = (int64_t)blockIdx.x * kFWarps + warp;
   if (q >= a.nq) return;
   const int64_t row = q * a.nprobe;
-  const size_t per = (size_t)a.fin * 16 + (size_t)((a.dim + 3) & ~int64_t(3)) * 4;
+  const size_t per = (size_t)a.fin_warp * 16 + (size_t)((a.dim + 3) & ~int64_t(3)) * 4;
   int64_t* cid = (int64_t*)(anns_dyn_smem + warp * per);
-  float* cex = (float*)(cid + a.fin);
-  uint32_t* cjp = (uint32_t*)(cex + a.fin);  // first the keys of the upper bounds
-  float* qs = (float*)(cjp + a.fin);
+  float* cex = (float*)(cid + a.fin_warp);
+  uint32_t* cjp = (uint32_t*)(cex + a.fin_warp);  // first the keys of the upper bounds
+  float* qs = (float*)(cjp + a.fin_warp);
   const int kq = a.kpq ? min(max(a.kpq[q], 0), a.k) : a.k;
   const int nc = a.ntake[q] > 0 ? a.qcnt[q] : 0;
   const uint2* cand = a.cand + q * a.cap;
   float T = nc > 0 ? a.thr[q] : INFINITY;
   int ns = 0;
-  bool over = nc > a.cap;
+  bool over = nc > a.cap, quant = false;
   if (!over) {
     for (int d = lane; d < a.dim; d += 32) qs[d] = a.Q[q * a.dim + d];
     auto ub_key = [&](int e) {
@@ -1265,7 +1283,7 @@ __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArg
       return bound_key(__fadd_ru(__uint_as_float(c.y), __fadd_ru(a.d2[p], a.eps[p])));
     };
     if (nc > kq) {
-      if (nc <= a.fin) {
+      if (nc <= a.fin_warp) {
         for (int e = lane; e < nc; e += 32) cjp[e] = ub_key(e);
         __syncwarp();
         T = fminf(T, warp_kth_of(nc, kq, [&](int e) { return cjp[e]; }));
@@ -1283,13 +1301,19 @@ __global__ void __launch_bounds__(kFWarps * 32) final_fp32_kernel(const FinalArg
         const int64_t p = row + (c.x >> kPosBits);
         w = c.x;
         in = !(__uint_as_float(c.y) > __fadd_ru(__fadd_ru(T, a.eps[p]), -a.d2[p]));
+        quant = quant || (in && a.bits[p] != 0);
       }
       const unsigned m = __ballot_sync(kFull, in);
       const int at = ns + __popc(m & ((1u << lane) - 1u));
-      if (in && at < a.fin) cjp[at] = w;
+      if (in && at < a.fin_warp) cjp[at] = w;
       ns += __popc(m);
     }
-    over = ns > a.fin;
+    over = ns > a.fin_warp;
+    quant = __any_sync(kFull, quant);
+  }
+  if (a.quant_list && (over || quant)) {
+    if (lane == 0) a.quant_list[atomicAdd(a.nquant, 1)] = (int32_t)q;
+    return;
   }
   if (over) {
     if (lane == 0) {
@@ -1482,7 +1506,7 @@ struct FilterWork {
   int2* sel;
   PassArgs p1{}, p2{};
   uint2* cand;
-  int32_t* over;
+  int32_t *over, *quant;
   void* Qf;
 };
 
@@ -1515,7 +1539,8 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
     p->cnt = w.take<int>(L);
     p->fill = w.take<int>(L);
   }
-  w.qcnt = w.take<int>(nq); w.nover = w.take<int>(1); w.alive = w.take<uint8_t>(P);
+  w.qcnt = w.take<int>(nq); w.nover = w.take<int>(2);  // and the count of `quant`
+  w.alive = w.take<uint8_t>(P);
   w.overflag = w.take<uint8_t>(nq);
   w.zero_bytes = w.bytes;
   for (PassArgs* p : {&w.p1, &w.p2}) {
@@ -1532,7 +1557,7 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
   w.eps = w.take<float>(P); w.eps0 = w.take<float>(P); w.thr = w.take<float>(nq); w.ub = w.take<float>(nq * filter_take(ix, k));
   w.sel = w.take<int2>(P);
   w.cand = w.take<uint2>(nq * filter_cap(k));
-  w.over = w.take<int32_t>(nq);
+  w.over = w.take<int32_t>(nq); w.quant = w.take<int32_t>(nq);
   w.qrows = w.take<float>(3 * nq);
   w.Qf = w.take<__half>(nq * Dp);
   return w;
@@ -1544,26 +1569,31 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
 // against 1.74; uneven GIST-shaped 2.5 against 3.6).
 template <int VPT>
 cudaError_t run_final_ds(const FinalArgs& a, cudaStream_t s) {
-  const int batch = a.k >= 64 && a.nprobe >= 48 && !a.npq ? kBatch : 1;
+  const int batch = a.k >= 64 && a.nprobe >= 48 && !a.npq && !a.quant_list ? kBatch : 1;
   auto go = [&](auto kern) {
     const size_t sm = final_smem(a.dim, a.Mp, a.fin, batch);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)a.nq, kFinalThreads, sm, s>>>(a);
+    // of a list usually a part of the batch: blocks for a few waves
+    kern<<<(unsigned)(a.quant_list ? std::min<int64_t>(a.nq, 2048) : a.nq), kFinalThreads, sm, s>>>(a);
     note_launch();
     return cudaGetLastError();
   };
   switch (a.dsub) {
-    case 2: return batch == 1 ? go(final_kernel<VPT, 2, 1>) : go(final_kernel<VPT, 2, kBatch>);
-    case 4: return batch == 1 ? go(final_kernel<VPT, 4, 1>) : go(final_kernel<VPT, 4, kBatch>);
-    case 8: return batch == 1 ? go(final_kernel<VPT, 8, 1>) : go(final_kernel<VPT, 8, kBatch>);
-    default: return batch == 1 ? go(final_kernel<VPT, 0, 1>) : go(final_kernel<VPT, 0, kBatch>);
+    case 2: return a.quant_list ? go(final_kernel<VPT, 2, 1, true>)
+                   : batch == 1 ? go(final_kernel<VPT, 2, 1, false>) : go(final_kernel<VPT, 2, kBatch, false>);
+    case 4: return a.quant_list ? go(final_kernel<VPT, 4, 1, true>)
+                   : batch == 1 ? go(final_kernel<VPT, 4, 1, false>) : go(final_kernel<VPT, 4, kBatch, false>);
+    case 8: return a.quant_list ? go(final_kernel<VPT, 8, 1, true>)
+                   : batch == 1 ? go(final_kernel<VPT, 8, 1, false>) : go(final_kernel<VPT, 8, kBatch, false>);
+    default: return a.quant_list ? go(final_kernel<VPT, 0, 1, true>)
+                    : batch == 1 ? go(final_kernel<VPT, 0, 1, false>) : go(final_kernel<VPT, 0, kBatch, false>);
   }
 }
 
 cudaError_t run_final_fp32(const FinalArgs& a, cudaStream_t s) {
   auto go = [&](auto kern) {
-    const size_t sm = kFWarps * ((size_t)a.fin * 16 + (size_t)((a.dim + 3) & ~int64_t(3)) * 4);
+    const size_t sm = kFWarps * ((size_t)a.fin_warp * 16 + (size_t)((a.dim + 3) & ~int64_t(3)) * 4);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((a.nq + kFWarps - 1) / kFWarps), kFWarps * 32, sm, s>>>(a);
@@ -1710,7 +1740,7 @@ size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k) {
 cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* qt, int64_t nq, int nprobe,
                                  const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
                                  const float* probe_d2, const uint8_t* bits, void* ws, const void* q16,
-                                 const float* q16_rows, bool quantised, bool exact_threshold, int64_t* ids_out, float* dists_out,
+                                 const float* q16_rows, bool quantised, bool exact_threshold, bool mixed, int64_t* ids_out, float* dists_out,
                                  int64_t* over_i, float* over_d, FilterResult* out, cudaStream_t s) {
   FilterWork w = filter_work(ix, nq, nprobe, k, (char*)ws);
   cudaError_t e = cudaMemsetAsync(w.base, 0, w.zero_bytes, s);
@@ -1785,12 +1815,14 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   }
   if (e != cudaSuccess) return e;
   if ((e = pass(std::integral_constant<int, 2>{}, w.p2)) != cudaSuccess) return e;
-  if (quantised) {
-    e = f.cap == 2048 ? run_final_ds<8>(f, s) : run_final_ds<16>(f, s);
-  } else {
-    f.fin = k <= 32 ? 256 : 512;
-    e = run_final_fp32(f, s);
-  }
+  // a mixed batch settles the queries whose candidates are all on FP32 tables (a
+  // predictor keeps those for the nearest lists) a warp each first (Deep-shaped,
+  // learned widths: 383 us in blocks, 156 + 188 us so)
+  f.fin_warp = k <= 32 ? 256 : 512;
+  f.quant_list = quantised && mixed ? w.quant : nullptr;
+  f.nquant = w.nover + 1;
+  if (!quantised || mixed) e = run_final_fp32(f, s);
+  if (e == cudaSuccess && quantised) e = f.cap == 2048 ? run_final_ds<8>(f, s) : run_final_ds<16>(f, s);
   out->over = w.over;
   out->nover = w.nover;
   out->alive = w.alive;

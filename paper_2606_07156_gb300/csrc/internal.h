@@ -294,11 +294,12 @@ struct FilterResult {
 // for the queries in out->over, which get padding in over_i / over_d (if
 // given). `quantised`: some pairs are on 5..16-bit tables (qt then holds the
 // query tables); `exact_threshold`: the nearest ones are, so that the k-th
-// distance is better bounded by exact distances than by upper bounds; q16 and q16_rows are the queries' FP16 operand if it exists.
+// distance is better bounded by exact distances than by upper bounds; `mixed`:
+// some pairs may be on FP32 tables too; q16 and q16_rows are the queries' FP16 operand if it exists.
 cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* qt, int64_t nq, int nprobe,
                                  const int32_t* nprobe_per_q, int k, const int32_t* k_per_q, const int32_t* probes,
                                  const float* probe_d2, const uint8_t* bits, void* ws, const void* q16,
-                                 const float* q16_rows, bool quantised, bool exact_threshold, int64_t* ids_out,
+                                 const float* q16_rows, bool quantised, bool exact_threshold, bool mixed, int64_t* ids_out,
                                  float* dists_out,
                                  int64_t* over_i, float* over_d, FilterResult* out, cudaStream_t s);
 
