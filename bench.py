@@ -484,12 +484,13 @@ def subspace_sweep(amp, index, W, cfg, nprobe: int, k: int, dev, nq: int = 2000)
 STAGES_CL = ("cl_distances", "cl_select (the whole tensor-core CL)", "precision_choice+query_tables")
 
 
-def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray):
+def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray, row_bytes: int = 0):
     """Names of the profile stages (anns_profile) for the search that ran, and
     the candidates for the roofline's dominant kernel: (label, source file, ms
     per step, algorithmic code bytes). `kernel` is the autotuner's choice
     ("split", "grouped", "automatic" (filtered), ...; None: the one without a trial), `st_ms` the stage
     times, `bits` and `pb` the pairs' table widths and code bytes [nq, nprobe].
+    `row_bytes`: the decoded FP16 rows the filter reads at least once.
     The split search runs its wide pairs (stage 3) and then every 1..8-bit pair
     (stage 4); the grouped search runs every rank-0 pair and the wide pairs in
     its query-major pass (stage 3), the other 1..8-bit pairs in the byte-table
@@ -508,7 +509,7 @@ def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray):
         names = STAGES_CL + ("filtered_search (plan + two GEMM passes + exact distances)", "grouped_kernel_5to8bit (unsettled)",
                              "grouped_kernel_4bit_nibble (pairs with candidates)", "grouped_merge")
         return names, [("filter_gemm_kernel (filtered search: all of plan, GEMM passes and exact distances)", "filter.cu",
-                        st_ms[3], int(pb.sum()))]
+                        st_ms[3], row_bytes)]
     names = STAGES_CL + ("search_before_grouped (invert + query-major)", "grouped_kernel_5to8bit",
                          "grouped_kernel_4bit_nibble", "grouped_merge")
     if not (st_ms[4] > 0.0 or st_ms[5] > 0.0):
@@ -787,7 +788,8 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
     # roofline of the dominant kernel of the adaptive step (search_stages)
     pb = pair_bytes(index, probes_ad, cfg["M"])
     st_ms = [v / max(cnt, 1) for v in stage_ms]
-    stage_names, cands = search_stages(tuned["kernel"] if tuned is not None else None, st_ms, bits_ad, pb)
+    stage_names, cands = search_stages(tuned["kernel"] if tuned is not None else None, st_ms, bits_ad, pb,
+                                       int(W["codes"].shape[0]) * cfg["dim"] * 2)
     kname, kfile, kms, nbytes = max(cands, key=lambda c: c[2])
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else None
@@ -802,7 +804,8 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
             "traffic": prof["dram_bytes_per_launch"] if prof else None,
             "algorithmic_bytes_per_launch": nbytes, "kernel_ms": round(kms, 4),
             "lookups_per_s": round(nbytes / (kms / 1e3), 1),
-            "achieved_is": "algorithmic bytes (one code byte per LUT lookup, query-major) / kernel time"}
+            "achieved_is": "decoded FP16 rows read once / time of the whole filtered stage" if kfile == "filter.cu" else
+                           "algorithmic bytes (one code byte per LUT lookup, query-major) / kernel time"}
     if prof:
         dram_gbs = prof["dram_bytes_per_launch"] / (kms / 1e3) / 1e9
         roof.update({"dram_gbs": round(dram_gbs, 1), "dram_frac": round(dram_gbs / peak, 4),
