@@ -563,42 +563,32 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
   } else {
     for (int l = threadIdx.x; l < nl; l += kRThreads) vals[l] = row[l];  // read back by this thread only
   }
-  // the np-th smallest of the threads' minima: at least np lists lie at or
-  // below it, and few more (a thread without lists, or with none but NaN: +inf)
-  float least = INFINITY;
-  each([&](int, float v) { least = fminf(least, v); });
-  const uint32_t mine = upper_key(least);
-  uint32_t lo = __reduce_min_sync(kFull, mine), hi = 0x7F800000u;
-  if (lane == 0) kr[0][warp] = lo;
-  __syncthreads();
-  for (int w = 0; w < kRWarps; ++w) lo = min(lo, kr[0][w]);
-  const uint32_t lowest = lo;
-  while (hi - lo > 4095u) {  // count(mine <= hi) >= np throughout, or hi = +inf
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    if (__syncthreads_count(mine <= mid) >= np) hi = mid;
-    else lo = mid + 1u;
-  }
-  // the values up to it, and the np-th smallest of them
-  {
-    const float U = __uint_as_float(hi);
-    each([&](int, float v) {
-      if (v <= U) {
-        const int at = atomicAdd(&total, 1);
-        if (at < kNear) near_keys[at] = upper_key(v);
-      }
-    });
-  }
-  __syncthreads();
-  const int nn = total;
-  __syncthreads();
-  if (threadIdx.x == 0) total = 0;
-  if (nn <= kNear) {
+  // Up to 32 lists are one batch of the distance kernel whichever of them are
+  // candidates: all are, without a limit. Up to 128, one warp bisects over the
+  // row, four values a lane, without the block's barriers.
+  // (BF16, D 96, nprobe 6, 10000 queries: 16 lists 79 us, 128 lists 114 us; the
+  // radix select this kernel had before 144 and 147 us.) Beyond, the block's
+  // barriers cost more than that radix select did up to some 2000 lists: 160
+  // lists 179 and 149 us, 900 lists 197 and 196 us; from 8192 on they cost less.
+  float X = INFINITY;
+  uint32_t hi = 0x7F800000u;
+  if (nl > 32 && nl <= 128) {
     if (warp == 0) {
-      uint32_t l2 = lowest, h2 = hi;
+      uint32_t key[4], l2 = 0xFFFFFFFFu, h2 = 0u;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int l = lane + 32 * j;
+        key[j] = l < nl ? upper_key(row[l]) : 0xFFFFFFFFu;  // past the row: never counted
+        l2 = min(l2, key[j]);
+        if (l < nl) h2 = max(h2, key[j]);
+      }
+      l2 = __reduce_min_sync(kFull, l2);
+      h2 = __reduce_max_sync(kFull, h2);
       while (h2 - l2 > 1023u) {
         const uint32_t mid = l2 + ((h2 - l2) >> 1);
         int c = 0;
-        for (int i = lane; i < nn; i += 32) c += near_keys[i] <= mid ? 1 : 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c += key[j] <= mid ? 1 : 0;
         if ((int)__reduce_add_sync(kFull, c) >= np) h2 = mid;
         else l2 = mid + 1u;
       }
@@ -606,24 +596,70 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
     }
     __syncthreads();
     hi = sh[0];
-  } else {  // many equal values, or fewer lists than threads: over all of them
-    lo = lowest;
-    hi = 0x7F800000u;
-    for (int step = 0; hi - lo > 1023u; ++step) {
+  } else if (nl > 128) {
+    // the np-th smallest of the threads' minima: at least np lists lie at or
+    // below it, and few more (a thread without lists, or with none but NaN: +inf)
+    float least = INFINITY;
+    each([&](int, float v) { least = fminf(least, v); });
+    const uint32_t mine = upper_key(least);
+    uint32_t lo = __reduce_min_sync(kFull, mine);
+    hi = __reduce_max_sync(kFull, (int)threadIdx.x < nl ? mine : 0u);
+    if (lane == 0) { kr[0][warp] = lo; kr[1][warp] = hi; }
+    __syncthreads();
+    for (int w = 0; w < kRWarps; ++w) { lo = min(lo, kr[0][w]); hi = max(hi, kr[1][w]); }
+    const uint32_t lowest = lo;
+    while (hi - lo > 4095u) {  // count(mine <= hi) >= np throughout
       const uint32_t mid = lo + ((hi - lo) >> 1);
-      const float midf = __uint_as_float(mid);
-      int c = 0;
-      each([&](int, float v) { c += v <= midf ? 1 : 0; });  // a NaN never counts
-      c = __reduce_add_sync(kFull, c);
-      if (lane == 0) kr[step & 1][warp] = (uint32_t)c;
-      __syncthreads();
-      int t = 0;
-      for (int w = 0; w < kRWarps; ++w) t += (int)kr[step & 1][w];
-      if (t >= np) hi = mid;
+      if (__syncthreads_count(mine <= mid) >= np) hi = mid;
       else lo = mid + 1u;
     }
+    // the values up to it, and the np-th smallest of them
+    {
+      const float U = __uint_as_float(hi);
+      each([&](int, float v) {
+        if (v <= U) {
+          const int at = atomicAdd(&total, 1);
+          if (at < kNear) near_keys[at] = upper_key(v);
+        }
+      });
+    }
+    __syncthreads();
+    const int nn = total;
+    __syncthreads();
+    if (threadIdx.x == 0) total = 0;
+    if (nn <= kNear) {
+      if (warp == 0) {
+        uint32_t l2 = lowest, h2 = hi;
+        while (h2 - l2 > 1023u) {
+          const uint32_t mid = l2 + ((h2 - l2) >> 1);
+          int c = 0;
+          for (int i = lane; i < nn; i += 32) c += near_keys[i] <= mid ? 1 : 0;
+          if ((int)__reduce_add_sync(kFull, c) >= np) h2 = mid;
+          else l2 = mid + 1u;
+        }
+        if (lane == 0) sh[0] = h2;
+      }
+      __syncthreads();
+      hi = sh[0];
+    } else {  // many equal values, or fewer lists than threads: over all of them
+      lo = lowest;
+      hi = 0x7F800000u;
+      for (int step = 0; hi - lo > 1023u; ++step) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        const float midf = __uint_as_float(mid);
+        int c = 0;
+        each([&](int, float v) { c += v <= midf ? 1 : 0; });  // a NaN never counts
+        c = __reduce_add_sync(kFull, c);
+        if (lane == 0) kr[step & 1][warp] = (uint32_t)c;
+        __syncthreads();
+        int t = 0;
+        for (int w = 0; w < kRWarps; ++w) t += (int)kr[step & 1][w];
+        if (t >= np) hi = mid;
+        else lo = mid + 1u;
+      }
+    }
   }
-  const float X = candidate_limit(a, __uint_as_float(hi), qn, qd);
+  if (nl > 32) X = candidate_limit(a, __uint_as_float(hi), qn, qd);
   __syncthreads();
   // B
   each([&](int l, float v) {

@@ -116,3 +116,22 @@ def test_fp32_coarse_stage_through_the_tensor_cores(amp, dim, nlist, nq):
             g.tap(amp.abi.TAP_COARSE_CANDIDATES, (nq,), np.int32)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("nlist", [17, 32, 33, 100, 128, 129, 255, 300])
+@pytest.mark.parametrize("cl", ["bf16", "fp8"])
+def test_short_rows_of_the_tensor_core_coarse_stage(amp, nlist, cl):
+    """Every list a candidate up to 32 lists, one warp's selection up to 128, the
+    block's beyond: the FP32 rule's probes and distances, ties and a repeated centroid included."""
+    r = np.random.Generator(np.random.PCG64(nlist))
+    C = r.standard_normal((nlist, 24)).astype(np.float32)
+    C[nlist // 2] = C[1]
+    Q = np.concatenate([C[:2], r.standard_normal((75, 24)).astype(np.float32), 50 * C[3:4]])
+    books = r.standard_normal((4, 256, 6)).astype(np.float32)
+    g = amp.Index(C, books, r.integers(0, 256, (nlist, 4)).astype(np.uint8), np.arange(nlist, dtype=np.int32), device=0)
+    for nprobe in (1, 16, min(nlist, 128)):
+        rp, rd = ivfpq.locate(ivfpq.coarse_d2_fp32(Q, C), nprobe)
+        p, d = g.locate(torch.from_numpy(Q).to("cuda:0"), nprobe, cl=cl)
+        np.testing.assert_array_equal(p.cpu().numpy(), rp)
+        np.testing.assert_array_equal(d.cpu().numpy(), rd)
+    g.close()
