@@ -159,30 +159,33 @@ int pack_index(Index& ix, const anns_build_desc* d, const std::vector<int64_t>& 
                const std::vector<double>& yn2) {
   const int64_t n = ix.n;
   const size_t code_bytes = std::max<size_t>((size_t)ix.ntiles * ix.nchunk * kTileChunkBytes, 16);
+  const int64_t step = std::min<int64_t>(n, (int64_t)1 << 24);  // vectors at a time: bounded temporary memory
   Temp codes, slots, lists, norms, rmax;
   cudaError_t e = cudaMalloc((void**)&ix.codes, code_bytes);
   if (e == cudaSuccess) e = cudaMalloc((void**)&ix.ltab, (size_t)ix.nlist * ix.Mp * kKsub * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&slots.p, std::max<size_t>(n * 8, 16));
-  if (e == cudaSuccess) e = cudaMalloc(&lists.p, std::max<size_t>(n * 4, 16));
+  if (e == cudaSuccess) e = cudaMalloc(&slots.p, std::max<size_t>(step * 8, 16));
+  if (e == cudaSuccess) e = cudaMalloc(&lists.p, std::max<size_t>(step * 4, 16));
   if (e == cudaSuccess) e = cudaMalloc(&norms.p, yn2.size() * 8);
   if (e == cudaSuccess) e = cudaMalloc(&rmax.p, (size_t)ix.nlist * 8);
-  const uint8_t* src = d->codes;
-  if (e == cudaSuccess && !d->on_device && n > 0) {
-    e = cudaMalloc(&codes.p, (size_t)n * ix.M);
-    if (e == cudaSuccess) e = cudaMemcpy(codes.p, d->codes, (size_t)n * ix.M, cudaMemcpyHostToDevice);
-    src = (const uint8_t*)codes.p;
-  }
+  if (e == cudaSuccess && !d->on_device) e = cudaMalloc(&codes.p, std::max<size_t>(step * ix.M, 16));
   if (e == cudaSuccess) e = cudaMemset(ix.codes, 0, code_bytes);
   if (e == cudaSuccess) e = cudaMemset(rmax.p, 0, (size_t)ix.nlist * 8);
   if (e == cudaSuccess) e = cudaMemcpy(norms.p, yn2.data(), yn2.size() * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && n > 0) e = cudaMemcpy(slots.p, slot.data(), n * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && n > 0) e = cudaMemcpy(lists.p, list_of.data(), n * 4, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(e, "index arrays");
-  if (n > 0) {
-    pack_codes_kernel<<<(unsigned)((n * ix.nchunk + 255) / 256), 256>>>(src, (const int64_t*)slots.p, n, (int)ix.M,
+  for (int64_t i0 = 0; i0 < n; i0 += step) {
+    const int64_t m = std::min(step, n - i0);
+    const uint8_t* src = d->codes + i0 * ix.M;
+    e = cudaMemcpy(slots.p, slot.data() + i0, m * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(lists.p, list_of.data() + i0, m * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !d->on_device) {
+      e = cudaMemcpy(codes.p, src, (size_t)m * ix.M, cudaMemcpyHostToDevice);
+      src = (const uint8_t*)codes.p;
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "index arrays");
+    pack_codes_kernel<<<(unsigned)((m * ix.nchunk + 255) / 256), 256>>>(src, (const int64_t*)slots.p, m, (int)ix.M,
                                                                         (int)ix.nchunk, ix.codes);
     note_launch();
-    radius_kernel<<<(unsigned)((n + 255) / 256), 256>>>(src, (const int32_t*)lists.p, n, (int)ix.M,
+    radius_kernel<<<(unsigned)((m + 255) / 256), 256>>>(src, (const int32_t*)lists.p, m, (int)ix.M,
                                                         (const double*)norms.p, (unsigned long long*)rmax.p);
     note_launch();
   }

@@ -8,6 +8,7 @@
 //   | (flag 1) anns_predictor | (flag 2) i32 nsv, i32 table_n, f64 ratio,
 //   f32 gamma, f32 inv_step, f32 mean[5], f32 inv_std[5], f32 sv [nsv*5],
 //   f32 beta [nsv] | u64 checksum.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -42,14 +43,14 @@ struct Reader {
   template <typename T> T val() { T v{}; get(&v, sizeof v); return v; }
 };
 
-// The codes of vector `row` (list order) from the warp-interleaved tiles: byte m
+// The codes of vectors r0 .. r0 + n - 1 (list order) from the warp-interleaved tiles: byte m
 // of vector v of list l sits in tile tile_off[l] + v / 32, chunk m / 16, lane
 // v % 32, byte m % 16.
 __global__ void unpack_codes_kernel(const uint8_t* __restrict__ packed, const int64_t* __restrict__ vec_off,
-                                    const int64_t* __restrict__ tile_off, int nlist, int64_t n, int M, int nchunk,
-                                    uint8_t* __restrict__ rows) {
-  const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (row >= n) return;
+                                    const int64_t* __restrict__ tile_off, int nlist, int64_t r0, int64_t n, int M,
+                                    int nchunk, uint8_t* __restrict__ rows) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, row = r0 + i;
+  if (i >= n) return;
   int lo = 0, hi = nlist - 1;  // the last list that starts at or before row
   while (lo < hi) {
     const int mid = lo + (hi - lo + 1) / 2;
@@ -58,7 +59,7 @@ __global__ void unpack_codes_kernel(const uint8_t* __restrict__ packed, const in
   }
   const int64_t v = row - vec_off[lo];
   const uint8_t* src = packed + (size_t)(tile_off[lo] + v / kTileVecs) * nchunk * kTileChunkBytes + (v % kTileVecs) * kChunkBytes;
-  for (int m = 0; m < M; ++m) rows[row * M + m] = src[(m >> 4) * kTileChunkBytes + (m & 15)];
+  for (int m = 0; m < M; ++m) rows[i * M + m] = src[(m >> 4) * kTileChunkBytes + (m & 15)];
 }
 
 uint64_t fnv1a(const uint8_t* p, size_t n) {
@@ -86,15 +87,17 @@ extern "C" int anns_export_index(anns_index* ix, float* centroids, float* codebo
   if (e == cudaSuccess && ids) e = cudaMemcpy(ids, ix->ids, (size_t)ix->n * 8, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && codes && ix->n > 0) {
     uint8_t* rows = nullptr;
-    e = cudaMalloc((void**)&rows, (size_t)ix->n * ix->M);
-    if (e == cudaSuccess) {
-      unpack_codes_kernel<<<(unsigned)((ix->n + 255) / 256), 256>>>(ix->codes, ix->vec_off, ix->tile_off, (int)ix->nlist,
-                                                                    ix->n, (int)ix->M, (int)ix->nchunk, rows);
+    const int64_t step = std::min<int64_t>(ix->n, (int64_t)1 << 24);  // vectors at a time: bounded temporary memory
+    e = cudaMalloc((void**)&rows, (size_t)step * ix->M);
+    for (int64_t r0 = 0; r0 < ix->n && e == cudaSuccess; r0 += step) {
+      const int64_t m = std::min(step, ix->n - r0);
+      unpack_codes_kernel<<<(unsigned)((m + 255) / 256), 256>>>(ix->codes, ix->vec_off, ix->tile_off, (int)ix->nlist, r0,
+                                                                m, (int)ix->M, (int)ix->nchunk, rows);
       note_launch();
       e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaMemcpy(codes, rows, (size_t)ix->n * ix->M, cudaMemcpyDeviceToHost);
-      cudaFree(rows);
+      if (e == cudaSuccess) e = cudaMemcpy(codes + r0 * ix->M, rows, (size_t)m * ix->M, cudaMemcpyDeviceToHost);
     }
+    if (rows) cudaFree(rows);
   }
   cudaSetDevice(prev);
   if (e != cudaSuccess) return cuda_fail(e, "index export");
