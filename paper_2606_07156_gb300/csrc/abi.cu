@@ -516,18 +516,32 @@ static bool use_lpt(const Index& ix, const int32_t* nprobe_per_q) {
   return ix.opt_schedule == ANNS_SCHED_LPT || (ix.opt_schedule == ANNS_SCHED_AUTO && nprobe_per_q);
 }
 
+static int reserve_filter(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P) {
+  int rc = grow(&ix.ws_fl, &ix.ws_fl_cap, filter_workspace_bytes(ix, nq, nprobe, k));
+  if (rc || !grouped_after_filter(ix, P, k)) return rc;
+  ListWork w{};
+  if ((rc = list_workspace(ix, nq, nprobe, k, w, nq))) return rc;
+  return grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k));
+}
+
 int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
                    const int32_t* nprobe_per_q) {
   int rc = ensure_workspace(ix, nq, nprobe);
   if (rc) return rc;
-  if (use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr)) {
-    if ((rc = grow(&ix.ws_fl, &ix.ws_fl_cap, filter_workspace_bytes(ix, nq, nprobe, k)))) return rc;
-    if (grouped_after_filter(ix, P, k)) {
-      ListWork w{};
-      if ((rc = list_workspace(ix, nq, nprobe, k, w, nq))) return rc;
-      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
-    }
-  } else {
+  bool filter = use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  if (filter && (rc = reserve_filter(ix, nq, nprobe, k, P))) {
+    if (rc != ANNS_ERR_OOM) return rc;
+    // No room for the filter's workspace, which is larger than the scan's:
+    // batches of this size scan from now on.
+    cudaGetLastError();
+    set_error("");
+    if (ix.ws_fl) cudaFree(ix.ws_fl);
+    ix.ws_fl = nullptr;
+    ix.ws_fl_cap = 0;
+    ix.fl_ws_limit = filter_workspace_bytes(ix, nq, nprobe, k) - 1;
+    filter = false;
+  }
+  if (!filter) {
     if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, nq, nprobe, k)) {
       ListWork w{};
       const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);

@@ -57,7 +57,6 @@ constexpr size_t kFilterSmem = 1024 + (size_t)kFStages * kFStage + kEpiWarps * k
 constexpr int kBatch = 4;          // quantised pairs a warp settles at a time
 constexpr int kPosBits = 25;       // candidate word: rank << 25 | position in the list
 constexpr int kTakeMax = 4096;
-constexpr size_t kFilterWorkspaceMax = (size_t)32 << 30;  // larger batches scan
 
 struct FItem { int row0, nv_cnt, slot0, pos0; };  // first row, vectors | queries << 16, first slot, position of row0 in its list
 // Slots: the pairs of a GEMM list by list, each list's first slot a multiple of 16.
@@ -1730,7 +1729,7 @@ bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t n
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))
     return false;
-  return filter_workspace_bytes(ix, nq, nprobe, k) <= kFilterWorkspaceMax;
+  return filter_workspace_bytes(ix, nq, nprobe, k) <= ix.fl_ws_limit;
 }
 
 size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k) {

@@ -64,6 +64,7 @@ struct Index {
   float* fl_ym = nullptr;
   int fl_w = 0;
   float fl_yscale = 1.f, fl_mu = 0.f;  // 1 / scale of the rows, |mu|
+  size_t fl_ws_limit = (size_t)32 << 30;  // workspace the filter may take (lowered where there was no room)
   int64_t fl_tiles = 0;                // sum over the lists of their 256-vector tiles
   // host copies of the small per-list tables
   std::string err;
