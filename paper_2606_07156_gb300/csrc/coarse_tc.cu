@@ -24,8 +24,8 @@
 // 3. Error bound per pair: |D~ - D2| <= eps(D~, rows), D2 the FP32-rule
 //    distance (derivation at rerank_bound). From the nprobe-th
 //    smallest D~ and the largest eps of any list follows a limit of D~ that no
-//    list of the FP32 top-nprobe exceeds (candidate_limit; rerank_stream_kernel
-//    uses each list's own eps); the lists below are re-ranked with the
+//    list of the FP32 top-nprobe exceeds (candidate_limit; rerank_radix_kernel and
+//    rerank_stream_kernel use each list's own eps); the lists below are re-ranked with the
 //    FP32 rule itself (same operation order as coarse.cu) and the nprobe
 //    smallest (D2, l) kept: identical output to the plain path. The re-rank
 //    runs in three kernels: a select kernel per query (the limit, the
@@ -447,6 +447,63 @@ __device__ __forceinline__ float batch_d2_any(const float* __restrict__ C, const
   return acc;
 }
 
+// An upper bound, within 2^8 - 1 units of the last place, of the np-th
+// smallest of keys[0..n) (1 <= np <= n), all in [kmin, kmax] <= +inf: radix
+// levels of 8 bits over key - kmin, the first level's shift fitted to the
+// range, each level counting only the keys inside the bin chosen before, until
+// the bins are at most 2^8 keys wide; the top of the last bin chosen.
+__device__ uint32_t block_select(const uint32_t* keys, int64_t n, int np, uint32_t kmin, uint32_t kmax, int* hist,
+                                 uint32_t* sh) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int shift = 0;
+  while (((kmax - kmin) >> shift) > 255u) ++shift;
+  uint32_t lo = 0;                        // relative start of the current range
+  uint32_t span_m1 = kmax - kmin;         // its length - 1 (keys <= 0x7F800000: no overflow)
+  int need = np;
+  for (;;) {
+    for (int i = tid; i < 256; i += blockDim.x) hist[i] = 0;
+    __syncthreads();
+    for (int64_t l = tid; l < n; l += blockDim.x) {
+      const uint32_t rel = keys[l] - kmin - lo;   // wraps below lo: outside the range
+      if (rel <= span_m1) atomicAdd(&hist[rel >> shift], 1);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int c[8], run = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { c[i] = hist[lane * 8 + i]; run += c[i]; }
+      int incl = run;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const int excl = incl - run;
+      int pick = -1, below = 0;
+      if (excl < need && need <= incl) {
+        int acc = excl;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (pick < 0 && acc + c[i] >= need) { pick = lane * 8 + i; below = acc; }
+          acc += c[i];
+        }
+      }
+      const unsigned who = __ballot_sync(kFull, pick >= 0);
+      const int src = who ? __ffs(who) - 1 : 0;
+      pick = __shfl_sync(kFull, pick, src);
+      below = __shfl_sync(kFull, below, src);
+      if (lane == 0) { sh[0] = who ? (uint32_t)pick : 255u; sh[1] = who ? (uint32_t)below : 0u; }
+    }
+    __syncthreads();
+    lo += sh[0] << shift;
+    need -= (int)sh[1];
+    span_m1 = (1u << shift) - 1u;
+    if (shift <= 8) break;
+    shift = shift >= 16 ? shift - 8 : 8;
+  }
+  return min(kmin + lo + span_m1, 0x7F800000u);  // the last bin may reach past +inf's key
+}
+
 // Candidate lists of the split re-rank: up to kCap candidates per query in
 // the workspace, their distances computed by rerank_dist_kernel (one warp per
 // 32 candidates, over all queries at once) and merged by rerank_merge_kernel.
@@ -472,6 +529,58 @@ __device__ __forceinline__ void write_probes(const RerankArgs& a, int64_t q, int
       a.probes[q * a.nprobe + e] = ok ? top.id[r] : -1;
       a.probe_d2[q * a.nprobe + e] = ok ? top.d[r] : INFINITY;
     }
+  }
+}
+
+// What follows a query's selection (a block; cand complete and visible): with at
+// most kCap candidates, the list goes to the workspace with one work item per 32
+// candidates; otherwise the block computes their FP32-rule distances itself, 32
+// per warp batch (batches dealt round-robin to the warps), each warp keeping its
+// top-np by (D2, l), the warps' lists merged at the end. tiles: the warps'
+// staging tiles [8][1056], qs: [dim rounded up to 4], neither over cand.
+template <int R, bool V4>
+__device__ __forceinline__ void rerank_candidates(const RerankArgs& a, const RerankSplit& sp, int64_t q, int np,
+                                                  const int32_t* cand, int nc_all, float* qs, float* tiles,
+                                                  uint32_t* sh) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0 && a.ncand) a.ncand[q] = nc_all;
+  if (nc_all <= kCap) {
+    for (int i = threadIdx.x; i < nc_all; i += kRThreads) sp.cbuf[q * kCap + i] = cand[i];
+    const int nb = (nc_all + 31) >> 5;
+    if (threadIdx.x == 0) sh[0] = (uint32_t)atomicAdd(sp.nitems, nb);
+    __syncthreads();
+    if (threadIdx.x < nb) sp.items[sh[0] + threadIdx.x] = make_int2((int)q, threadIdx.x);
+    return;
+  }
+  // in the block: the query itself and the staging tiles
+  const int dq = (a.dim + 3) & ~3;
+  for (int d = threadIdx.x; d < dq; d += kRThreads) qs[d] = d < a.dim ? a.Q[q * a.dim + d] : 0.f;
+  __syncthreads();
+  WarpTopK<R, int32_t> top;
+  top.init();
+  float thd = INFINITY;
+  int32_t thi = INT32_MAX;
+  float* tile = tiles + warp * kRTile;
+  for (int b0 = warp * 32; b0 < nc_all; b0 += kRWarps * 32) {
+    const int nc = min(32, nc_all - b0);
+    const float dc = V4 ? batch_d2_v4(a.C, qs, a.dim, cand + b0, nc, tile)
+                        : batch_d2_any(a.C, qs, a.dim, cand + b0, nc, tile);
+    top.offer(lane < nc, dc, lane < nc ? cand[b0 + lane] : 0, np, thd, thi);
+  }
+  __syncthreads();  // tiles are free: they hold the warps' lists
+  float* md = tiles;
+  int32_t* mi = (int32_t*)(tiles + kRWarps * R * 32);
+#pragma unroll
+  for (int r = 0; r < R; ++r) { md[(warp * R + r) * 32 + lane] = top.d[r]; mi[(warp * R + r) * 32 + lane] = top.id[r]; }
+  __syncthreads();
+  if (warp == 0) {
+    for (int w = 1; w < kRWarps; ++w)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float v = md[(w * R + r) * 32 + lane];
+        top.offer(v != INFINITY, v, mi[(w * R + r) * 32 + lane], np, thd, thi);
+      }
+    write_probes<R>(a, q, np, top);
   }
 }
 
@@ -506,11 +615,7 @@ __device__ __forceinline__ float candidate_limit(const RerankArgs& a, float T0, 
 // 20000 queries, 8192 lists, nprobe 64: 462 us, bound by issue and barriers; 728
 // us when each list's own bound was formed (25 operations a list) for a radix
 // select over the upper bounds. The shared bound keeps a few more candidates.
-// Then, with at most kCap candidates, the list goes to the workspace with one
-// work item per 32 candidates; otherwise the block computes their FP32-rule
-// distances itself, 32 per warp batch (batches dealt round-robin to the
-// warps), each warp keeping its top-np by (D2, l), the warps' lists merged at
-// the end. Queries with np = 0 get their padding here.
+// Then rerank_candidates. Queries with np = 0 get their padding here.
 // Dynamic shared memory: qs [dim rounded up to 4] | candidate list [nlist
 // rounded up to 4] | the warps' staging tiles [8][1056]; VPT = 0: qs | D~, later
 // the tiles | candidate list.
@@ -531,9 +636,9 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t q = blockIdx.x, nlist = a.nlist;
   const int np = a.npq ? min(max(a.npq[q], 0), a.nprobe) : a.nprobe;
-  WarpTopK<R, int32_t> top;
-  top.init();
   if (np == 0) {
+    WarpTopK<R, int32_t> top;
+    top.init();
     if (warp == 0) write_probes<R>(a, q, 0, top);
     if (threadIdx.x == 0 && a.ncand) a.ncand[q] = 0;
     return;
@@ -566,10 +671,9 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
   // Up to 32 lists are one batch of the distance kernel whichever of them are
   // candidates: all are, without a limit. Up to 128, one warp bisects over the
   // row, four values a lane, without the block's barriers.
-  // (BF16, D 96, nprobe 6, 10000 queries: 16 lists 79 us, 128 lists 114 us; the
-  // radix select this kernel had before 144 and 147 us.) Beyond, the block's
-  // barriers cost more than that radix select did up to some 2000 lists: 160
-  // lists 179 and 149 us, 900 lists 197 and 196 us; from 8192 on they cost less.
+  // (Whole coarse stage, BF16, D 96, nprobe 6, 10000 queries: 16 lists 79 us, 128
+  // lists 112 us; by the radix select 144 and 147 us.) Rows of 129 to kRadixLists
+  // lists go to rerank_radix_kernel.
   float X = INFINITY;
   uint32_t hi = 0x7F800000u;
   if (nl > 32 && nl <= 128) {
@@ -666,43 +770,102 @@ __global__ void __launch_bounds__(kRThreads, 3) rerank_select_kernel(RerankArgs 
     if (!(v > X)) cand[atomicAdd(&total, 1)] = l;
   });
   __syncthreads();
-  const int nc_all = total;
-  if (threadIdx.x == 0 && a.ncand) a.ncand[q] = nc_all;
-  if (nc_all <= kCap) {
-    for (int i = threadIdx.x; i < nc_all; i += kRThreads) sp.cbuf[q * kCap + i] = cand[i];
-    const int nb = (nc_all + 31) >> 5;
-    if (threadIdx.x == 0) sh[0] = (uint32_t)atomicAdd(sp.nitems, nb);
-    __syncthreads();
-    if (threadIdx.x < nb) sp.items[sh[0] + threadIdx.x] = make_int2((int)q, threadIdx.x);
+  rerank_candidates<R, V4>(a, sp, q, np, cand, total, qs, tiles, sh);
+}
+
+// The same selection for rows of 129 to kRadixLists lists: every list's upper key
+// and lower bound in shared memory, T by a radix select, whose three or four
+// passes of two barriers cost less there than the bisection's some twenty
+// barriers, at any number of queries. (Whole coarse stage, BF16, D 96, 10000
+// queries, nprobe 48, this kernel / the bisection: 160 lists 196 / 246 us, 512
+// lists 217 / 260, 900 lists 250 / 277, 1500 lists 272 / 307, 2048 lists 301 /
+// 323, 3000 lists 375 / 348, 8192 lists 626 / 478.)
+// A: eps, the key of D~ + eps and the lower bound D~ - eps of every list, and
+//    the keys' range.
+// B: T >= the np-th smallest key, within 255 units of the last place
+//    (block_select).
+// C: the candidates, D~ - eps <= T, appended to a block-wide list.
+// Dynamic shared memory: qs [dim rounded up to 4] | keys [nlist rounded up to
+// 4] (then the candidate list) | lower [nlist], whose space then holds the
+// warps' staging tiles [8][1056].
+template <int R, bool V4>
+__global__ void __launch_bounds__(kRThreads, 3) rerank_radix_kernel(RerankArgs a, RerankSplit sp) {
+  __shared__ int hist[256];
+  __shared__ uint32_t sh[2];
+  __shared__ int total;
+  __shared__ uint32_t kr[2][kRWarps];
+  const int dq = (a.dim + 3) & ~3;
+  const int64_t nl4 = (a.nlist + 3) & ~3;
+  float* qs = (float*)anns_dyn_smem;
+  uint32_t* keys = (uint32_t*)(qs + dq);
+  float* lower = (float*)(keys + nl4);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t q = blockIdx.x, nlist = a.nlist;
+  const int np = a.npq ? min(max(a.npq[q], 0), a.nprobe) : a.nprobe;
+  if (np == 0) {
+    WarpTopK<R, int32_t> top;
+    top.init();
+    if (warp == 0) write_probes<R>(a, q, 0, top);
+    if (threadIdx.x == 0 && a.ncand) a.ncand[q] = 0;
     return;
   }
-  // C, in the block: the query itself and the staging tiles
-  for (int d = threadIdx.x; d < dq; d += kRThreads) qs[d] = d < a.dim ? a.Q[q * a.dim + d] : 0.f;
-  __syncthreads();
-  float thd = INFINITY;
-  int32_t thi = INT32_MAX;
-  float* tile = tiles + warp * kRTile;
-  for (int b0 = warp * 32; b0 < nc_all; b0 += kRWarps * 32) {
-    const int nc = min(32, nc_all - b0);
-    const float dc = V4 ? batch_d2_v4(a.C, qs, a.dim, cand + b0, nc, tile)
-                        : batch_d2_any(a.C, qs, a.dim, cand + b0, nc, tile);
-    top.offer(lane < nc, dc, lane < nc ? cand[b0 + lane] : 0, np, thd, thi);
-  }
-  __syncthreads();  // tiles are free: they hold the warps' lists
-  float* md = tiles;
-  int32_t* mi = (int32_t*)(tiles + kRWarps * R * 32);
+  const float* row = a.dt + q * nlist;
+  const float qn = a.qrows[q], qd = a.qrows[a.nq + q];
+  if (threadIdx.x == 0) total = 0;
+  // eight lists per thread per round, all their loads issued before any use
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0;
+  for (int64_t b0 = threadIdx.x; b0 < nlist; b0 += 8 * kRThreads) {
+    float d[8], cn[8], cd[8];
 #pragma unroll
-  for (int r = 0; r < R; ++r) { md[(warp * R + r) * 32 + lane] = top.d[r]; mi[(warp * R + r) * 32 + lane] = top.id[r]; }
-  __syncthreads();
-  if (warp == 0) {
-    for (int w = 1; w < kRWarps; ++w)
+    for (int j = 0; j < 8; ++j) {
+      const int64_t l = b0 + j * kRThreads;
+      const bool in = l < nlist;
+      d[j] = in ? row[l] : 0.f;
+      cn[j] = in ? a.crows[l] : 0.f;
+      cd[j] = in ? a.crows[nlist + l] : 0.f;
+    }
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const float v = md[(w * R + r) * 32 + lane];
-        top.offer(v != INFINITY, v, mi[(w * R + r) * 32 + lane], np, thd, thi);
+    for (int j = 0; j < 8; ++j) {
+      const int64_t l = b0 + j * kRThreads;
+      if (l < nlist) {
+        const float b = rerank_bound(d[j], qn, qd, cn[j], cd[j], a.kef, a.kfp);
+        const uint32_t k = upper_key(d[j] + b);
+        keys[l] = k;
+        lower[l] = d[j] - b;
+        kmin = min(kmin, k);
+        kmax = max(kmax, k);
       }
-    write_probes<R>(a, q, np, top);
+    }
   }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    kmin = min(kmin, __shfl_xor_sync(kFull, kmin, o));
+    kmax = max(kmax, __shfl_xor_sync(kFull, kmax, o));
+  }
+  if (lane == 0) { kr[0][warp] = kmin; kr[1][warp] = kmax; }
+  __syncthreads();
+  kmin = 0xFFFFFFFFu;
+  kmax = 0;
+  for (int w = 0; w < kRWarps; ++w) {
+    kmin = min(kmin, kr[0][w]);
+    kmax = max(kmax, kr[1][w]);
+  }
+  const float T = __uint_as_float(block_select(keys, nlist, np, kmin, kmax, hist, sh));
+  __syncthreads();  // keys are free: they become the candidate list
+  int32_t* cand = (int32_t*)keys;
+  for (int64_t b0 = (int64_t)warp * 32; b0 < nlist; b0 += kRThreads) {
+    const int64_t l = b0 + lane;
+    const bool c = l < nlist && !(lower[l] > T);
+    const unsigned m = __ballot_sync(kFull, c);
+    if (m) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&total, __popc(m));
+      at = __shfl_sync(kFull, at, 0);
+      if (c) cand[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)l;
+    }
+  }
+  __syncthreads();
+  rerank_candidates<R, V4>(a, sp, q, np, cand, total, qs, lower, sh);
 }
 
 constexpr int kDWarps = 4;  // warps per block of the distance kernel
@@ -886,6 +1049,8 @@ int fmt_elem(int prec) { return prec == ANNS_PREC_FP8E4M3 ? 1 : 2; }
 // Dynamic shared memory of the select kernel for this index: qs | the
 // candidate list | tiles, and D~ where it does not fit in registers.
 constexpr int kRegLists = 32 * kRThreads;
+constexpr int kRadixLists = 2048;  // rows up to here, beyond 128 lists: rerank_radix_kernel
+static_assert(kRadixLists <= kRWarps * kRTile, "its lower bounds lie in the tiles' space");
 size_t rerank_smem(const Index& ix) {
   const size_t nl4 = (size_t)((ix.nlist + 3) & ~3);
   const size_t tiles = (size_t)kRWarps * kRTile * 4;
@@ -1063,8 +1228,11 @@ cudaError_t launch_coarse_tc(const Index& ix, int prec, const float* Q, int64_t 
           return v4 ? run(rerank_select_kernel<RR, true, V>, g, kRThreads, smem, a, sp)
                     : run(rerank_select_kernel<RR, false, V>, g, kRThreads, smem, a, sp);
         };
+        if (ix.nlist > 128 && ix.nlist <= kRadixLists)
+          return v4 ? run(rerank_radix_kernel<RR, true>, g, kRThreads, smem, a, sp)
+                    : run(rerank_radix_kernel<RR, false>, g, kRThreads, smem, a, sp);
         const int64_t per = (ix.nlist + kRThreads - 1) / kRThreads;
-        return per <= 4    ? sel(std::integral_constant<int, 4>{})
+        return per <= 1    ? sel(std::integral_constant<int, 1>{})
                : per <= 16 ? sel(std::integral_constant<int, 16>{})
                : per <= 32 ? sel(std::integral_constant<int, 32>{})
                            : sel(std::integral_constant<int, 0>{});
