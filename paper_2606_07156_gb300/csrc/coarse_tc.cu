@@ -237,13 +237,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) coarse_tc_kernel(
     if (!ok) {
       *abort_flag = 1;
       atomicExch(status, ANNS_DEV_TIMEOUT);
-      // let the copies already issued land before the CTA exits (long limit):
-      // stage st received ceil((g - st) / S) copies, the last completing the
-      // phase of parity (count - 1) & 1, and no copy follows it
-      for (int st = 0; st < kStages; ++st) {
-        const int64_t count = g > st ? (g - st + kStages - 1) / kStages : 0;
-        if (count > 0) mbar_wait(full0 + 8 * st, (uint32_t)((count - 1) & 1));
-      }
+    }
+    // Every copy issued lands before the CTA exits (long limit), also where this
+    // thread issued all of them and another role gave up on one still in flight:
+    // stage st received ceil((g - st) / S) copies, the last completing the phase
+    // of parity (count - 1) & 1, and no copy follows it.
+    for (int st = 0; st < kStages; ++st) {
+      const int64_t count = g > st ? (g - st + kStages - 1) / kStages : 0;
+      if (count > 0) mbar_wait(full0 + 8 * st, (uint32_t)((count - 1) & 1));
     }
   } else if (tid == 32) {
     // MMA issuer: tile i of this CTA accumulates into TMEM columns (i & 1) * 256

@@ -478,18 +478,19 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
       it = nx;
       nx = n2;
     }
-    if (!ok) {
-      if (lane == 0) {
+    if (lane == 0) {
+      if (!ok) {
         *abort_flag = 1;
         atomicExch(a.status, ANNS_DEV_TIMEOUT);
-        // the copies already issued land before the CTA exits (coarse_tc.cu)
-        for (uint32_t st = 0; st < kFStages; ++st) {
-          const uint32_t count = g > st ? (g - st + kFStages - 1) / kFStages : 0;
-          if (count > 0) mbar_wait(full0 + 8 * st, (count - 1) & 1);
-        }
       }
-      __syncwarp();
+      // Every copy lands before the CTA exits, also where another role gave up
+      // after the last one was issued (coarse_tc.cu).
+      for (uint32_t st = 0; st < kFStages; ++st) {
+        const uint32_t count = g > st ? (g - st + kFStages - 1) / kFStages : 0;
+        if (count > 0) mbar_wait(full0 + 8 * st, (count - 1) & 1);
+      }
     }
+    __syncwarp();
   } else if (tid == 32) {
     // MMA issuer: this CTA's n-th item accumulates into TMEM columns (n & 1) * 256 + 128 * half
     uint32_t g = 0;
