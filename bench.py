@@ -484,6 +484,14 @@ def subspace_sweep(amp, index, W, cfg, nprobe: int, k: int, dev, nq: int = 2000)
 STAGES_CL = ("cl_distances", "cl_select (the whole tensor-core CL)", "precision_choice+query_tables")
 
 
+def stage_kernel(tuned, filtered: bool):
+    """Which search search_stages names: the filtered one where it ran (whatever
+    option led to it), else the autotuner's choice (`tuned`, None: no trial)."""
+    if filtered:
+        return "automatic"
+    return {"split": "split", "split_scan": "split", "automatic": None}.get(tuned, tuned)
+
+
 def search_stages(kernel, st_ms, bits: np.ndarray, pb: np.ndarray, row_bytes: int = 0):
     """Names of the profile stages (anns_profile) for the search that ran, and
     the candidates for the roofline's dominant kernel: (label, source file, ms
@@ -649,7 +657,8 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
     # picks on this batch (kernel, query order, grouped work-order chunk);
     # the others in the automatic one
     KN = {abi.KERNEL_BASIC: "query-major", abi.KERNEL_LIST_MAJOR: "list-major", abi.KERNEL_GROUPED: "grouped",
-          abi.KERNEL_SPLIT: "split", abi.KERNEL_AUTO: "automatic"}
+          abi.KERNEL_SPLIT: "split", abi.KERNEL_SPLIT_SCAN: "split_scan",
+          abi.KERNEL_FILTERED: "filtered", abi.KERNEL_AUTO: "automatic"}
     SN = {abi.SCHED_AUTO: "automatic", abi.SCHED_NATURAL: "natural", abi.SCHED_LPT: "longest-first"}
     tuned = None
     if not args.no_autotune:
@@ -702,6 +711,7 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
     # stage view of the adaptive step (the last search before the taps below)
     probes_ad = index.tap(abi.TAP_PROBES, (nq, nprobe), np.int32)
     bits_ad = index.tap(abi.TAP_BITS, (nq, nprobe), np.uint8)
+    filtered_ad = bool(index.tap(abi.TAP_FILTERED, (1,), np.int32)[0])
     ms_pol = {"mlp": ms_ad}
     for name, pol in policies.items():
         if name != "mlp":
@@ -788,7 +798,7 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
     # roofline of the dominant kernel of the adaptive step (search_stages)
     pb = pair_bytes(index, probes_ad, cfg["M"])
     st_ms = [v / max(cnt, 1) for v in stage_ms]
-    stage_names, cands = search_stages(tuned["kernel"] if tuned is not None else None, st_ms, bits_ad, pb,
+    stage_names, cands = search_stages(stage_kernel(tuned["kernel"] if tuned is not None else None, filtered_ad), st_ms, bits_ad, pb,
                                        int(W["codes"].shape[0]) * cfg["dim"] * 2)
     kname, kfile, kms, nbytes = max(cands, key=lambda c: c[2])
     peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
@@ -978,9 +988,9 @@ def run_uneven(args, rank: int, world: int, local_rank: int):
             ids, dists = run(pol)
             full[name] = (ids, dists)
             mix = bits_mix(index, abi, nq, NP, npq)
-            # the automatic kernel (grouped for the adaptive policies) and, for
-            # them, the split query-major search, each under both query orders
-            for kern in (("auto", "split") if name != "plain" else ("auto",)):
+            # the automatic kernel (filtered or grouped for the adaptive policies) and,
+            # for them, the split query-major search, each under both query orders
+            for kern in (("auto", "split_scan") if name != "plain" else ("auto",)):
                 index.set_kernel(kern)
                 for sched in ("natural", "lpt"):
                     index.set_schedule(sched)

@@ -274,6 +274,7 @@ int anns_get_info(const anns_index* index, anns_index_info* out);
  *   COARSE_APPROX     float [nq * nlist] tensor-core distances D~ (last
  *                     search with cl_prec = BF16, FP16 or FP8E4M3)
  *   COARSE_CANDIDATES int32 [nq] lists re-ranked in FP32 per query (same)
+ *   FILTERED int32: 1 = the search went through the filter, 0 = it scanned
  * Index taps:
  *   LIST_SIZES int64 [nlist], LIST_RADIUS float [nlist],
  *   PACKED_IDS int64 [n] (ids in list order, lists ascending),
@@ -282,7 +283,8 @@ int anns_get_info(const anns_index* index, anns_index_info* out);
 enum {
   ANNS_TAP_PROBES = 0, ANNS_TAP_PROBE_D2 = 1, ANNS_TAP_BITS = 2, ANNS_TAP_FEATURES = 3,
   ANNS_TAP_COARSE_APPROX = 4, ANNS_TAP_COARSE_CANDIDATES = 5,
-  ANNS_TAP_LIST_SIZES = 10, ANNS_TAP_LIST_RADIUS = 11, ANNS_TAP_PACKED_IDS = 12, ANNS_TAP_STATUS = 13
+  ANNS_TAP_LIST_SIZES = 10, ANNS_TAP_LIST_RADIUS = 11, ANNS_TAP_PACKED_IDS = 12, ANNS_TAP_STATUS = 13,
+  ANNS_TAP_FILTERED = 14
 };
 int anns_debug_tap(anns_index* index, int32_t what, void* out, size_t bytes);
 
@@ -384,6 +386,10 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
  *      1..8-bit pairs with byte tables only (no FP32 table in shared memory,
  *      so more blocks per SM), bounded by and merged with the partial. Large
  *      batches are filtered first, as with ANNS_KERNEL_AUTO.
+ *    ANNS_KERNEL_SPLIT_SCAN: the split search by itself, never filtered.
+ *    ANNS_KERNEL_FILTERED: filtered whatever the size of the batch; as
+ *      ANNS_KERNEL_AUTO where the filter cannot serve it (fixed 4-bit tables,
+ *      no decoded vectors, workspace too large).
  *  ANNS_OPT_SCHEDULE: the order in which the query-major kernel takes queries
  *    (the greedy load scheduling of Section 4.3, applied to queries).
  *    ANNS_SCHED_AUTO (default): longest first when nprobe_per_q is given (an
@@ -414,7 +420,7 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
 enum { ANNS_OPT_KERNEL = 0, ANNS_OPT_SCHEDULE = 1, ANNS_OPT_QCHUNK = 2, ANNS_OPT_WAIT_CYCLES = 3,
        ANNS_OPT_NIBBLE = 4 };
 enum { ANNS_KERNEL_AUTO = 0, ANNS_KERNEL_BASIC = 1, ANNS_KERNEL_LIST_MAJOR = 2, ANNS_KERNEL_GROUPED = 3,
-       ANNS_KERNEL_SPLIT = 4 };
+       ANNS_KERNEL_SPLIT = 4, ANNS_KERNEL_SPLIT_SCAN = 5, ANNS_KERNEL_FILTERED = 6 };
 enum { ANNS_SCHED_AUTO = 0, ANNS_SCHED_NATURAL = 1, ANNS_SCHED_LPT = 2 };
 int anns_set_option(anns_index* index, int32_t option, int64_t value);
 
@@ -438,7 +444,9 @@ void anns_graph_free(anns_graph* graph);
 /* Autotuner: times every available configuration on the given batch (reps
  * timed searches each, after one untimed): the automatic choice (filtered for
  * a large batch), the query-major kernel in query order and longest first, the
- * split search in both, the list-major kernel, and the grouped kernel in
+ * split search in both (as ANNS_KERNEL_SPLIT_SCAN where ANNS_KERNEL_SPLIT would
+ * be filtered), the filtered search where it can serve the batch and the
+ * automatic choice is another, the list-major kernel, and the grouped kernel in
  * both query orders with its automatic work order and with query chunks of
  * a half and a quarter of the batch (when >= 256 queries). Installs the
  * fastest as the index's options and reports all of them (at most cap, in

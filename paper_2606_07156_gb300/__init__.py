@@ -217,10 +217,13 @@ class Index:
 
     def set_kernel(self, which: str):
         """'auto', 'basic' (query-major), 'lists' (list-major, one warp per pair),
-        'grouped' (narrow pairs packed four or eight queries to a gather) or 'split'
-        (query-major in two passes: wide pairs, then 1..8-bit pairs on byte tables only)."""
+        'grouped' (narrow pairs packed four or eight queries to a gather), 'split'
+        (query-major in two passes: wide pairs, then 1..8-bit pairs on byte tables only;
+        large batches filtered first, as with 'auto'), 'split_scan' (the same, never
+        filtered) or 'filtered' (through the filter whatever the batch's size)."""
         v = {"auto": abi.KERNEL_AUTO, "basic": abi.KERNEL_BASIC, "lists": abi.KERNEL_LIST_MAJOR,
-             "grouped": abi.KERNEL_GROUPED, "split": abi.KERNEL_SPLIT}[which]
+             "grouped": abi.KERNEL_GROUPED, "split": abi.KERNEL_SPLIT,
+             "split_scan": abi.KERNEL_SPLIT_SCAN, "filtered": abi.KERNEL_FILTERED}[which]
         abi.anns_set_option(self.handle, abi.OPT_KERNEL, v)
 
     def locate(self, queries, nprobe: int, cl: str = "fp32", nprobe_per_q=None, stream=None):

@@ -354,10 +354,14 @@ PolicyArgs policy_args(const Index& ix, const anns_precision_policy& pol, int64_
   return p;
 }
 
+// The scanning search is chosen by the library's rules (for ANNS_KERNEL_FILTERED:
+// where the filter cannot serve the batch).
+bool automatic(const Index& ix) { return ix.opt_kernel == ANNS_KERNEL_AUTO || ix.opt_kernel == ANNS_KERNEL_FILTERED; }
+
 // One launch for a few queries on an index whose centroids a block reads in
 // about a microsecond (half a megabyte).
 bool front_fits(const Index& ix, const anns_precision_policy& P, int64_t nq) {
-  return ix.opt_kernel == ANNS_KERNEL_AUTO && P.cl_prec == ANNS_PREC_FP32 && P.lut_mode != ANNS_LUT_SVR && nq <= 64 &&
+  return automatic(ix) && P.cl_prec == ANNS_PREC_FP32 && P.lut_mode != ANNS_LUT_SVR && nq <= 64 &&
          ix.nlist <= 2048 && ix.nlist * ix.dim <= 131072 && ix.dim <= 4096;
 }
 
@@ -458,7 +462,7 @@ static int coarse_route(const Index& ix, int cl_prec, int64_t nq) {
 // widths: 285 us grouped, 140 us so)
 static bool small_mixed(const Index& ix, int64_t nq, int nprobe) {
   const double pair_us = (double)ix.Mp * (256.0 + (double)ix.n / (double)ix.nlist) / 6500.0;
-  return ix.opt_kernel == ANNS_KERNEL_AUTO && ix.opt_schedule == ANNS_SCHED_AUTO && search_split(nq, nprobe, 1) > 1 &&
+  return automatic(ix) && ix.opt_schedule == ANNS_SCHED_AUTO && search_split(nq, nprobe, 1) > 1 &&
          std::ceil((double)nq * nprobe / 304.0) * pair_us < 120.0;
 }
 
@@ -467,7 +471,7 @@ static bool small_mixed(const Index& ix, int64_t nq, int nprobe) {
 // batch is large enough for groups.
 static bool use_grouped(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
   if (ix.opt_kernel == ANNS_KERNEL_GROUPED) return grouped_supported(ix, k);
-  if (ix.opt_kernel != ANNS_KERNEL_AUTO || small_mixed(ix, nq, nprobe)) return false;
+  if (!automatic(ix) || small_mixed(ix, nq, nprobe)) return false;
   const bool narrow_possible = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
                                P.lut_mode == ANNS_LUT_EXPLICIT || P.lut_mode == ANNS_LUT_SVR ||
                                (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8);
@@ -498,11 +502,11 @@ static bool nibble_possible(const anns_precision_policy& P) {
 // Blocks per query of the automatic query-major search (all queries of such a
 // batch run at once: their order does not matter).
 static int split_of(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
-  return ix.opt_kernel == ANNS_KERNEL_AUTO && ix.opt_schedule == ANNS_SCHED_AUTO && !use_grouped(ix, P, nq, nprobe, k)
+  return automatic(ix) && ix.opt_schedule == ANNS_SCHED_AUTO && !use_grouped(ix, P, nq, nprobe, k)
              ? search_split(nq, nprobe, k) : 1;
 }
 
-static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven) {
+bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven) {
   return filter_supported(ix, P, nq, nprobe, k, use_grouped(ix, P, nq, nprobe, k), uneven) && (!nibble_possible(P) || grouped_supported(ix, k));
 }
 
@@ -510,6 +514,10 @@ static bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t 
 // tables, and for the 5..8-bit pairs of the queries it does not settle.
 static bool grouped_after_filter(const Index& ix, const anns_precision_policy& P, int k) {
   return (nibble_possible(P) || (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8)) && grouped_supported(ix, k);
+}
+
+static bool split_search(const Index& ix) {
+  return ix.opt_kernel == ANNS_KERNEL_SPLIT || ix.opt_kernel == ANNS_KERNEL_SPLIT_SCAN;
 }
 
 static bool use_lpt(const Index& ix, const int32_t* nprobe_per_q) {
@@ -547,7 +555,7 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
       const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
       if ((rc = list_workspace(ix, nq, nprobe, k, w, qchunk))) return rc;
     }
-    if (use_grouped(ix, P, nq, nprobe, k) || ix.opt_kernel == ANNS_KERNEL_SPLIT) {
+    if (use_grouped(ix, P, nq, nprobe, k) || split_search(ix)) {
       if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
     }
     const int split = split_of(ix, P, nq, nprobe, k);
@@ -578,6 +586,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
   const bool want_feat = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
                          P.lut_mode == ANNS_LUT_SVR;
   const bool filter = use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  ix.last_filtered = filter;
   const bool front = !filter && front_fits(ix, P, nq);
   if (front) {
     e = launch_front(ix, P, Q, nq, nprobe, nprobe_per_q, want_feat ? ix.ws_feat : nullptr, s);
@@ -678,7 +687,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
       order = lpt_order_ptr(ix.ws_sched, nq);
     }
     if (ev) cudaEventRecord(ev[3], s);
-    if (ix.opt_kernel == ANNS_KERNEL_SPLIT) {
+    if (split_search(ix)) {
       // wide pairs (FP32, 12/16 bits) into a partial top-k per query, then
       // the 1..8-bit pairs with byte tables only, merged with it
       float* part_d = (float*)ix.ws_grp;
@@ -926,7 +935,7 @@ extern "C" int anns_set_option(anns_index* ix, int32_t option, int64_t value) {
   if (!ix) return fail(ANNS_ERR_INVALID_ARG, "null index");
   switch (option) {
     case ANNS_OPT_KERNEL:
-      if (value < ANNS_KERNEL_AUTO || value > ANNS_KERNEL_SPLIT)
+      if (value < ANNS_KERNEL_AUTO || value > ANNS_KERNEL_FILTERED)
         return fail(ANNS_ERR_INVALID_ARG, "unknown kernel choice");
       ix->opt_kernel = (int)value;
       return ANNS_OK;

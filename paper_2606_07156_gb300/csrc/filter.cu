@@ -1731,7 +1731,9 @@ void free_filter(Index& ix) {
 
 bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
                       bool grouped_otherwise, bool uneven) {
-  if (ix.fl_w == 0 || (ix.opt_kernel != ANNS_KERNEL_AUTO && ix.opt_kernel != ANNS_KERNEL_SPLIT)) return false;
+  if (ix.fl_w == 0 || (ix.opt_kernel != ANNS_KERNEL_AUTO && ix.opt_kernel != ANNS_KERNEL_SPLIT &&
+                       ix.opt_kernel != ANNS_KERNEL_FILTERED))
+    return false;
   if (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits < 5) return false;  // every pair would be scanned anyway
   const int64_t pairs = nq * nprobe;
   // Small searches are over before the filter's fifteen launches (100 us; 250 us
@@ -1749,7 +1751,8 @@ bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t n
                          (256.0 + (double)ix.n / (double)ix.nlist) / 2000.0 * std::max(1.0, (double)nq * split / 400.0) +
                          (k > 32 ? 60.0 + 8.0 * probes : 0.0);
   const double lookups = probes * (double)nq * (double)ix.Mp * ((double)ix.n / (double)ix.nlist + 512.0);
-  if (grouped_otherwise ? lookups < (k > 32 ? 2e7 : 2e9) : scan_us < 100.0) return false;
+  if (ix.opt_kernel == ANNS_KERNEL_FILTERED) {  // whatever the batch
+  } else if (grouped_otherwise ? lookups < (k > 32 ? 2e7 : 2e9) : scan_us < 100.0) return false;
   const int64_t tiles = (ix.max_list + kTv - 1) / kTv;
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))

@@ -35,6 +35,7 @@ void make_shadow(const Index& ix, Index& sh) {
   sh.ws_sched = nullptr; sh.ws_tc = nullptr; sh.st_q = nullptr; sh.st_out = nullptr; sh.st_pq = nullptr;
   sh.ws_tc_cap = 0;
   sh.ws_tc_valid = false;
+  sh.last_filtered = false;
   sh.ws_fl = nullptr;
   sh.ws_fl_cap = 0;
   sh.ws_grp = nullptr;
@@ -148,9 +149,20 @@ extern "C" int anns_autotune(anns_index* ix, const float* Q, int64_t nq, int32_t
   const int64_t qchunk0 = ix->opt_qchunk;
   struct Cand { int kernel, schedule; int64_t qchunk; };
   std::vector<Cand> cands = {{ANNS_KERNEL_AUTO, ANNS_SCHED_AUTO, 0},  // the filtered search, where it serves the call
-                             {ANNS_KERNEL_BASIC, ANNS_SCHED_NATURAL, 0}, {ANNS_KERNEL_BASIC, ANNS_SCHED_LPT, 0},
-                             {ANNS_KERNEL_SPLIT, ANNS_SCHED_NATURAL, 0}, {ANNS_KERNEL_SPLIT, ANNS_SCHED_LPT, 0},
-                             {ANNS_KERNEL_LIST_MAJOR, ANNS_SCHED_NATURAL, 0}};
+                             {ANNS_KERNEL_BASIC, ANNS_SCHED_NATURAL, 0}, {ANNS_KERNEL_BASIC, ANNS_SCHED_LPT, 0}};
+  // the filtered search once, and the split search itself
+  ix->opt_kernel = ANNS_KERNEL_AUTO;
+  ix->opt_schedule = ANNS_SCHED_AUTO;
+  const bool auto_filtered = use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  ix->opt_kernel = ANNS_KERNEL_SPLIT;
+  const bool split_filtered = use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  const int split = split_filtered ? ANNS_KERNEL_SPLIT_SCAN : ANNS_KERNEL_SPLIT;
+  ix->opt_kernel = ANNS_KERNEL_FILTERED;
+  if (!auto_filtered && use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr))
+    cands.push_back({ANNS_KERNEL_FILTERED, ANNS_SCHED_AUTO, 0});
+  cands.push_back({split, ANNS_SCHED_NATURAL, 0});
+  cands.push_back({split, ANNS_SCHED_LPT, 0});
+  cands.push_back({ANNS_KERNEL_LIST_MAJOR, ANNS_SCHED_NATURAL, 0});
   // the grouped kernel under both query orders, with its automatic work order
   // and with query chunks of a half and a quarter of the batch (at least 256)
   std::vector<int64_t> chunks = {0};

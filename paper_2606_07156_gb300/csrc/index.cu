@@ -354,6 +354,10 @@ extern "C" int anns_debug_tap(anns_index* ix, int32_t what, void* out, size_t by
       need = (size_t)ix->ws_tc_nq * 4;
       break;
     }
+    case ANNS_TAP_FILTERED:
+      if (bytes < 4) return fail(ANNS_ERR_INVALID_ARG, "tap buffer too small");
+      *(int32_t*)out = ix->last_filtered ? 1 : 0;
+      return ANNS_OK;
     case ANNS_TAP_STATUS: {
       if (bytes < 4) return fail(ANNS_ERR_INVALID_ARG, "tap buffer too small");
       int v = 0;

@@ -66,6 +66,7 @@ struct Index {
   float fl_yscale = 1.f, fl_mu = 0.f;  // 1 / scale of the rows, |mu|
   size_t fl_ws_limit = (size_t)32 << 30;  // workspace the filter may take (lowered where there was no room)
   int64_t fl_tiles = 0;                // sum over the lists of their 256-vector tiles
+  bool last_filtered = false;          // the last search went through the filter
   // host copies of the small per-list tables
   std::string err;
   int64_t* h_list_len64 = nullptr;
@@ -206,6 +207,8 @@ cudaError_t launch_lpt_order(const Index& ix, const int32_t* probes, const int32
 int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int32_t* nprobe_per_q, int k,
                     const int32_t* k_per_q, const anns_precision_policy& P, int64_t* ids_out,
                     float* dists_out, cudaStream_t s, bool profile);
+// Whether a search with these options goes through the filter.
+bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven);
 // Grows every workspace buffer a search of this shape needs.
 int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
                    const int32_t* nprobe_per_q);
