@@ -362,16 +362,18 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
 
 /* Index options.
  *  ANNS_OPT_KERNEL: which search kernel anns_search launches.
- *    ANNS_KERNEL_AUTO (default): filtered when the batch is large enough: a
+ *    ANNS_KERNEL_AUTO (default): the search estimated to be the fastest for the
+ *      shape of the batch and the index: grouped when the policy can choose tables
+ *      of at most 8 bits (k <= 128), else query-major; query-major with several
+ *      blocks a query for few queries; or filtered, mostly large batches: a
  *      tensor-core GEMM of the lists' decoded vectors (held in FP16, 2 * dim
  *      bytes a vector, where that is at most a quarter of the free device
  *      memory when the index is built) with the queries bounds every distance,
  *      and only the vectors that can reach a query's top-k are evaluated by the
  *      exact rules; pairs on tables of at most 4 bits with such vectors, and
- *      queries with too many, are scanned by the kernels below. Else grouped
- *      when the policy can choose tables of at most 8 bits (k <= 128) and the
- *      batch is not very small, else query-major (several blocks a query for a
- *      few queries).
+ *      queries with too many, are scanned by the kernels below. (Of an uneven
+ *      batch the mean of nprobe_per_q counts where it is in host memory, else a
+ *      sixth of nprobe is assumed.)
  *    ANNS_KERNEL_BASIC: query-major, one block per query walking its probes.
  *    ANNS_KERNEL_GROUPED: the pairs on 1..8-bit tables taken four per list,
  *      their byte tables interleaved so that one shared-memory gather serves
@@ -384,8 +386,8 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
  *    ANNS_KERNEL_SPLIT: query-major in two passes split by table width: the
  *      FP32 and 12/16-bit pairs into a per-query partial top-k, then the
  *      1..8-bit pairs with byte tables only (no FP32 table in shared memory,
- *      so more blocks per SM), bounded by and merged with the partial. Large
- *      batches are filtered first, as with ANNS_KERNEL_AUTO.
+ *      so more blocks per SM), bounded by and merged with the partial.
+ *      Filtered where that is estimated to be faster.
  *    ANNS_KERNEL_SPLIT_SCAN: the split search by itself, never filtered.
  *    ANNS_KERNEL_FILTERED: filtered whatever the size of the batch; as
  *      ANNS_KERNEL_AUTO where the filter cannot serve it (fixed 4-bit tables,

@@ -219,7 +219,7 @@ class Index:
         """'auto', 'basic' (query-major), 'lists' (list-major, one warp per pair),
         'grouped' (narrow pairs packed four or eight queries to a gather), 'split'
         (query-major in two passes: wide pairs, then 1..8-bit pairs on byte tables only;
-        large batches filtered first, as with 'auto'), 'split_scan' (the same, never
+        filtered where that is estimated to be faster), 'split_scan' (the same, never
         filtered) or 'filtered' (through the filter whatever the batch's size)."""
         v = {"auto": abi.KERNEL_AUTO, "basic": abi.KERNEL_BASIC, "lists": abi.KERNEL_LIST_MAJOR,
              "grouped": abi.KERNEL_GROUPED, "split": abi.KERNEL_SPLIT,

@@ -454,30 +454,6 @@ static int coarse_route(const Index& ix, int cl_prec, int64_t nq) {
   return cl_prec == ANNS_PREC_FP32 && coarse_fp32_by_tc(ix, nq) ? ANNS_PREC_FP16 : cl_prec;
 }
 
-// A batch of few pairs whose policy the grouped kernels would serve, but that
-// the query-major kernel with several blocks a query finishes sooner: the pairs
-// form no groups, and the regrouping, two grouped kernels and merge are some
-// 200 us of latency. A block scans a pair in about Mp (256 + list) / 6500 us
-// with the GPU full (304 blocks). (16 queries, 32 lists of 2441, M = 48, mixed
-// widths: 285 us grouped, 140 us so)
-static bool small_mixed(const Index& ix, int64_t nq, int nprobe) {
-  const double pair_us = (double)ix.Mp * (256.0 + (double)ix.n / (double)ix.nlist) / 6500.0;
-  return automatic(ix) && ix.opt_schedule == ANNS_SCHED_AUTO && search_split(nq, nprobe, 1) > 1 &&
-         std::ceil((double)nq * nprobe / 304.0) * pair_us < 120.0;
-}
-
-// The grouped kernel (narrow pairs packed four to a word): on request, or by
-// default for a policy that can choose 1..8-bit tables, when k <= 128 and the
-// batch is large enough for groups.
-static bool use_grouped(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
-  if (ix.opt_kernel == ANNS_KERNEL_GROUPED) return grouped_supported(ix, k);
-  if (!automatic(ix) || small_mixed(ix, nq, nprobe)) return false;
-  const bool narrow_possible = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
-                               P.lut_mode == ANNS_LUT_EXPLICIT || P.lut_mode == ANNS_LUT_SVR ||
-                               (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits <= 8);
-  return narrow_possible && grouped_supported(ix, k);
-}
-
 // Whether every pair the policy can put outside 1..8 bits is an FP32 pair
 // (no 12- or 16-bit tables): the split search's wide pass then needs no
 // level table.
@@ -492,23 +468,18 @@ static bool wide_tables_fp32(const anns_precision_policy& P) {
   }
 }
 
-// Whether the policy can pick tables of at most 4 bits (the filter only marks
-// such pairs; the grouped kernels scan them).
-static bool nibble_possible(const anns_precision_policy& P) {
+// The policies whose tables are chosen pair by pair.
+bool nibble_possible(const anns_precision_policy& P) {
   return P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 || P.lut_mode == ANNS_LUT_EXPLICIT ||
          P.lut_mode == ANNS_LUT_SVR;
 }
 
-// Blocks per query of the automatic query-major search (all queries of such a
-// batch run at once: their order does not matter).
-static int split_of(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
-  return automatic(ix) && ix.opt_schedule == ANNS_SCHED_AUTO && !use_grouped(ix, P, nq, nprobe, k)
-             ? search_split(nq, nprobe, k) : 1;
-}
-
-bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven) {
-  return filter_supported(ix, P, nq, nprobe, k, use_grouped(ix, P, nq, nprobe, k), uneven) && (!nibble_possible(P) || grouped_supported(ix, k));
-}
+// Probes per query as far as the host knows. Counts on the device are not read:
+// uneven batches have many short probe sequences (Zipf-distributed counts up to
+// 64 or 128 a mean of a fifth to a seventh), so a sixth; a batch whose counts are
+// all near nprobe then keeps the base search (route.cu) until it is that much
+// larger. anns_search_host has the counts on the host and passes their mean.
+double mean_probes(int nprobe, const int32_t* nprobe_per_q) { return nprobe_per_q ? nprobe / 6.0 : nprobe; }
 
 // Whether the grouped kernels follow the filter: for the pairs on 1..4-bit
 // tables, and for the 5..8-bit pairs of the queries it does not settle.
@@ -533,11 +504,10 @@ static int reserve_filter(Index& ix, int64_t nq, int nprobe, int k, const anns_p
 }
 
 int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
-                   const int32_t* nprobe_per_q) {
+                   const int32_t* nprobe_per_q, Route& r) {
   int rc = ensure_workspace(ix, nq, nprobe);
   if (rc) return rc;
-  bool filter = use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
-  if (filter && (rc = reserve_filter(ix, nq, nprobe, k, P))) {
+  if (r.filter && (rc = reserve_filter(ix, nq, nprobe, k, P))) {
     if (rc != ANNS_ERR_OOM) return rc;
     // No room for the filter's workspace, which is larger than the scan's:
     // batches of this size scan from now on.
@@ -547,20 +517,19 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
     ix.ws_fl = nullptr;
     ix.ws_fl_cap = 0;
     ix.fl_ws_limit = filter_workspace_bytes(ix, nq, nprobe, k) - 1;
-    filter = false;
+    r.filter = false;
   }
-  if (!filter) {
-    if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || use_grouped(ix, P, nq, nprobe, k)) {
+  if (!r.filter) {
+    if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || r.grouped) {
       ListWork w{};
       const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
       if ((rc = list_workspace(ix, nq, nprobe, k, w, qchunk))) return rc;
     }
-    if (use_grouped(ix, P, nq, nprobe, k) || split_search(ix)) {
+    if (r.grouped || split_search(ix)) {
       if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k)))) return rc;
     }
-    const int split = split_of(ix, P, nq, nprobe, k);
-    if (split > 1) {
-      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq * split, k)))) return rc;
+    if (r.split > 1) {
+      if ((rc = grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq * r.split, k)))) return rc;
     } else if (ix.opt_kernel != ANNS_KERNEL_LIST_MAJOR && use_lpt(ix, nprobe_per_q)) {
       if ((rc = grow(&ix.ws_sched, &ix.ws_sched_cap, lpt_workspace_bytes(nq)))) return rc;
     }
@@ -573,8 +542,9 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
 
 int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int32_t* nprobe_per_q, int k,
                     const int32_t* k_per_q, const anns_precision_policy& P, int64_t* ids_out,
-                    float* dists_out, cudaStream_t s, bool profile) {
-  int rc = reserve_search(ix, nq, nprobe, k, P, nprobe_per_q);
+                    float* dists_out, cudaStream_t s, bool profile, double probes) {
+  Route route = route_of(ix, P, nq, nprobe, k, probes > 0.0 ? probes : mean_probes(nprobe, nprobe_per_q));
+  int rc = reserve_search(ix, nq, nprobe, k, P, nprobe_per_q, route);
   if (rc) return rc;
   cudaEvent_t* ev = profile ? next_profile_slot(ix) : nullptr;
   if (ev) cudaEventRecord(ev[0], s);
@@ -585,7 +555,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
   const int cl = coarse_route(ix, P.cl_prec, nq);
   const bool want_feat = P.lut_mode == ANNS_LUT_MLP || P.lut_mode == ANNS_LUT_HEURISTIC_EQ2 ||
                          P.lut_mode == ANNS_LUT_SVR;
-  const bool filter = use_filter(ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
+  const bool filter = route.filter;
   ix.last_filtered = filter;
   const bool front = !filter && front_fits(ix, P, nq);
   if (front) {
@@ -662,7 +632,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     if (ev) cudaEventRecord(ev[3], s);
     e = launch_search_lists(ix, ix.ws_qt, nq, nprobe, nprobe_per_q, k, k_per_q, ix.ws_probes, ix.ws_probe_d2,
                             ix.ws_bits, tbytes, w, ids_out, dists_out, s);
-  } else if (use_grouped(ix, P, nq, nprobe, k)) {
+  } else if (route.grouped) {
     ListWork w{};
     if ((rc = list_workspace(ix, nq, nprobe, k, w, grouped_qchunk(ix, nq)))) return rc;
     // longest-first order of the query-major pass, over the pairs it scans
@@ -679,7 +649,7 @@ int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int
     if (e == cudaSuccess && ev) cudaEventRecord(ev[7], s);
     return e == cudaSuccess ? ANNS_OK : cuda_fail(e, "search kernel");
   } else {
-    const int split = split_of(ix, P, nq, nprobe, k);
+    const int split = route.split;
     const int32_t* order = nullptr;
     if (split == 1 && use_lpt(ix, nprobe_per_q)) {
       e = launch_lpt_order(ix, ix.ws_probes, nprobe_per_q, nq, nprobe, ix.ws_sched, s, ix.ws_bits, false);
@@ -745,10 +715,10 @@ void free_workspace(Index& ix) {
 
 }  // namespace anns
 
-extern "C" int anns_search(anns_index* ix, const float* Q, int64_t nq, int32_t nprobe,
-                           const int32_t* nprobe_per_q, int32_t k, const int32_t* k_per_q,
-                           const anns_precision_policy* pol, int64_t* ids_out, float* dists_out,
-                           void* stream) {
+// probes: the mean of nprobe_per_q where the caller knows it, else 0.
+static int search(anns_index* ix, const float* Q, int64_t nq, int32_t nprobe, const int32_t* nprobe_per_q, int32_t k,
+                  const int32_t* k_per_q, const anns_precision_policy* pol, int64_t* ids_out, float* dists_out,
+                  void* stream, double probes) {
   int rc = check_search_args(ix, Q, nq, nprobe, k, pol, ids_out, dists_out);
   if (rc) return rc;
   if (nq == 0) return ANNS_OK;
@@ -756,7 +726,14 @@ extern "C" int anns_search(anns_index* ix, const float* Q, int64_t nq, int32_t n
   anns_precision_policy plain{};
   plain.lut_mode = ANNS_LUT_PLAIN_FP32;
   return search_sequence(*ix, Q, nq, nprobe, nprobe_per_q, k, k_per_q, pol ? *pol : plain, ids_out, dists_out,
-                         (cudaStream_t)stream, true);
+                         (cudaStream_t)stream, true, probes);
+}
+
+extern "C" int anns_search(anns_index* ix, const float* Q, int64_t nq, int32_t nprobe,
+                           const int32_t* nprobe_per_q, int32_t k, const int32_t* k_per_q,
+                           const anns_precision_policy* pol, int64_t* ids_out, float* dists_out,
+                           void* stream) {
+  return search(ix, Q, nq, nprobe, nprobe_per_q, k, k_per_q, pol, ids_out, dists_out, stream, 0.0);
 }
 
 extern "C" int anns_locate(anns_index* ix, const float* Q, int64_t nq, int32_t nprobe,
@@ -811,7 +788,12 @@ extern "C" int anns_search_host(anns_index* ix, const float* Q, int64_t nq, int3
   if (e == cudaSuccess && dnp) e = cudaMemcpyAsync(dnp, nprobe_per_q, nq * 4, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && dk) e = cudaMemcpyAsync(dk, k_per_q, nq * 4, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return cuda_fail(e, "copy queries in");
-  if ((rc = anns_search(ix, dq, nq, nprobe, dnp, k, dk, pol, di, dd, stream))) return rc;
+  double probes = 0.0;
+  if (nprobe_per_q) {
+    for (int64_t q = 0; q < nq; ++q) probes += std::min(std::max(nprobe_per_q[q], 0), nprobe);
+    probes = std::max(probes / (double)nq, 1e-3);
+  }
+  if ((rc = search(ix, dq, nq, nprobe, dnp, k, dk, pol, di, dd, stream, probes))) return rc;
   e = cudaMemcpyAsync(ids_out, di, (size_t)nq * k * 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dists_out, dd, (size_t)nq * k * 4, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

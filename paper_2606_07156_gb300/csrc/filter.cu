@@ -1729,31 +1729,11 @@ void free_filter(Index& ix) {
   ix.fl_w = 0;
 }
 
-bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
-                      bool grouped_otherwise, bool uneven) {
-  if (ix.fl_w == 0 || (ix.opt_kernel != ANNS_KERNEL_AUTO && ix.opt_kernel != ANNS_KERNEL_SPLIT &&
-                       ix.opt_kernel != ANNS_KERNEL_FILTERED))
-    return false;
+bool filter_possible(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
+  if (ix.fl_w == 0) return false;
   if (P.lut_mode == ANNS_LUT_FIXED_BITS && P.fixed_bits < 5) return false;  // every pair would be scanned anyway
-  const int64_t pairs = nq * nprobe;
-  // Small searches are over before the filter's fifteen launches (100 us; 250 us
-  // with the grouped kernels behind them) are. Query-major, a block scans a pair
-  // in about Mp (256 + list) / 2000 us, some 400 blocks at a time (777 queries,
-  // 19 lists of 150, M = 20, 12 bits: 530 us scanned, 200 us filtered), and
-  // lists of k > 32 entries add some 8 us a pair and 60 us for their merge (3
-  // queries, 27 lists of 692, M = 24, k = 128: 413 and 199 us). The grouped
-  // kernels take about 4.6e9 look-ups a millisecond (77 queries, 64 lists of
-  // 1094, M = 48: 304 us grouped, 364 us filtered), ten times less with k > 32
-  // (39 queries, 11 lists of 608, M = 64, k = 128: 1345 us).
-  const double probes = uneven ? nprobe / 6.0 : nprobe;  // their number per query is on the device
-  const int split = ix.opt_kernel == ANNS_KERNEL_AUTO ? search_split(nq, nprobe, k) : 1;
-  const double scan_us = std::max(1.0, probes / split) * (double)ix.Mp *
-                         (256.0 + (double)ix.n / (double)ix.nlist) / 2000.0 * std::max(1.0, (double)nq * split / 400.0) +
-                         (k > 32 ? 60.0 + 8.0 * probes : 0.0);
-  const double lookups = probes * (double)nq * (double)ix.Mp * ((double)ix.n / (double)ix.nlist + 512.0);
-  if (ix.opt_kernel == ANNS_KERNEL_FILTERED) {  // whatever the batch
-  } else if (grouped_otherwise ? lookups < (k > 32 ? 2e7 : 2e9) : scan_us < 100.0) return false;
-  const int64_t tiles = (ix.max_list + kTv - 1) / kTv;
+  if (nibble_possible(P) && !grouped_supported(ix, k)) return false;
+  const int64_t pairs = nq * nprobe, tiles = (ix.max_list + kTv - 1) / kTv;
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))
     return false;

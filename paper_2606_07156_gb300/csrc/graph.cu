@@ -151,15 +151,14 @@ extern "C" int anns_autotune(anns_index* ix, const float* Q, int64_t nq, int32_t
   std::vector<Cand> cands = {{ANNS_KERNEL_AUTO, ANNS_SCHED_AUTO, 0},  // the filtered search, where it serves the call
                              {ANNS_KERNEL_BASIC, ANNS_SCHED_NATURAL, 0}, {ANNS_KERNEL_BASIC, ANNS_SCHED_LPT, 0}};
   // the filtered search once, and the split search itself
-  ix->opt_kernel = ANNS_KERNEL_AUTO;
   ix->opt_schedule = ANNS_SCHED_AUTO;
-  const bool auto_filtered = use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
-  ix->opt_kernel = ANNS_KERNEL_SPLIT;
-  const bool split_filtered = use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr);
-  const int split = split_filtered ? ANNS_KERNEL_SPLIT_SCAN : ANNS_KERNEL_SPLIT;
-  ix->opt_kernel = ANNS_KERNEL_FILTERED;
-  if (!auto_filtered && use_filter(*ix, P, nq, nprobe, k, nprobe_per_q != nullptr))
+  auto filtered = [&](int kernel) {
+    ix->opt_kernel = kernel;
+    return route_of(*ix, P, nq, nprobe, k, mean_probes(nprobe, nprobe_per_q)).filter;
+  };
+  if (!filtered(ANNS_KERNEL_AUTO) && filtered(ANNS_KERNEL_FILTERED))
     cands.push_back({ANNS_KERNEL_FILTERED, ANNS_SCHED_AUTO, 0});
+  const int split = filtered(ANNS_KERNEL_SPLIT) ? ANNS_KERNEL_SPLIT_SCAN : ANNS_KERNEL_SPLIT;
   cands.push_back({split, ANNS_SCHED_NATURAL, 0});
   cands.push_back({split, ANNS_SCHED_LPT, 0});
   cands.push_back({ANNS_KERNEL_LIST_MAJOR, ANNS_SCHED_NATURAL, 0});

@@ -295,6 +295,7 @@ extern "C" int anns_build_index_from_arrays(const anns_build_desc* d, anns_index
   ix->h_radius = new float[nlist];
   std::vector<int32_t> len32(nlist);
   for (int64_t l = 0; l < nlist; ++l) {
+    if (n > 0) ix->list_seen += (double)cnt[l] * ((double)cnt[l] / (double)n);
     ix->h_list_len64[l] = cnt[l];
     len32[l] = (int32_t)cnt[l];
   }

@@ -33,6 +33,7 @@ struct Index {
   int device = 0;
   int64_t n = 0, dim = 0, nlist = 0, M = 0, dsub = 0, Mp = 0, nchunk = 0;
   int64_t ntiles = 0, max_list = 0;
+  double list_seen = 0.0;               // vectors of a probed list: sum n_l^2 / sum n_l
   bool ids32 = false;           // every id in [INT32_MIN, INT32_MAX): 32-bit ids in the 128-entry top-k lists
   float* centroids = nullptr;   // [nlist*dim]
   float* codebooks = nullptr;   // [M*256*dsub]
@@ -206,12 +207,16 @@ cudaError_t launch_lpt_order(const Index& ix, const int32_t* probes, const int32
 // whose workspace is already large enough when `no_alloc` is set.
 int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int32_t* nprobe_per_q, int k,
                     const int32_t* k_per_q, const anns_precision_policy& P, int64_t* ids_out,
-                    float* dists_out, cudaStream_t s, bool profile);
-// Whether a search with these options goes through the filter.
-bool use_filter(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, bool uneven);
+                    float* dists_out, cudaStream_t s, bool profile, double probes = 0.0);
+// The search that serves a batch (route.cu): filtered or not; where it is not, the
+// grouped kernels, else query-major with `split` blocks a query. `probes`: probes
+// per query on average.
+struct Route { bool filter = false, grouped = false; int split = 1; };
+Route route_of(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k, double probes);
+double mean_probes(int nprobe, const int32_t* nprobe_per_q);
 // Grows every workspace buffer a search of this shape needs.
 int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
-                   const int32_t* nprobe_per_q);
+                   const int32_t* nprobe_per_q, Route& r);
 // Frees the workspace buffers (not the index arrays).
 void free_workspace(Index& ix);
 
@@ -282,9 +287,11 @@ cudaError_t launch_scan_pairs(const Index& ix, const float* Q, const float* qt, 
 // Tensor-core filter in front of the exact rules (filter.cu).
 int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<float>& books);
 void free_filter(Index& ix);
-// Whether the filter serves the call; grouped_otherwise: the grouped kernels would.
-bool filter_supported(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k,
-                      bool grouped_otherwise, bool uneven);
+// Whether the filter can serve the call.
+bool filter_possible(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k);
+// Whether the policy can choose tables of at most 4 bits for some pairs (the
+// filter only marks such pairs; the grouped kernels scan them).
+bool nibble_possible(const anns_precision_policy& P);
 size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k);
 // What the filter leaves: queries for the scanning kernel (their number on the
 // device) and the pairs on tables of at most 4 bits that are worth a scan.

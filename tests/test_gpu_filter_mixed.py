@@ -1,5 +1,5 @@
 """The filtered search of mixed table widths with k <= 32, the learned policy's
-default on large batches: queries with FP32 survivors only settled by a warp, the
+way on large batches: queries with FP32 survivors only settled by a warp, the
 others by a block, 4-bit pairs (of every rank, the nearest among them) marked and
 scanned eight to a word under the filter's bound, and queries with more
 candidates than fit handed to the scan. Every call asserts that it was filtered
@@ -44,9 +44,9 @@ def pair(amp):
     g.close()
 
 
-def run(amp, g, o, Q, nprobe, k, pol, bits, kern, **kw):
+def run(amp, g, o, Q, nprobe, k, pol, bits, **kw):
     kwd = {f: cuda(v) for f, v in kw.items()}
-    g.set_kernel(kern)
+    g.set_kernel("filtered")
     try:
         i, d = g.search(cuda(Q), nprobe, k, pol, **kwd)
         assert g.tap(amp.abi.TAP_FILTERED, (1,), np.int32)[0] == 1
@@ -65,8 +65,8 @@ def run(amp, g, o, Q, nprobe, k, pol, bits, kern, **kw):
 
 
 @pytest.mark.parametrize("k", [1, 10, 32])
-@pytest.mark.parametrize("kern,uneven", [("auto", False), ("filtered", False), ("filtered", True)])
-def test_explicit_widths(amp, pair, k, kern, uneven):
+@pytest.mark.parametrize("uneven", [False, True])
+def test_explicit_widths(amp, pair, k, uneven):
     r, g, o = pair
     nq, nprobe = 4000, 40
     Q = (o.centroids[r.integers(0, NLIST, nq)] + 0.5 * r.standard_normal((nq, DIM))).astype(np.float32)
@@ -79,7 +79,7 @@ def test_explicit_widths(amp, pair, k, kern, uneven):
         kw = dict(nprobe_per_q=r.integers(0, nprobe + 1, nq).astype(np.int32),
                   k_per_q=r.integers(0, k + 1, nq).astype(np.int32))
         kw["nprobe_per_q"][:4] = nprobe
-    run(amp, g, o, Q, nprobe, k, amp.policy("explicit", pair_bits=cuda(bits)), bits, kern, **kw)
+    run(amp, g, o, Q, nprobe, k, amp.policy("explicit", pair_bits=cuda(bits)), bits, **kw)
 
 
 @pytest.mark.parametrize("k", [10, 32])
@@ -91,4 +91,4 @@ def test_learned_widths(amp, pair, k, width_map):
     p["inv_std"] = np.abs(p["inv_std"]) + 0.1
     g.set_predictor(p)
     Q = (o.centroids[r.integers(0, NLIST, nq)] + 0.5 * r.standard_normal((nq, DIM))).astype(np.float32)
-    run(amp, g, o, Q, nprobe, k, amp.policy("mlp", margin=0.1, width_map=width_map), None, "auto")
+    run(amp, g, o, Q, nprobe, k, amp.policy("mlp", margin=0.1, width_map=width_map), None)

@@ -47,8 +47,8 @@ def same(got, want, what=""):
 
 
 def test_split_search_by_itself(amp):
-    """A batch that 'split' filters: 'split_scan' runs the two passes, wide pairs
-    into a partial top-k and then the 1..8-bit pairs, with the same results."""
+    """'split_scan' runs the two passes, wide pairs into a partial top-k and then the
+    1..8-bit pairs, with the filtered search's results."""
     r, g, o = make(amp, 64, 16, 40, 30_000, 1)
     nq, nprobe = 1200, 20
     Q = queries(r, o, nq)
@@ -60,7 +60,7 @@ def test_split_search_by_itself(amp):
                 b = bits if np.isscalar(bits) else bits[:16]
                 ri, rd = ivfpq.search(o, Q[:16], nprobe, k, bits=b)
                 res = []
-                for kern, f in (("split", True), ("split_scan", False), ("basic", False)):
+                for kern, f in (("filtered", True), ("split_scan", False), ("basic", False)):
                     g.set_kernel(kern)
                     res.append(g.search(cuda(Q), nprobe, k, pol))
                     assert filtered(amp, g) == f, (kern, k)
