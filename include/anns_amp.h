@@ -417,10 +417,17 @@ int anns_sync_status(anns_index* index, void* cuda_stream);
  *    on tables of at most 4 bits are taken eight per list, their levels
  *    interleaved as nibbles so that one gather serves eight queries (the
  *    5..8-bit pairs stay four per word); 0 = all 1..8-bit pairs four per word.
+ *  ANNS_OPT_FILTER_BYTES: the most device memory in bytes that a filtered
+ *    search's workspace may take (default 2^35); a batch that needs more, or for
+ *    which an allocation fails, is scanned, that call only. 0 = no search is
+ *    filtered, and the decoded vectors are freed (graphs captured with them keep
+ *    them until they are freed themselves); a later value > 0 forms them again,
+ *    under the same condition as when the index is built. ANNS_TAP_FILTERED says
+ *    what the last search did. The change waits for the device.
  * Every kernel, schedule, chunk size and packing returns identical results.
  * Errors: INVALID_ARG. */
 enum { ANNS_OPT_KERNEL = 0, ANNS_OPT_SCHEDULE = 1, ANNS_OPT_QCHUNK = 2, ANNS_OPT_WAIT_CYCLES = 3,
-       ANNS_OPT_NIBBLE = 4 };
+       ANNS_OPT_NIBBLE = 4, ANNS_OPT_FILTER_BYTES = 5 };
 enum { ANNS_KERNEL_AUTO = 0, ANNS_KERNEL_BASIC = 1, ANNS_KERNEL_LIST_MAJOR = 2, ANNS_KERNEL_GROUPED = 3,
        ANNS_KERNEL_SPLIT = 4, ANNS_KERNEL_SPLIT_SCAN = 5, ANNS_KERNEL_FILTERED = 6 };
 enum { ANNS_SCHED_AUTO = 0, ANNS_SCHED_NATURAL = 1, ANNS_SCHED_LPT = 2 };

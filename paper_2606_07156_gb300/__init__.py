@@ -245,6 +245,11 @@ class Index:
         """Grouped search: pairs on <= 4-bit tables eight to a word (default on)."""
         abi.anns_set_option(self.handle, abi.OPT_NIBBLE, 1 if on else 0)
 
+    def set_filter_bytes(self, nbytes: int):
+        """Most workspace in bytes a filtered search may take (default 2**35); 0: never
+        filtered, and the decoded vectors are freed."""
+        abi.anns_set_option(self.handle, abi.OPT_FILTER_BYTES, int(nbytes))
+
     def set_schedule(self, which: str):
         """'auto', 'natural' or 'lpt' (longest query first) for the query-major kernel."""
         v = {"auto": abi.SCHED_AUTO, "natural": abi.SCHED_NATURAL, "lpt": abi.SCHED_LPT}[which]

@@ -22,7 +22,7 @@ PREC_FP32, PREC_BF16, PREC_FP8E4M3, PREC_FP16 = 0, 1, 2, 3
 TAP_PROBES, TAP_PROBE_D2, TAP_BITS, TAP_FEATURES = 0, 1, 2, 3
 TAP_COARSE_APPROX, TAP_COARSE_CANDIDATES = 4, 5
 TAP_LIST_SIZES, TAP_LIST_RADIUS, TAP_PACKED_IDS, TAP_STATUS, TAP_FILTERED = 10, 11, 12, 13, 14
-OPT_KERNEL, OPT_SCHEDULE, OPT_QCHUNK, OPT_WAIT_CYCLES, OPT_NIBBLE = 0, 1, 2, 3, 4
+OPT_KERNEL, OPT_SCHEDULE, OPT_QCHUNK, OPT_WAIT_CYCLES, OPT_NIBBLE, OPT_FILTER_BYTES = 0, 1, 2, 3, 4, 5
 KERNEL_AUTO, KERNEL_BASIC, KERNEL_LIST_MAJOR, KERNEL_GROUPED, KERNEL_SPLIT, KERNEL_SPLIT_SCAN, KERNEL_FILTERED = 0, 1, 2, 3, 4, 5, 6
 SCHED_AUTO, SCHED_NATURAL, SCHED_LPT = 0, 1, 2
 

@@ -503,23 +503,13 @@ static int reserve_filter(Index& ix, int64_t nq, int nprobe, int k, const anns_p
   return grow(&ix.ws_grp, &ix.ws_grp_cap, grouped_workspace_bytes(nq, k));
 }
 
-int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
-                   const int32_t* nprobe_per_q, Route& r) {
+static int reserve_route(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
+                         const int32_t* nprobe_per_q, const Route& r) {
   int rc = ensure_workspace(ix, nq, nprobe);
   if (rc) return rc;
-  if (r.filter && (rc = reserve_filter(ix, nq, nprobe, k, P))) {
-    if (rc != ANNS_ERR_OOM) return rc;
-    // No room for the filter's workspace, which is larger than the scan's:
-    // batches of this size scan from now on.
-    cudaGetLastError();
-    set_error("");
-    if (ix.ws_fl) cudaFree(ix.ws_fl);
-    ix.ws_fl = nullptr;
-    ix.ws_fl_cap = 0;
-    ix.fl_ws_limit = filter_workspace_bytes(ix, nq, nprobe, k) - 1;
-    r.filter = false;
-  }
-  if (!r.filter) {
+  if (r.filter) {
+    if ((rc = reserve_filter(ix, nq, nprobe, k, P))) return rc;
+  } else {
     if (ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR || r.grouped) {
       ListWork w{};
       const int64_t qchunk = ix.opt_kernel == ANNS_KERNEL_LIST_MAJOR ? nq : grouped_qchunk(ix, nq);
@@ -538,6 +528,21 @@ int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precisio
     if ((rc = grow(&ix.ws_tc, &ix.ws_tc_cap, coarse_tc_workspace_bytes(ix, nq)))) return rc;
   }
   return ANNS_OK;
+}
+
+int reserve_search(Index& ix, int64_t nq, int nprobe, int k, const anns_precision_policy& P,
+                   const int32_t* nprobe_per_q, Route& r) {
+  int rc = reserve_route(ix, nq, nprobe, k, P, nprobe_per_q, r);
+  if (rc != ANNS_ERR_OOM || (!r.filter && !ix.ws_fl)) return rc;
+  // No room for, or beside, the filter's workspace, which is larger than the
+  // scan's: it is given back and this call scans. The next one tries again.
+  cudaGetLastError();
+  set_error("");
+  if (ix.ws_fl) cudaFree(ix.ws_fl);
+  ix.ws_fl = nullptr;
+  ix.ws_fl_cap = 0;
+  r.filter = false;
+  return reserve_route(ix, nq, nprobe, k, P, nprobe_per_q, r);
 }
 
 int search_sequence(Index& ix, const float* Q, int64_t nq, int nprobe, const int32_t* nprobe_per_q, int k,
@@ -937,6 +942,22 @@ extern "C" int anns_set_option(anns_index* ix, int32_t option, int64_t value) {
       if (value != 0 && value != 1) return fail(ANNS_ERR_INVALID_ARG, "nibble option must be 0 or 1");
       ix->opt_nibble = (int)value;
       return ANNS_OK;
+    case ANNS_OPT_FILTER_BYTES: {
+      if (value < 0) return fail(ANNS_ERR_INVALID_ARG, "filter workspace must be >= 0");
+      DeviceGuard g(ix->device);
+      if (value == 0 && ix->fl_w) {  // the rows are given back once no search uses them
+        const cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return cuda_fail(e, "filter rows");
+        free_filter(*ix);
+      }
+      if (value < (int64_t)ix->ws_fl_cap && ix->ws_fl) {
+        cudaFree(ix->ws_fl);  // waits for the searches that use it
+        ix->ws_fl = nullptr;
+        ix->ws_fl_cap = 0;
+      }
+      ix->opt_filter_bytes = value;
+      return value > 0 && !ix->fl_w ? restore_filter(*ix) : ANNS_OK;
+    }
     default: return fail(ANNS_ERR_INVALID_ARG, "unknown option");
   }
 }

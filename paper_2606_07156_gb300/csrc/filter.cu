@@ -1647,6 +1647,14 @@ cudaError_t run_gemm(const Index& ix, const CUtensorMap& tmY, const CUtensorMap&
 
 }  // namespace
 
+struct FilterRows {
+  void* p[4] = {};
+  ~FilterRows() {
+    for (void* x : p)
+      if (x) cudaFree(x);
+  }
+};
+
 // The index's part of the filter: decoded FP16 rows and their scalars. Left
 // out (the search then scans) for values that are not finite, and where the
 // rows would take more than a quarter of the free device memory.
@@ -1689,15 +1697,19 @@ int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<
   cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemGetInfo");
   if (yb + (size_t)rows * 4 > free_b / 4) return ANNS_OK;
-  e = cudaMalloc(&ix.fl_y, yb);
-  if (e == cudaSuccess) e = cudaMalloc(&ix.fl_s, (size_t)rows * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&ix.fl_stat, (size_t)ix.nlist * sizeof(float4));
-  if (e == cudaSuccess) e = cudaMalloc(&ix.fl_ym, (size_t)ix.M * sizeof(float));
+  auto hold = std::make_shared<FilterRows>();
+  const size_t bytes[4] = {yb, (size_t)rows * sizeof(float), (size_t)ix.nlist * sizeof(float4), (size_t)ix.M * sizeof(float)};
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaMalloc(&hold->p[i], bytes[i]);
   if (e == cudaErrorMemoryAllocation) {  // no room: the index works without
     cudaGetLastError();
-    free_filter(ix);
     return ANNS_OK;
   }
+  if (e != cudaSuccess) return cuda_fail(e, "filter arrays");
+  ix.fl_hold = hold;
+  ix.fl_y = hold->p[0];
+  ix.fl_s = (float*)hold->p[1];
+  ix.fl_stat = hold->p[2];
+  ix.fl_ym = (float*)hold->p[3];
   if (e == cudaSuccess) e = cudaMemcpy(ix.fl_ym, ym.data(), ix.M * sizeof(float), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(mu.data(), ix.tc_mu, ix.dim * sizeof(float), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemset(ix.fl_stat, 0, (size_t)ix.nlist * sizeof(float4));
@@ -1721,12 +1733,18 @@ int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<
 }
 
 void free_filter(Index& ix) {
-  void* ptrs[] = {ix.fl_y, ix.fl_s, ix.fl_stat, ix.fl_ym};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
+  ix.fl_hold.reset();
   ix.fl_y = ix.fl_stat = nullptr;
   ix.fl_s = ix.fl_ym = nullptr;
   ix.fl_w = 0;
+}
+
+int restore_filter(Index& ix) {
+  std::vector<float> cent((size_t)ix.nlist * ix.dim), books((size_t)ix.M * kKsub * ix.dsub);
+  cudaError_t e = cudaMemcpy(cent.data(), ix.centroids, cent.size() * sizeof(float), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(books.data(), ix.codebooks, books.size() * sizeof(float), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "filter rows");
+  return prepare_filter(ix, cent, books);
 }
 
 bool filter_possible(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k) {
@@ -1737,7 +1755,7 @@ bool filter_possible(const Index& ix, const anns_precision_policy& P, int64_t nq
   if (pairs > INT32_MAX / 2 || nq * kTakeMax > INT32_MAX || max_slots(ix, pairs) > INT32_MAX ||
       max_items(ix, pairs, nq, tiles) > ((int64_t)1 << 26))
     return false;
-  return filter_workspace_bytes(ix, nq, nprobe, k) <= ix.fl_ws_limit;
+  return (int64_t)filter_workspace_bytes(ix, nq, nprobe, k) <= ix.opt_filter_bytes;
 }
 
 size_t filter_workspace_bytes(const Index& ix, int64_t nq, int nprobe, int k) {

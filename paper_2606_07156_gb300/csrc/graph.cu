@@ -80,6 +80,8 @@ extern "C" int anns_graph_capture(anns_index* ix, const float* Q, int64_t nq, in
   if (rc == ANNS_OK) {
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = cuda_fail(e, "search before capture");
+    // scanned, perhaps for want of memory: the captured search scans too
+    if (!gr->shadow.last_filtered) gr->shadow.opt_filter_bytes = 0;
   }
   if (rc == ANNS_OK) {
     e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);

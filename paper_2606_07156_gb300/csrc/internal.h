@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -65,7 +66,8 @@ struct Index {
   float* fl_ym = nullptr;
   int fl_w = 0;
   float fl_yscale = 1.f, fl_mu = 0.f;  // 1 / scale of the rows, |mu|
-  size_t fl_ws_limit = (size_t)32 << 30;  // workspace the filter may take (lowered where there was no room)
+  std::shared_ptr<void> fl_hold;       // owns those four; captured graphs keep them for their replays
+  int64_t opt_filter_bytes = (int64_t)32 << 30;  // ANNS_OPT_FILTER_BYTES: workspace the filter may take
   int64_t fl_tiles = 0;                // sum over the lists of their 256-vector tiles
   bool last_filtered = false;          // the last search went through the filter
   // host copies of the small per-list tables
@@ -287,6 +289,7 @@ cudaError_t launch_scan_pairs(const Index& ix, const float* Q, const float* qt, 
 // Tensor-core filter in front of the exact rules (filter.cu).
 int prepare_filter(Index& ix, const std::vector<float>& cent, const std::vector<float>& books);
 void free_filter(Index& ix);
+int restore_filter(Index& ix);  // prepare_filter from the index's own arrays
 // Whether the filter can serve the call.
 bool filter_possible(const Index& ix, const anns_precision_policy& P, int64_t nq, int nprobe, int k);
 // Whether the policy can choose tables of at most 4 bits for some pairs (the
