@@ -202,45 +202,47 @@ __global__ void __launch_bounds__(256) coarse_select_kernel(const float* __restr
 
 }  // namespace
 
-// A batch whose (query, list) pairs fill the GPU at most a few times over.
+// A batch whose (query, list) pairs fill the GPU at most a few times over. Its
+// two kernels have lines of their own. A thread per (query, list) reads its row by
+// itself, so from about 4e7 operands on the tiled kernel, whose rows are shared, is
+// faster (whole stage, D = 768: 8 queries x 4096 lists 45 us, tiled 90; 32 x 1024
+// 44 and 70; 64 x 1024 72 and 71; 64 x 4096 224 and 93).
 static bool small_batch(const Index& ix, int64_t nq) { return nq <= 64 && nq * ix.nlist <= (1 << 18); }
+static bool thread_rows(const Index& ix, int64_t nq) {
+  return small_batch(ix, nq) && ix.dim % 4 == 0 && ((uintptr_t)ix.centroids & 15u) == 0 &&
+         (double)nq * (double)ix.nlist * (double)ix.dim <= 4e7;
+}
+// A block per query selects in some 8 us however short the row; a warp in less on
+// short ones, in more the more probes it inserts (whole stage, D = 100, one query,
+// block / warp: 3 probes, 16 to 256 lists 16.3 to 17.3 / 7.8 to 9.0 us, 1024 lists
+// 17.2 / 11.5; 32 probes, 256 lists 17.6 / 12.3; 100 probes, 64 lists 17.6, by a
+// warp beside the tiled distances 22, 128 lists 17.8 and 58).
+static bool block_select(const Index& ix, int64_t nq, int nprobe) {
+  return small_batch(ix, nq) && ix.nlist > (nprobe <= 8 ? 1024 : nprobe <= 32 ? 256 : 32);
+}
 
 cudaError_t launch_coarse(const Index& ix, const float* Q, int64_t nq, int nprobe,
                           const int32_t* nprobe_per_q, float* d2, int32_t* probes,
                           float* probe_d2, cudaStream_t s, cudaEvent_t between) {
-  if (small_batch(ix, nq)) {
-    const bool v4 = ix.dim % 4 == 0 && ((uintptr_t)ix.centroids & 15u) == 0;
-    if (v4) {
-      coarse_d2_small_kernel<<<dim3((unsigned)((ix.nlist + 127) / 128), (unsigned)nq), 128, 0, s>>>(
-          Q, ix.centroids, ix.nlist, (int)ix.dim, d2);
-    } else {
-      coarse_d2_kernel<<<dim3((unsigned)((ix.nlist + kTL - 1) / kTL), (unsigned)((nq + kTQ - 1) / kTQ)), 256, 0, s>>>(
-          Q, ix.centroids, nq, ix.nlist, ix.dim, d2);
-    }
-    note_launch();
-    if (between) cudaEventRecord(between, s);
-    auto go = [&](auto kern) {
-      kern<<<(unsigned)nq, kSmallThreads, 0, s>>>(d2, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2);
-    };
-    switch ((nprobe + 31) / 32) {
-      case 1: go(coarse_select_small_kernel<1>); break;
-      case 2: go(coarse_select_small_kernel<2>); break;
-      case 3: go(coarse_select_small_kernel<3>); break;
-      default: go(coarse_select_small_kernel<4>); break;
-    }
-    note_launch();
-    return cudaGetLastError();
+  if (thread_rows(ix, nq)) {
+    coarse_d2_small_kernel<<<dim3((unsigned)((ix.nlist + 127) / 128), (unsigned)nq), 128, 0, s>>>(
+        Q, ix.centroids, ix.nlist, (int)ix.dim, d2);
+  } else {
+    dim3 g1((unsigned)((ix.nlist + kTL - 1) / kTL), (unsigned)std::min<int64_t>((nq + kTQ - 1) / kTQ, 65535));
+    coarse_d2_kernel<<<g1, 256, 0, s>>>(Q, ix.centroids, nq, ix.nlist, ix.dim, d2);
   }
-  dim3 g1((unsigned)((ix.nlist + kTL - 1) / kTL), (unsigned)std::min<int64_t>((nq + kTQ - 1) / kTQ, 65535));
-  coarse_d2_kernel<<<g1, 256, 0, s>>>(Q, ix.centroids, nq, ix.nlist, ix.dim, d2); note_launch();
+  note_launch();
   if (between) cudaEventRecord(between, s);
-  const unsigned g2 = (unsigned)((nq + 7) / 8);
-  const int R = (nprobe + 31) / 32;
-  switch (R) {
-    case 1: coarse_select_kernel<1><<<g2, 256, 0, s>>>(d2, nq, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2); break;
-    case 2: coarse_select_kernel<2><<<g2, 256, 0, s>>>(d2, nq, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2); break;
-    case 3: coarse_select_kernel<3><<<g2, 256, 0, s>>>(d2, nq, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2); break;
-    default: coarse_select_kernel<4><<<g2, 256, 0, s>>>(d2, nq, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2); break;
+  const bool by_block = block_select(ix, nq, nprobe);
+  auto select = [&](auto small, auto kern) {
+    if (by_block) small<<<(unsigned)nq, kSmallThreads, 0, s>>>(d2, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2);
+    else kern<<<(unsigned)((nq + 7) / 8), 256, 0, s>>>(d2, nq, ix.nlist, nprobe, nprobe_per_q, probes, probe_d2);
+  };
+  switch ((nprobe + 31) / 32) {
+    case 1: select(coarse_select_small_kernel<1>, coarse_select_kernel<1>); break;
+    case 2: select(coarse_select_small_kernel<2>, coarse_select_kernel<2>); break;
+    case 3: select(coarse_select_small_kernel<3>, coarse_select_kernel<3>); break;
+    default: select(coarse_select_small_kernel<4>, coarse_select_kernel<4>); break;
   }
   note_launch();
   return cudaGetLastError();

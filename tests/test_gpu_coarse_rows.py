@@ -46,3 +46,33 @@ def test_rows_around_the_radix_select(nlist, dim, cl):
         np.testing.assert_array_equal(d[keep], rd[keep])
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("nq,nlist,dim,nprobe", [(64, 33, 24, 8), (64, 33, 24, 9), (3, 256, 100, 8), (3, 257, 100, 8),
+                                                 (3, 32, 768, 32), (40, 1300, 768, 40), (41, 1300, 768, 40), (64, 4096, 100, 16),
+                                                 (65, 4096, 36, 16)])
+def test_few_queries_by_the_fp32_rule(nq, nlist, dim, nprobe):
+    """Both sides of the lines between the small kernels and the others: a thread or a tile for the
+    distances, a block or a warp for the selection, with tied distances and per-query nprobe."""
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2606_07156_gb300 as amp
+    r = np.random.Generator(np.random.PCG64(nq + nlist))
+    C = r.standard_normal((nlist, dim)).astype(np.float32)
+    C[5:9] = C[4]
+    Q = np.concatenate([C[3:6], r.standard_normal((nq, dim)).astype(np.float32)])[:nq]
+    npq = r.integers(0, nprobe + 1, nq).astype(np.int32)
+    g = amp.Index(C, r.standard_normal((2, 256, dim // 2)).astype(np.float32),
+                  r.integers(0, 256, (nlist, 2)).astype(np.uint8), np.arange(nlist, dtype=np.int32), device=0)
+    try:
+        D2 = ivfpq.coarse_d2_fp32(Q, C)
+        rp, rd = ivfpq.locate(D2, nprobe)
+        p, d = g.locate(torch.from_numpy(Q).to("cuda:0"), nprobe)
+        np.testing.assert_array_equal(p.cpu().numpy(), rp)
+        np.testing.assert_array_equal(d.cpu().numpy(), rd)
+        out = np.arange(nprobe)[None, :] >= npq[:, None]
+        p, d = g.locate(torch.from_numpy(Q).to("cuda:0"), nprobe, nprobe_per_q=torch.from_numpy(npq).to("cuda:0"))
+        np.testing.assert_array_equal(p.cpu().numpy(), np.where(out, -1, rp))
+        np.testing.assert_array_equal(d.cpu().numpy(), np.where(out, np.inf, rd))
+    finally:
+        g.close()
