@@ -1535,13 +1535,20 @@ struct FilterWork {
 };
 
 // Vectors of GEMM 1 per query: more of them lower T and with it the candidates
-// of GEMM 2. While the index's rows sit in L2 the second pass over them is cheap
-// (SIFT-shaped, 1024 -> 2048: GEMM 1 35 -> 56 us, GEMM 2 545 -> 454 us); rows
-// read from HBM make GEMM 1 cost as much as it saves (Deep-shaped, 1024 -> 2048:
-// 132 -> 253 us for 32 us less in GEMM 2).
+// of GEMM 2, at the cost of reading more rows twice. How much is saved depends on
+// the data, what it costs on how many of the rows stay in L2 between the groups
+// that share them. Whole plain search, k 10, 10000 queries, 32 probes, 1024 / 2048
+// vectors, by the bytes of the rows (L2: 129 MB):
+//   D 96, Deep-shaped:  24 MB 636 / 587 us, 96 MB 785 / 742, 192 MB 1102 / 1101,
+//                       384 MB 1154 / 885, 576 MB 882 / 941, 960 MB 934 / 1005,
+//                       1.9 GB 1162 / 1265
+//   D 128, SIFT-shaped: 32 MB 717 / 665, 128 MB 923 / 853, 260 MB 1339 / 947, 512 MB
+//                       1616 / 1139, 1 GB 1868 / 1290
+//   D 384, embeddings:  768 MB 1401 / 1307 (8 probes 864 / 891); D 768, 1.5 GB 1843 / 1869
+// so 2048 up to half a gigabyte, where it was never slower.
 int filter_take(const Index& ix, int k) {
-  const bool in_l2 = (double)ix.ntiles * kTileVecs * ix.fl_w * 2.0 <= 256e6;
-  return k <= 16 ? (in_l2 ? 2048 : 1024) : k <= 32 ? 2048 : kTakeMax;
+  const bool few_rows = (double)ix.ntiles * kTileVecs * ix.fl_w * 2.0 <= 537e6;
+  return k <= 16 ? (few_rows ? 2048 : 1024) : k <= 32 ? 2048 : kTakeMax;
 }
 int filter_fin(int k) { return k <= 32 ? 1024 : 2048; }
 int filter_cap(int k) { return k <= 32 ? 2048 : 4096; }
@@ -1587,13 +1594,17 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
   return w;
 }
 
-// Four pairs to a warp where a query has candidates in most of many probes (k
-// and nprobe large: embedding-shaped, 60 of 64 pairs, 8.4 -> 5.2 ms); else one,
-// which keeps more blocks resident (SIFT-shaped, about 10 pairs: 0.92 ms
-// against 1.74; uneven GIST-shaped 2.5 against 3.6).
+// Four pairs to a warp share the reading of a query's table rows, one pair to a
+// warp keeps twice the blocks resident. Four pay where a query has candidates in
+// most of many probes of wide tables, and cost a quarter on narrow ones (whole
+// search, fixed 8 bits, 2000 queries, 1M vectors, one / four pairs a warp):
+//   M 96, D 768 (embeddings): k 64, 16, 32, 64 probes 2816 / 2984, 3709 / 3527, 5450 /
+//     4229 us; k 100, 64 probes 6028 / 4578; k 40, 64 probes 4906 / 3917; k 10 2336 / 2916
+//   M 120, D 960 (GIST-shaped): 64 probes, k 64 11322 / 11711, k 100 14018 / 14406
+//   M 48, D 96: 64 probes, k 64 751 / 999, k 128 1216 / 1514; M 32, D 128: k 64 1162 / 1432
 template <int VPT>
 cudaError_t run_final_ds(const FinalArgs& a, cudaStream_t s) {
-  const int batch = a.k >= 64 && a.nprobe >= 48 && !a.npq && !a.quant_list ? kBatch : 1;
+  const int batch = a.Mp >= 96 && a.k >= 64 && a.nprobe >= 48 && !a.npq && !a.quant_list ? kBatch : 1;
   auto go = [&](auto kern) {
     const size_t sm = final_smem(a.dim, a.Mp, a.fin, batch);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
