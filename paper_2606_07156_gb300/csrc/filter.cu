@@ -379,7 +379,7 @@ struct GemmArgs {
   const FItem* items; const int* nitems;
   const float2* gk;
   const int2* gd; float* ub;                              // GEMM 1
-  const int* gp; const uint8_t* bits; int nprobe;         // GEMM 2
+  const int* gp; int nprobe;                              // GEMM 2
   int* qcnt; uint2* cand; int cap; uint8_t* alive;
   int* full;               // set once a query has more candidates than fit
   const float* sx;
@@ -1614,15 +1614,19 @@ cudaError_t run_final_ds(const FinalArgs& a, cudaStream_t s) {
     note_launch();
     return cudaGetLastError();
   };
+  auto pick = [&](auto ds) {
+    constexpr int DS = decltype(ds)::value;
+    if (a.quant_list) return go(final_kernel<VPT, DS, 1, true>);
+    if constexpr (VPT == 16) {  // k > 32
+      if (batch > 1) return go(final_kernel<VPT, DS, kBatch, false>);
+    }
+    return go(final_kernel<VPT, DS, 1, false>);
+  };
   switch (a.dsub) {
-    case 2: return a.quant_list ? go(final_kernel<VPT, 2, 1, true>)
-                   : batch == 1 ? go(final_kernel<VPT, 2, 1, false>) : go(final_kernel<VPT, 2, kBatch, false>);
-    case 4: return a.quant_list ? go(final_kernel<VPT, 4, 1, true>)
-                   : batch == 1 ? go(final_kernel<VPT, 4, 1, false>) : go(final_kernel<VPT, 4, kBatch, false>);
-    case 8: return a.quant_list ? go(final_kernel<VPT, 8, 1, true>)
-                   : batch == 1 ? go(final_kernel<VPT, 8, 1, false>) : go(final_kernel<VPT, 8, kBatch, false>);
-    default: return a.quant_list ? go(final_kernel<VPT, 0, 1, true>)
-                    : batch == 1 ? go(final_kernel<VPT, 0, 1, false>) : go(final_kernel<VPT, 0, kBatch, false>);
+    case 2: return pick(std::integral_constant<int, 2>{});
+    case 4: return pick(std::integral_constant<int, 4>{});
+    case 8: return pick(std::integral_constant<int, 8>{});
+    default: return pick(std::integral_constant<int, 0>{});
   }
 }
 
@@ -1803,7 +1807,7 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   GemmArgs g{};
   g.sx = ix.fl_s; g.nK = Dp / kKE; g.ksteps = (int)((ix.dim + 15) / 16); g.status = ix.dev_status;
   g.wait_limit = ix.opt_wait_cycles > 0 ? ix.opt_wait_cycles : kWaitCycles;
-  g.nprobe = nprobe; g.bits = bits; g.ub = w.ub; g.qcnt = w.qcnt; g.cand = w.cand; g.cap = filter_cap(k);
+  g.nprobe = nprobe; g.ub = w.ub; g.qcnt = w.qcnt; g.cand = w.cand; g.cap = filter_cap(k);
   g.alive = w.alive; g.full = w.nover + 2;
   auto pass = [&](auto mode, const PassArgs& w1) {
     constexpr int MODE = decltype(mode)::value;
@@ -1842,7 +1846,7 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   } else {
     const unsigned tb = (unsigned)((nq + 3) / 4);
     switch (p.take / 32) {
-    case 32: threshold_kernel<32><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
+      case 32: threshold_kernel<32><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
       case 64: threshold_kernel<64><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
       default: threshold_kernel<128><<<tb, 128, 0, s>>>(p, w.p2, w.ub); break;
     }

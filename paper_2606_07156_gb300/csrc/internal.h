@@ -180,7 +180,7 @@ enum { QM_TABLES_ALL = 0, QM_TABLES_FP32 = 1, QM_TABLES_NARROW = 2 };
 // the order in which blocks take the queries; split > 1: that many blocks a
 // query, row q * split + i of the results for its part i; with `count` (device) only its
 // first *count entries run. skip_narrow 1 leaves out the 1..8-bit pairs of
-// probe rank >= 1, 2 those of every rank, 3 the 1..4-bit pairs of every rank. With
+// probe rank >= 1, 2 those of every rank. With
 // QM_TABLES_NARROW only the 1..8-bit pairs are scanned, and part_d / part_i
 // (or NULL), the query's top-k over its other pairs ([nq * k]), bound the
 // scan and join the final merge.

@@ -426,8 +426,7 @@ struct SearchArgs {
   const int32_t* probes; const float* probe_d2; const uint8_t* bits;
   const int32_t* order; const int* count;  // count: only the first *count entries of `order`
   // 1: leave out the pairs on 1..8-bit tables of rank >= 1 (the grouped
-  // kernels take them); 2: of every rank (the narrow pass takes them); 3: the
-  // pairs on 1..4-bit tables (the grouped kernels take the ones worth a scan)
+  // kernels take them); 2: of every rank (the narrow pass takes them)
   int skip_narrow;
   int split;  // blocks per query: block i of a query takes every split-th of its pairs, result row q * split + i
   int ids32;  // every id fits in int32 (the 128-entry lists then hold 32-bit ids)
@@ -539,8 +538,7 @@ __global__ void __launch_bounds__(kThreads, qm_blocks<MODE, NCHUNK, R>()) search
         const bool narrow = b >= 1 && b <= 8;
         const bool use = l >= 0 && n_l > 0 &&
                          (MODE == kModeNarrow ? narrow
-                                              : !(narrow && (a.skip_narrow == 2 || (a.skip_narrow == 1 && j >= 1) ||
-                                                             (a.skip_narrow == 3 && b <= 4))));
+                                              : !(narrow && (a.skip_narrow == 2 || (a.skip_narrow == 1 && j >= 1))));
         const unsigned m = __ballot_sync(kFull, use);
         const int at = base + __popc(m & ((1u << lane) - 1u));
         if (use && (a.split == 1 || at % a.split == part))
