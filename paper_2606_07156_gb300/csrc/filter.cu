@@ -619,9 +619,10 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
         // A query with more candidates than fit is scanned whatever else is found
         // for it: its pairs take no more of them, only the mark that has them
         // scanned. (174 queries, 37 lists of 1186, D 384, M 96, 6 bits, bounds too
-        // wide to drop anything: 7.6 million pushes took 8.2 ms.) Looked up only
-        // after an item with many candidates: two dependent reads of L2 an item
-        // cost a batch with few of them 4 %.
+        // wide to drop anything: this pass 8.2 ms, 6.0 so, most of it still in the
+        // additions to the counts; such widths are not filtered by the automatic
+        // choice.) Looked up only after an item with many candidates: two dependent
+        // reads of L2 an item cost a batch with few of them 4 %.
         if (nfull && found > 64) {
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
