@@ -381,7 +381,6 @@ struct GemmArgs {
   const int2* gd; float* ub;                              // GEMM 1
   const int* gp; int nprobe;                              // GEMM 2
   int* qcnt; uint2* cand; int cap; uint8_t* alive;
-  int* full;               // set once a query has more candidates than fit
   const float* sx;
   int nK, ksteps;
   int* status; long long wait_limit;
@@ -544,13 +543,12 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     int* sp = (int*)(mine + 64 * 16);                 // staged candidates: pair, position, D~ - D2
     int* spos = sp + kPush;
     float* sv = (float*)(spos + kPush);
-    int staged = 0, found = 0;                        // found: candidates of the item
+    int staged = 0;
     auto flush = [&]() {
       __syncwarp();
       for (int e = lane; e < staged; e += 32) {
         const int p = sp[e], q = p / a.nprobe;
         const int at = atomicAdd(a.qcnt + q, 1);
-        if (at == a.cap) *a.full = 1;
         if (at < a.cap)
           a.cand[(int64_t)q * a.cap + at] = make_uint2((uint32_t)(p - q * a.nprobe) << kPosBits | (uint32_t)spos[e],
                                                        __float_as_uint(sv[e]));
@@ -580,7 +578,6 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
           sv[e] = t;
         }
         staged += __popc(who);
-        found += __popc(who);
       }
     };
     // the next item's columns are requested while this one is drained, its item
@@ -589,12 +586,10 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
     float2 nk[2] = {};
     int2 nd[2] = {};
     float ns = 0.f;
-    int nfull = 0;
     auto load_cols = [&](const FItem& f) {  // and the thread's row scalar
       const int nv = f.nv_cnt & 0xFFFF;
       // rows past the list's end hold the next list's vectors: never candidates
       ns = r0 + lane < nv ? __ldg(a.sx + f.row0 + r0 + lane) : INFINITY;
-      if constexpr (MODE == 2) nfull = *(volatile const int*)a.full;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const int col = lane + 32 * par + 64 * c, s = f.slot0 + col;
@@ -615,26 +610,6 @@ __global__ void __launch_bounds__(kFThreads, 1) filter_gemm_kernel(const __grid_
       const FItem it = nx;
       const int nv = it.nv_cnt & 0xFFFF, cnt = it.nv_cnt >> 16, b = n & 1, r = r0 + lane;
       const float s = ns;
-      if constexpr (MODE == 2) {
-        // A query with more candidates than fit is scanned whatever else is found
-        // for it: its pairs take no more of them, only the mark that has them
-        // scanned. (174 queries, 37 lists of 1186, D 384, M 96, 6 bits, bounds too
-        // wide to drop anything: this pass 8.2 ms, 6.0 so, most of it still in the
-        // additions to the counts; such widths are not filtered by the automatic
-        // choice.) Looked up only after an item with many candidates: two dependent
-        // reads of L2 an item cost a batch with few of them 4 %.
-        if (nfull && found > 64) {
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int p = nd[c].x;
-            if (lane + 32 * par + 64 * c < cnt && p >= 0 && *(volatile const int*)(a.qcnt + p / a.nprobe) > a.cap) {
-              a.alive[p] = 1;
-              nk[c].x = -INFINITY;
-            }
-          }
-        }
-        found = 0;
-      }
       __syncwarp();
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -1571,7 +1546,7 @@ FilterWork filter_work(const Index& ix, int64_t nq, int nprobe, int k, char* bas
     p->cnt = w.take<int>(L);
     p->fill = w.take<int>(L);
   }
-  w.qcnt = w.take<int>(nq); w.nover = w.take<int>(3);  // the count of `quant`, whether any query overflowed
+  w.qcnt = w.take<int>(nq); w.nover = w.take<int>(2);  // and the count of `quant`
   w.alive = w.take<uint8_t>(P);
   w.overflag = w.take<uint8_t>(nq);
   w.zero_bytes = w.bytes;
@@ -1809,7 +1784,7 @@ cudaError_t launch_search_filter(const Index& ix, const float* Q, const float* q
   g.sx = ix.fl_s; g.nK = Dp / kKE; g.ksteps = (int)((ix.dim + 15) / 16); g.status = ix.dev_status;
   g.wait_limit = ix.opt_wait_cycles > 0 ? ix.opt_wait_cycles : kWaitCycles;
   g.nprobe = nprobe; g.ub = w.ub; g.qcnt = w.qcnt; g.cand = w.cand; g.cap = filter_cap(k);
-  g.alive = w.alive; g.full = w.nover + 2;
+  g.alive = w.alive;
   auto pass = [&](auto mode, const PassArgs& w1) {
     constexpr int MODE = decltype(mode)::value;
     plan_scan_kernel<<<1, 1024, 0, s>>>(ix.list_len, (int)ix.nlist, w1); note_launch();
